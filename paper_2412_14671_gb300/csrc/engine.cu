@@ -585,14 +585,14 @@ int forward_adjoint(muster_ctx* ctx, int l, const float4* th) {
       {
         // W and the NC coefficient volumes per pair; F, mu_F and S_FF once per fixed session
         Scope s(ctx, KK_SIM_FWD, (double)nb * Vi * (4.0 + 4.0 * NC) + (double)n_fixed * Vi * 12.0);
-        launch_sim_fwd(pd, nb, ctx->Bc, ctx->Wbuf, Vi, ctx->coef, Vi, ctx->sim_part + (size_t)b0 * g.ctas, ni,
+        launch_sim_fwd(pd, nb, ctx->Bc, ctx->N - 1, ctx->Wbuf, Vi, ctx->coef, Vi, ctx->sim_part + (size_t)b0 * g.ctas, ni,
                        ctx->p.window, ctx->p.similarity, ctx->p.sim_eps, &ctx->maps[l], ctx->flag_dev + 1,
                        ctx->stream);
       }
       {
         // coefficients, W and dL/dW per pair; F once per fixed session
         Scope s(ctx, KK_SIM_BWD, (double)nb * Vi * (8.0 + 4.0 * NC) + (double)n_fixed * Vi * 4.0);
-        launch_sim_bwd(pd, nb, ctx->Bc, ctx->Wbuf, Vi, ctx->coef, Vi, ctx->dLdW, ni, ctx->p.window, ctx->p.similarity,
+        launch_sim_bwd(pd, nb, ctx->Bc, ctx->N - 1, ctx->Wbuf, Vi, ctx->coef, Vi, ctx->dLdW, ni, ctx->p.window, ctx->p.similarity,
                        scale, &ctx->maps[l], ctx->flag_dev + 1, ctx->stream);
       }
       {

@@ -159,11 +159,12 @@ void make_sim_maps(SimMaps* m, const float* W, int n_pairs, const float* imgs, i
                    Dims ni, int window, int kind);
 // maps (nullable): TMA staging of the inputs when maps->fwd_ok / bwd_ok; err (nullable) is
 // set to 1 if a bounded wait for a copy ran out (the results are then not valid)
-void launch_sim_fwd(const PairDesc* pd, int n_pairs, int batch, const float* W, size_t Wstride, float* coef,
+// group: neighbouring pairs that share a fixed image (they run beside each other on a tile)
+void launch_sim_fwd(const PairDesc* pd, int n_pairs, int batch, int group, const float* W, size_t Wstride, float* coef,
                     size_t coef_stride, double* partials, Dims ni, int window, int kind, float eps,
                     const SimMaps* maps, int* err, cudaStream_t s);
-void launch_sim_bwd(const PairDesc* pd, int n_pairs, int batch, const float* W, size_t Wstride, const float* coef,
-                    size_t coef_stride, float* dLdW, Dims ni, int window, int kind, float scale,
+void launch_sim_bwd(const PairDesc* pd, int n_pairs, int batch, int group, const float* W, size_t Wstride,
+                    const float* coef, size_t coef_stride, float* dLdW, Dims ni, int window, int kind, float scale,
                     const SimMaps* maps, int* err, cudaStream_t s);
 // batch: the most pairs one launch of this context takes (n_pairs <= batch); it sets the
 // D chunking, so every launch of a context splits a pair the same way.

@@ -2,19 +2,39 @@
 // averaged over the valid windows (Eq. sum_lncc, Eq. sim_loss), and its adjoint.
 //
 // Window R has lower corner c (centre c + R); the valid corners are
-// 0 <= c_a <= n_a - w. Both kernels stream along D: a CTA of 256 threads owns a
-// 32 (W) x 16 (H) tile of windows (forward) or voxels (adjoint) and a chunk of D.
-// Per plane the (32 + 2R) x (16 + 2R) halo region of the inputs is staged in
-// shared memory, summed along W by running sums over float4 runs, along H by
-// running sums (two rows per thread), and along D through a shared-memory ring of
-// the last 2R+1 plane sums with a running total that is re-summed exactly every
-// 2R+1 planes. When the width is a multiple of 4 the halo planes are copied by
-// the tensor memory accelerator (two stages, mbarrier completion, zero fill
-// outside the volume); otherwise each thread loads its share of the plane.
+// 0 <= c_a <= n_a - w. Forward and adjoint are streamed separable box sums: a CTA owns a
+// 32 (W) x 16 (H) tile of windows (forward) or voxels (adjoint) and a chunk of D, and walks D
+// plane by plane, in two roles that run beside each other:
+//  - W warps, a thread per 8 neighbouring sums of one halo row: box sums along W from 16-byte
+//    loads of the staged plane into one of two buffers of W sums;
+//  - H/D warps, a thread per column and 4 rows: box sums along H, then along D through a
+//    shared-memory ring of the last 2R+1 plane sums with a running total that is re-summed
+//    exactly every 2R+1 planes (bounded FP32 drift), and the outputs of the plane.
+// The roles hand the buffers over by named barriers (full / empty), so the W pass of one plane
+// overlaps the H and D passes of the one before, and no barrier holds all warps of the CTA.
+//
+// What bounds them: the shared-memory pipe (bytes moved through L1 per output), then instruction
+// issue. The layout is chosen for both: 8 sums per W task read 14 inputs (w = 7) instead of 10 for
+// every 4, four rows per H/D thread read 10 W sums instead of 16, the ring moves 16 bytes per
+// access, and the row pitches (4 modulo 8 floats) keep the W task's accesses free of bank conflicts.
+// Measured on 90 pairs of 160 x 192 x 160, w = 7, SiLNCC: forward 1678 us, adjoint 1451 us (L1 data
+// pipe 76 and 81 % busy, DRAM 39 and 57 %); one role per thread with a barrier per plane, W sums in
+// runs of 4 and two rows per thread took 2605 and 1802 us. 4 CTAs of 7 warps run on an SM; cut for
+// 3, the forward takes 1895 us.
+//
+// The order of the additions is part of the results, and the layout keeps it: along W runs of 4
+// sums (a pairwise tree, then a running sum), along H runs of 2, along D the ring. An optimiser
+// amplifies the last bits of the gradient (the 20-step registration of three 48^3 volumes moves
+// its velocities by 6e-5 when they change), and LNCC, which divides by sqrt(S_FF S_WW), has
+// gradients that follow the rounding of the sums in flat regions.
+//
+// Inputs are staged two planes ahead, by the tensor memory accelerator (mbarrier completion, zero
+// fill outside the volume) when the width is a multiple of 4 and the bases are 16-byte aligned,
+// otherwise by 4-byte asynchronous copies.
 //
 // The fixed image's window statistics (mu_F, S_FF) depend on the session only and
 // are computed once per level (k_fixed_stats); the forward per pair then needs
-// the box sums of W', W'^2 and F'W' only.
+// the box sums of W' and F'W' (and of W'^2 for LNCC) only.
 // Forward: for every corner of the image grid it writes the coefficients of
 //   dSim_R/dW(p) = A_R W(p) - B_R F(p) - C_R   (zero for invalid corners)
 //   SiLNCC: A = 1 (implicit; 2/|R| is applied by the adjoint), B = beta = S_FW/(S_FF+eps),
@@ -22,11 +42,15 @@
 //   LNCC:   A = S_FW S_FF / Q^{3/2}, B = 1/sqrt(Q), C = A mu_W - B mu_F, Q = S_FF S_WW + eps,
 // and adds Sim_R to a per-CTA partial sum. Sums are taken on values shifted by
 // one voxel of the tile (variance is shift invariant) to limit cancellation.
+// SiLNCC needs S_WW only in the loss, where sum_R S_WW = sum_p cnt(p) W'(p)^2 - sum_R (sum W')^2/|R|
+// with cnt(p) the number of the CTA's windows that hold voxel p: the W pass adds the first term
+// once per voxel, which spares a third box sum (a third of the ring and of the arithmetic).
 // Adjoint: dL/dW(p) = scale * (W(p) sum A - F(p) sum B - sum C) over the
 // windows containing p (corners p - 2R .. p).
 #include <cudaTypedefs.h>
 #include <string.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "kernels.h"
@@ -35,24 +59,7 @@
 namespace muster {
 
 namespace {
-constexpr int kThreads = 256, TX = 32;
-
-// The CTA's sum of the per-thread compensated sums (hi + lo), valid in thread 0: float-float
-// sums within each warp, then the warp sums in double.
-__device__ __forceinline__ double block_sum(FF x, float* sh) {
-  x = warp_sum_ff(x);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) {
-    sh[2 * w] = x.hi;
-    sh[2 * w + 1] = x.lo;
-  }
-  __syncthreads();
-  double r = 0.0;
-  if (threadIdx.x == 0)
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) r += (double)sh[2 * i] + (double)sh[2 * i + 1];
-  return r;
-}
+constexpr int kThreads = 256, TX = 32;  // k_fixed_stats
 
 // Statistics of the fixed image of every window, once per session and level:
 // out[0][c] = mu_F and out[1][c] = S_FF (centred sum of squares) at corner c, or for SiLNCC
@@ -138,30 +145,96 @@ __global__ void __launch_bounds__(kThreads) k_fixed_stats(const float* __restric
 }
 
 // ---------------------------------------------------------------------------
-// Streaming box sums, version with running sums in all three directions.
-// CTA tile: 32 (W) x 16 (H) windows (forward) or voxels (adjoint), 256 threads
-// (16 output rows against 2R halo rows keep the W pass's share of halo work small).
-//  - W pass: 8 tasks per halo row, each 4 consecutive outputs from one float4
-//    run of 4 + 2R inputs (running sum along W);
-//  - H pass: one thread per column and pair of rows (running sum);
-//  - D pass: a ring of the last 2R+1 plane sums in shared memory, one owner
-//    thread per output, running sum re-summed exactly every 2R+1 planes.
-constexpr int T3X = 32, T3Y = 16, YO = 2, NT3 = T3X * T3Y / YO;  // 256 threads
-static_assert(YO == 2, "the D ring of the TMA-staged kernels keeps a thread's two rows as a float2");
-// a tensor copy must start on a 16-byte boundary: the forward's box starts at x0 = 32 * blockIdx.x
-static_assert(T3X % 4 == 0, "the staged forward box must start at a multiple of 4 floats");
+constexpr int kTX = 32, kTY = 16;   // outputs of a CTA's tile along W and H
+constexpr int kXO = 8;              // sums of one W task
+constexpr int kYO = 4;              // rows of one H/D thread
+constexpr int kHD = kTX * kTY / kYO;  // H/D threads
+// a tensor copy must start on a 16-byte boundary: the forward's box starts at x0 = 32 * tile
+static_assert(kTX % 4 == 0, "the staged forward box must start at a multiple of 4 floats");
 
-template <int R, int NM>
-struct Geo3 {
+// tile shapes for window radius R
+template <int R>
+struct Box {
   static constexpr int WW = 2 * R + 1;
-  static constexpr int RX = T3X + 2 * R, RY = T3Y + 2 * R;
-  static constexpr int NV = (4 + 2 * R + 3) / 4;  // float4 per W-pass run
-  static constexpr int RXS = ((RX + 3) / 4) * 4 > 28 + 4 * NV ? ((RX + 3) / 4) * 4 : 28 + 4 * NV;
-  static constexpr int NE = RY * RX, NSLOT = (NE + NT3 - 1) / NT3;
-  // shared memory (floats): inputs [NIN][RY][RXS], W sums [NM][RY][T3X], ring [WW][NM][T3Y][T3X]
-  __host__ __device__ static constexpr size_t in_floats(int nin) { return (size_t)nin * RY * RXS; }
-  __host__ __device__ static constexpr size_t sx_floats() { return (size_t)NM * RY * T3X; }
-  __host__ __device__ static constexpr size_t ring_floats() { return (size_t)WW * NM * T3Y * T3X; }
+  static constexpr int RX = kTX + 2 * R, RY = kTY + 2 * R;  // halo columns and rows of a plane
+  static constexpr int NI = kXO + 2 * R;                    // inputs of a W task
+  static constexpr int NV = (NI + (2 * R & 3) + 3) / 4;     // its float4 loads at most (bwd_xoff columns early)
+  static constexpr int NTASK = RY * (kTX / kXO);            // W tasks of a plane
+  static constexpr int WT = (NTASK + 31) / 32 * 32;         // W threads
+  static constexpr int NT = kHD + WT;
+  static constexpr int PX = R <= 2 ? 36 : 44;               // row pitch of a staged plane
+  static constexpr int PS = 36;                             // row pitch of the W sums
+  static constexpr int TS = (RY * PX + 31) & ~31;           // floats of one staged plane (128-byte multiple)
+  static_assert(PX >= kTX - kXO + 4 * NV && PX % 8 == 4 && PS % 8 == 4, "pitches");
+  __host__ __device__ static constexpr int sx_floats(int nm) { return nm * RY * PS; }
+  __host__ __device__ static constexpr int ring_floats(int nm) { return WW * nm * kTX * kTY; }
+  // dynamic shared memory: [2 stages][nin][TS], [2 planes][nm] W sums, D ring
+  __host__ __device__ static constexpr size_t bytes(int nin, int nm) {
+    return sizeof(float) * (size_t)(2 * nin * TS + 2 * sx_floats(nm) + ring_floats(nm));
+  }
+};
+
+// x offset of the adjoint's staged box: its first column x0 - 2R is rounded down to a
+// multiple of 4 (16-byte aligned tile coordinate), so the box starts XOFF columns early
+template <int R>
+__host__ __device__ constexpr int bwd_xoff() {
+  return (2 * R) & 3;
+}
+
+// the launch's tiles: a one-dimensional grid over groups of `grp` pairs, then D chunks, tiles
+// and, fastest, the pairs of the group
+struct Tiles {
+  int np, grp, gx, gy, nzc, tz;
+};
+struct Tile {
+  int pair, x0, y0, z0, part;  // part: index of the CTA's partial sum
+};
+// Pairs that share a fixed image (the engine orders them by fixed image) run beside each other
+// on the same tile, so that its F, mu_F and S_FF planes are read from L2 by all but the first
+// (10 sessions of 160 x 192 x 160: forward 1678 us, in pair order 1763 us).
+__device__ __forceinline__ Tile tile_of(const Tiles& g) {
+  const unsigned per = (unsigned)g.gx * g.gy * g.nzc;
+  unsigned id = blockIdx.x;
+  const unsigned span = g.grp * per, first = id / span * g.grp;
+  id -= id / span * span;
+  const unsigned in = min((unsigned)g.grp, (unsigned)g.np - first);
+  Tile t;
+  t.pair = (int)(first + id % in);
+  id /= in;
+  t.part = (int)(t.pair * per + id);
+  t.x0 = (int)(id % g.gx) * kTX;
+  id /= g.gx;
+  t.y0 = (int)(id % g.gy) * kTY;
+  t.z0 = (int)(id / g.gy) * g.tz;
+  return t;
+}
+
+// The CTA's sum of the per-thread float-float sums, valid in thread 0: float-float
+// sums within each warp, then the warp sums in double.
+template <int NT>
+__device__ __forceinline__ double block_sum(FF x, float* sh) {
+  x = warp_sum_ff(x);
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  __syncthreads();
+  if (l == 0) {
+    sh[2 * w] = x.hi;
+    sh[2 * w + 1] = x.lo;
+  }
+  __syncthreads();
+  double r = 0.0;
+  if (threadIdx.x == 0)
+    for (int i = 0; i < NT / 32; ++i) r += (double)sh[2 * i] + (double)sh[2 * i + 1];
+  return r;
+}
+
+// compensated (Kahan) running sum
+struct KSum {
+  float s = 0.f, c = 0.f;
+  __device__ __forceinline__ void add(float x) {
+    const float y = x - c, t = s + y;
+    c = (t - s) - y;
+    s = t;
+  }
 };
 
 // pairwise sum of v[0..N-1]: a dependency chain of depth log2(N) instead of N - 1
@@ -188,765 +261,503 @@ __device__ __forceinline__ void runsum(const float* v, float* out) {
   }
 }
 
-template <int R, int KIND>
-__global__ void __launch_bounds__(NT3) k_sim_fwd3(const PairDesc* __restrict__ pd, const float* __restrict__ Wb,
-                                                       size_t Wstride, float* __restrict__ coef, size_t cstride,
-                                                       double* __restrict__ part, Dims n, float eps, int tz, int nzc) {
-  using G = Geo3<R, 3>;
-  constexpr int WW = G::WW, RX = G::RX, RY = G::RY, RXS = G::RXS, NV = G::NV, NE = G::NE, NSLOT = G::NSLOT;
-  constexpr int NC = KIND == 0 ? 2 : 3;
-  extern __shared__ __align__(16) float smem[];
-  float* sF = smem;
-  float* sW = sF + RY * RXS;
-  float* sx = sW + RY * RXS;                 // [3][RY][T3X]
-  float* ring = sx + G::sx_floats();         // [WW][3][T3Y][T3X]
-  __shared__ float sh[2 * (NT3 / 32)];
-  const int pair = blockIdx.z / nzc, zc = blockIdx.z - pair * nzc;
-  const int x0 = blockIdx.x * T3X, y0 = blockIdx.y * T3Y, z0 = zc * tz;
-  const int tid = threadIdx.x;
-  const PairDesc d = pd[pair];
-  const float* __restrict__ F = d.Ii;
-  const float* __restrict__ Fs = d.Fs;
-  const float* __restrict__ W = Wb + (size_t)pair * Wstride;
-  float* __restrict__ C = coef + (size_t)pair * NC * cstride;
-  const int plane = n.n1 * n.n2;
-  int soff[NSLOT], sidx[NSLOT];
-  bool sok[NSLOT];
-#pragma unroll
-  for (int k = 0; k < NSLOT; ++k) {
-    const int e = tid + NT3 * k;
-    const int ry = e / RX, rx = e - ry * RX;
-    const int gy = y0 + ry, gx = x0 + rx;
-    sok[k] = e < NE && gy < n.n1 && gx < n.n2;
-    soff[k] = gy * n.n2 + gx;
-    sidx[k] = e < NE ? ry * RXS + rx : -1;
+// The same for products v[k] = a[k] b[k]: a product that enters one addition only is fused into
+// it, the others are rounded first (p). In a run of 4 those are the products past the first sum's
+// window and, within it, all but the first three, which leave the running sum again.
+template <int N>
+struct ProdTree {
+  template <int K>  // sum of the products K .. K + N - 1
+  __device__ __forceinline__ static float of(const float* a, const float* b, const float* p) {
+    if constexpr (N == 1) {
+      return p[K];
+    } else {
+      constexpr int NL = N / 2;
+      if constexpr (NL == 1 && K >= 3)
+        return __fmaf_rn(a[K], b[K], ProdTree<N - NL>::template of<K + NL>(a, b, p));
+      else if constexpr (N - NL == 1 && K + NL >= 3)
+        return __fmaf_rn(a[K + NL], b[K + NL], ProdTree<NL>::template of<K>(a, b, p));
+      else
+        return __fadd_rn(ProdTree<NL>::template of<K>(a, b, p), ProdTree<N - NL>::template of<K + NL>(a, b, p));
+    }
   }
-  const int so = min(z0 + R, n.n0 - 1) * plane + min(y0 + R, n.n1 - 1) * n.n2 + min(x0 + R, n.n2 - 1);
-  const float shF = F[so], shW = W[so];
-  const float inv_nw = 1.f / (float)(WW * WW * WW);
-  const int mx = n.n2 - WW, my = n.n1 - WW, mz = n.n0 - WW;
-  // roles: W pass (8 tasks per halo row), H/D pass and outputs (thread = column, YO rows)
-  const int col = tid & 31, yseg = tid >> 5;
-  float S[YO][3];
+};
+template <int WW>
+__device__ __forceinline__ void runsum4(const float* a, const float* b, float* out) {
+  float p[WW];
 #pragma unroll
-  for (int i = 0; i < YO; ++i)
+  for (int k = 0; k < WW; ++k) p[k] = __fmul_rn(a[k], b[k]);
+  out[0] = ProdTree<WW>::template of<0>(a, b, p);
 #pragma unroll
-    for (int m = 0; m < 3; ++m) S[i][m] = 0.f;
-  for (int j = 0; j < WW; ++j)
-#pragma unroll
-    for (int m = 0; m < 3; ++m)
-#pragma unroll
-      for (int i = 0; i < YO; ++i) ring[((j * 3 + m) * T3Y + YO * yseg + i) * T3X + col] = 0.f;
-  float lsum = 0.f, lcomp = 0.f;
-  const int zend = min(z0 + tz, n.n0);
-  const int niter = (zend - z0) + 2 * R;
-  float pf[NSLOT], pw[NSLOT];
-  auto fetch = [&](int zin) {
-    const bool zok = zin < n.n0;
-    const int zo = zin * plane;
-#pragma unroll
-    for (int k = 0; k < NSLOT; ++k) {
-      pf[k] = 0.f;
-      pw[k] = 0.f;
-      if (zok && sok[k]) {
-        pf[k] = F[zo + soff[k]] - shF;
-        pw[k] = W[zo + soff[k]] - shW;
-      }
-    }
-  };
-  // mu_F and S_FF of this thread's windows in the next output plane (loaded one plane ahead)
-  float pmu[YO], psf[YO];
-  const bool xin = x0 + col <= mx;
-  auto fetch_stats = [&](int cz) {
-#pragma unroll
-    for (int i = 0; i < YO; ++i) {
-      const int cy = y0 + YO * yseg + i;
-      pmu[i] = 0.f;
-      psf[i] = 0.f;
-      if (xin && cy <= my && cz <= mz) {
-        const int o = cz * plane + cy * n.n2 + x0 + col;
-        pmu[i] = Fs[o];
-        psf[i] = Fs[(size_t)plane * n.n0 + o];
-      }
-    }
-  };
-  fetch(z0);
-  int j = 0;  // ring slot of this plane
-  for (int it = 0; it < niter; ++it) {
-    const int zin = z0 + it;
-#pragma unroll
-    for (int k = 0; k < NSLOT; ++k)
-      if (sidx[k] >= 0) {
-        sF[sidx[k]] = pf[k];
-        sW[sidx[k]] = pw[k];
-      }
-    float muF_c[YO], Sff_c[YO];
-#pragma unroll
-    for (int i = 0; i < YO; ++i) muF_c[i] = pmu[i], Sff_c[i] = psf[i];
-    __syncthreads();
-    if (it + 1 < niter) {
-      fetch(zin + 1);
-      if (it + 1 >= 2 * R) fetch_stats(zin + 1 - 2 * R);
-    }
-    for (int task = tid; task < 8 * RY; task += NT3) {
-      const int xrow = task >> 3, xseg = task & 7;
-      float f[4 * NV], w[4 * NV];
-      const float4* pF = reinterpret_cast<const float4*>(sF + xrow * RXS + 4 * xseg);
-      const float4* pW = reinterpret_cast<const float4*>(sW + xrow * RXS + 4 * xseg);
-#pragma unroll
-      for (int q = 0; q < NV; ++q) {
-        const float4 a = pF[q], b = pW[q];
-        f[4 * q] = a.x, f[4 * q + 1] = a.y, f[4 * q + 2] = a.z, f[4 * q + 3] = a.w;
-        w[4 * q] = b.x, w[4 * q + 1] = b.y, w[4 * q + 2] = b.z, w[4 * q + 3] = b.w;
-      }
-      float ww[4 + 2 * R], fw[4 + 2 * R];
-#pragma unroll
-      for (int k = 0; k < 4 + 2 * R; ++k) {
-        ww[k] = w[k] * w[k];
-        fw[k] = f[k] * w[k];
-      }
-      float o0[4], o1[4], o2[4];
-      runsum<WW, 4>(w, o0);
-      runsum<WW, 4>(ww, o1);
-      runsum<WW, 4>(fw, o2);
-      float4* dst = reinterpret_cast<float4*>(sx + xrow * T3X + 4 * xseg);
-      dst[0] = make_float4(o0[0], o0[1], o0[2], o0[3]);
-      dst[RY * T3X / 4] = make_float4(o1[0], o1[1], o1[2], o1[3]);
-      dst[2 * RY * T3X / 4] = make_float4(o2[0], o2[1], o2[2], o2[3]);
-    }
-    __syncthreads();
-    {
-#pragma unroll
-      for (int m = 0; m < 3; ++m) {
-        float v[YO + 2 * R], a[YO];
-#pragma unroll
-        for (int k = 0; k < YO + 2 * R; ++k) v[k] = sx[(m * RY + YO * yseg + k) * T3X + col];
-        runsum<WW, YO>(v, a);
-#pragma unroll
-        for (int i = 0; i < YO; ++i) {
-          float* rp = ring + ((j * 3 + m) * T3Y + YO * yseg + i) * T3X + col;
-          S[i][m] += a[i] - *rp;
-          *rp = a[i];
-        }
-      }
-      if (j == WW - 1) {  // exact re-sum bounds the drift of the running sums
-#pragma unroll
-        for (int m = 0; m < 3; ++m)
-#pragma unroll
-          for (int i = 0; i < YO; ++i) {
-            float t = 0.f;
-            for (int q = 0; q < WW; ++q) t += ring[((q * 3 + m) * T3Y + YO * yseg + i) * T3X + col];
-            S[i][m] = t;
-          }
-      }
-      if (it >= 2 * R) {
-        const int cz = zin - 2 * R, cx = x0 + col;
-#pragma unroll
-        for (int i = 0; i < YO; ++i) {
-          const int cy = y0 + YO * yseg + i;
-          if (cx >= n.n2 || cy >= n.n1) continue;
-          const int o = cz * plane + cy * n.n2 + cx;
-          float c0 = 0.f, c1 = 0.f, c2 = 0.f;
-          if (cx <= mx && cy <= my && cz <= mz) {
-            const float muF = muF_c[i], Sff = Sff_c[i];
-            const float Sww = fmaxf(S[i][1] - S[i][0] * S[i][0] * inv_nw, 0.f);
-            const float Sfw = S[i][2] - (muF - shF) * S[i][0];
-            const float muW = S[i][0] * inv_nw + shW;
-            float val;
-            if (KIND == 0) {
-              const float beta = Sfw * Sff;  // Sff holds 1 / (S_FF + eps) for SiLNCC
-              val = (Sww - Sfw * beta) * inv_nw;
-              c0 = beta;
-              c1 = muW - beta * muF;
-            } else {
-              const float Q = Sff * Sww + eps;
-              const float rq = 1.f / sqrtf(Q);
-              val = 1.f - Sfw * rq;
-              c0 = Sfw * Sff * rq * rq * rq;
-              c1 = rq;
-              c2 = c0 * muW - c1 * muF;
-            }
-            const float yk = val - lcomp;
-            const float tk = lsum + yk;
-            lcomp = (tk - lsum) - yk;
-            lsum = tk;
-          }
-          C[o] = c0;
-          C[cstride + o] = c1;
-          if (KIND == 1) C[2 * cstride + o] = c2;
-        }
-      }
-    }
-    j = (j + 1 == WW) ? 0 : j + 1;
-  }
-  const double sum = block_sum(FF{lsum, -lcomp}, sh);
-  if (threadIdx.x == 0) part[((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = sum;
+  for (int i = 1; i < 4; ++i)
+    out[i] = __fadd_rn(out[i - 1], __fmaf_rn(a[i + WW - 1], b[i + WW - 1], -p[i - 1]));
 }
 
-template <int R, int KIND>
-__global__ void __launch_bounds__(NT3) k_sim_bwd3(const PairDesc* __restrict__ pd, const float* __restrict__ Wb,
-                                                       size_t Wstride, const float* __restrict__ coef, size_t cstride,
-                                                       float* __restrict__ dLdW, Dims n, float scale, int tz, int nzc) {
-  constexpr int NC = KIND == 0 ? 2 : 3;
-  using G = Geo3<R, NC>;
-  constexpr int WW = G::WW, RX = G::RX, RY = G::RY, RXS = G::RXS, NV = G::NV, NE = G::NE, NSLOT = G::NSLOT;
-  extern __shared__ __align__(16) float smem[];
-  float* sc = smem;                            // [NC][RY][RXS]
-  float* sx = sc + G::in_floats(NC);           // [NC][RY][T3X]
-  float* ring = sx + G::sx_floats();           // [WW][NC][T3Y][T3X]
-  const int pair = blockIdx.z / nzc, zc = blockIdx.z - pair * nzc;
-  const int x0 = blockIdx.x * T3X, y0 = blockIdx.y * T3Y, z0 = zc * tz;
-  const int tid = threadIdx.x;
-  const float* __restrict__ F = pd[pair].Ii;
-  const float* __restrict__ W = Wb + (size_t)pair * Wstride;
-  const float* __restrict__ Cf = coef + (size_t)pair * NC * cstride;
-  float* __restrict__ out = dLdW + (size_t)pair * Wstride;
-  const int plane = n.n1 * n.n2;
-  int soff[NSLOT], sidx[NSLOT];
-  bool sok[NSLOT];
+// ---- hand-over of the two buffers of W sums between the roles (named barriers; 0 is
+// __syncthreads). Whole warps take part, converged first: bar.sync / bar.arrive are aligned.
+enum { kBarFull = 1, kBarEmpty = 3, kBarStage = 5 };  // full, empty: one per buffer
+__device__ __forceinline__ void bar_sync(int id, int threads) {
+  __syncwarp();
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(int id, int threads) {
+  __syncwarp();
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// ---- staged input planes of the W warps, two stages of NIN arrays. TMA: one thread issues a
+// 4-D tile copy (x, y, z, volume) per array and plane, an mbarrier per stage tracks completion.
+// Waits are bounded: a wait that runs out sets *err and the kernel carries on without waiting (its
+// results are then reported as invalid by the host), so no CTA can hang. Otherwise every W thread
+// copies its share of a plane with 4-byte asynchronous copies, zeros outside the volume.
+__device__ __forceinline__ void copy4(float* dst, const float* src, int bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(bytes)
+               : "memory");
+}
+template <int R, int NIN, bool TMA>
+struct Stages {
+  float* stage;
+  uint64_t* bar;
+  const CUtensorMap* map[NIN];
+  int vol[NIN];
+  const float* src[NIN];  // the volumes of the unstaged path
+  int x0, y0, z0, niter, wt;
+  Dims n;
+  bool ok;
+  __device__ __forceinline__ void load(int it) {  // plane z0 + it into stage it & 1
+    using B = Box<R>;
+    float* dst = stage + (it & 1) * NIN * B::TS;
+    if (TMA) {
+      if (wt == 0) {
+        mbar_expect_tx(&bar[it & 1], (unsigned)(NIN * B::RY * B::PX * 4));
 #pragma unroll
-  for (int k = 0; k < NSLOT; ++k) {
-    const int e = tid + NT3 * k;
-    const int ry = e / RX, rx = e - ry * RX;
-    const int gy = y0 - 2 * R + ry, gx = x0 - 2 * R + rx;
-    sok[k] = e < NE && gy >= 0 && gy < n.n1 && gx >= 0 && gx < n.n2;
-    soff[k] = gy * n.n2 + gx;
-    sidx[k] = e < NE ? ry * RXS + rx : -1;
-  }
-  const int mx = n.n2 - WW, my = n.n1 - WW, mz = n.n0 - WW;
-  const int col = tid & 31, yseg = tid >> 5;
-  const int px = x0 + col;
-  float cnt_xy[YO];
-#pragma unroll
-  for (int i = 0; i < YO; ++i) {
-    const int py = y0 + YO * yseg + i;
-    const int cxn = max(0, min(px, mx) - max(0, px - 2 * R) + 1);
-    const int cyn = max(0, min(py, my) - max(0, py - 2 * R) + 1);
-    cnt_xy[i] = (float)(cxn * cyn);
-  }
-  float S[YO][NC];
-#pragma unroll
-  for (int i = 0; i < YO; ++i)
-#pragma unroll
-    for (int m = 0; m < NC; ++m) S[i][m] = 0.f;
-  for (int j = 0; j < WW; ++j)
-#pragma unroll
-    for (int m = 0; m < NC; ++m)
-#pragma unroll
-      for (int i = 0; i < YO; ++i) ring[((j * NC + m) * T3Y + YO * yseg + i) * T3X + col] = 0.f;
-  const int zend = min(z0 + tz, n.n0);
-  const int niter = (zend - z0) + 2 * R;
-  float pc[NC][NSLOT];
-  auto fetch = [&](int zin) {
-    const bool zok = zin >= 0 && zin < n.n0;
-    const int zo = zin * plane;
-#pragma unroll
-    for (int k = 0; k < NSLOT; ++k) {
-      const bool ok = zok && sok[k];
-#pragma unroll
-      for (int m = 0; m < NC; ++m) pc[m][k] = ok ? Cf[(size_t)m * cstride + zo + soff[k]] : 0.f;
-    }
-  };
-  // W and F at this thread's voxels of the next output plane (loaded one plane ahead)
-  float pwv[YO], pfv[YO];
-  const bool xin = px < n.n2;
-  auto fetch_wf = [&](int pz) {
-#pragma unroll
-    for (int i = 0; i < YO; ++i) {
-      const int py = y0 + YO * yseg + i;
-      pwv[i] = 0.f;
-      pfv[i] = 0.f;
-      if (xin && py < n.n1) {
-        const int o = pz * plane + py * n.n2 + px;
-        pwv[i] = W[o];
-        pfv[i] = F[o];
+        for (int a = 0; a < NIN; ++a) tma_load4(dst + a * B::TS, map[a], x0, y0, z0 + it, vol[a], &bar[it & 1]);
       }
-    }
-  };
-  fetch(z0 - 2 * R);
-  int j = 0;
-  for (int it = 0; it < niter; ++it) {
-    const int zin = z0 - 2 * R + it;  // corner plane
+    } else {
+      // a warp per row, columns lane and lane + 32; outside the volume the copy reads nothing
+      const int z = z0 + it, lane = wt & 31, xa = x0 + lane, xb = xa + 32;
+      const bool zin = z >= 0 && z < n.n0;
+      const int ina = zin && xa >= 0 && xa < n.n2 ? 4 : 0, inb = zin && xb >= 0 && xb < n.n2 ? 4 : 0;
+      const int ca = ina ? xa : 0, cb = inb ? xb : 0, zo = zin ? z * n.n1 : 0;
+      for (int row = wt >> 5; row < B::RY; row += B::WT / 32) {
+        const int y = y0 + row;
+        const bool yin = y >= 0 && y < n.n1;
+        const int o = (zo + (yin ? y : 0)) * n.n2;
 #pragma unroll
-    for (int k = 0; k < NSLOT; ++k)
-      if (sidx[k] >= 0) {
-#pragma unroll
-        for (int m = 0; m < NC; ++m) sc[m * RY * RXS + sidx[k]] = pc[m][k];
-      }
-    float wv_c[YO], fv_c[YO];
-#pragma unroll
-    for (int i = 0; i < YO; ++i) wv_c[i] = pwv[i], fv_c[i] = pfv[i];
-    __syncthreads();
-    if (it + 1 < niter) {
-      fetch(zin + 1);
-      if (it + 1 >= 2 * R) fetch_wf(zin + 1);
-    }
-    for (int task = tid; task < 8 * RY; task += NT3) {
-      const int xrow = task >> 3, xseg = task & 7;
-#pragma unroll
-      for (int m = 0; m < NC; ++m) {
-        float v[4 * NV];
-        const float4* src = reinterpret_cast<const float4*>(sc + (m * RY + xrow) * RXS + 4 * xseg);
-#pragma unroll
-        for (int q = 0; q < NV; ++q) {
-          const float4 a = src[q];
-          v[4 * q] = a.x, v[4 * q + 1] = a.y, v[4 * q + 2] = a.z, v[4 * q + 3] = a.w;
-        }
-        float o[4];
-        runsum<WW, 4>(v, o);
-        *reinterpret_cast<float4*>(sx + (m * RY + xrow) * T3X + 4 * xseg) = make_float4(o[0], o[1], o[2], o[3]);
-      }
-    }
-    __syncthreads();
-    {
-#pragma unroll
-      for (int m = 0; m < NC; ++m) {
-        float v[YO + 2 * R], a[YO];
-#pragma unroll
-        for (int k = 0; k < YO + 2 * R; ++k) v[k] = sx[(m * RY + YO * yseg + k) * T3X + col];
-        runsum<WW, YO>(v, a);
-#pragma unroll
-        for (int i = 0; i < YO; ++i) {
-          float* rp = ring + ((j * NC + m) * T3Y + YO * yseg + i) * T3X + col;
-          S[i][m] += a[i] - *rp;
-          *rp = a[i];
+        for (int a = 0; a < NIN; ++a) {
+          float* to = dst + a * B::TS + row * B::PX + lane;
+          copy4(to, src[a] + (o + ca), yin ? ina : 0);
+          if (lane < 2 * R) copy4(to + 32, src[a] + (o + cb), yin ? inb : 0);
         }
       }
-      if (j == WW - 1) {
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+  }
+  __device__ __forceinline__ void start() {
+    ok = true;
+    load(0);
+    if (niter > 1)
+      load(1);
+    else if (!TMA)
+      asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  __device__ __forceinline__ void wait(int it) {  // plane it is in its stage
+    if (TMA) {
+      ok = ok && mbar_wait(&bar[it & 1], (unsigned)(it >> 1) & 1u);  // after a failure, stop waiting
+    } else {
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+      bar_sync(kBarStage, Box<R>::WT);
+    }
+  }
+  __device__ __forceinline__ void next(int it) {  // every W thread is past plane it: refill its stage
+    bar_sync(kBarStage, Box<R>::WT);
+    if (TMA) {
+      if (it + 2 < niter) {
+        if (wt == 0) fence_proxy_async();
+        load(it + 2);
+      }
+    } else if (it + 2 < niter) {
+      load(it + 2);
+    } else {
+      asm volatile("cp.async.commit_group;" ::: "memory");  // keeps the group count of wait()
+    }
+  }
+  // report a failed wait, then give the copies still in flight into this CTA's stages one more
+  // bounded wait (the last use of each stage) before the CTA's shared memory is released
+  __device__ __forceinline__ void finish(int* err) {
+    if (!TMA || ok) return;
+    if (err) atomicOr(err, 1);
+    for (int st = 0; st < 2 && st < niter; ++st) {
+      const int last = niter - 1 - ((niter - 1 - st) & 1);  // last iteration that used stage st
+      mbar_wait(&bar[st], (unsigned)(last >> 1) & 1u);
+    }
+  }
+};
+
+// the 8 sums of one moment of a W task, of values or of products, into the W sums
+__device__ __forceinline__ void store8(float* __restrict__ dst, const float (&o)[kXO]) {
+  *reinterpret_cast<float4*>(dst) = make_float4(o[0], o[1], o[2], o[3]);
+  *reinterpret_cast<float4*>(dst + 4) = make_float4(o[4], o[5], o[6], o[7]);
+}
+template <int R>
+__device__ __forceinline__ void w_sums(const float* v, float* __restrict__ dst) {
+  float o[kXO];
+  runsum<Box<R>::WW, 4>(v, o);
+  runsum<Box<R>::WW, 4>(v + 4, o + 4);
+  store8(dst, o);
+}
+template <int R>
+__device__ __forceinline__ void w_sums(const float* a, const float* b, float* __restrict__ dst) {
+  float o[kXO];
+  runsum4<Box<R>::WW>(a, b, o);
+  runsum4<Box<R>::WW>(a + 4, b + 4, o + 4);
+  store8(dst, o);
+}
+
+// H and D passes of one plane for a thread's column and rows: S += newest - oldest plane sum,
+// re-summed from the ring when its last slot was written (as a tree, or with SEQ one after the other)
+template <int R, int NM, bool SEQ = false>
+struct Ring {
+  static constexpr int kSlot = kHD;  // float4 (the thread's rows) of one moment of one plane
+  float4* mem;
+  float S[NM][kYO];
+  int j;
+  __device__ __forceinline__ void init(float* base) {
+    mem = reinterpret_cast<float4*>(base) + threadIdx.x;
+    j = 0;
 #pragma unroll
-        for (int m = 0; m < NC; ++m)
+    for (int m = 0; m < NM; ++m)
 #pragma unroll
-          for (int i = 0; i < YO; ++i) {
-            float t[WW];
+      for (int i = 0; i < kYO; ++i) S[m][i] = 0.f;
 #pragma unroll
-            for (int q = 0; q < WW; ++q) t[q] = ring[((q * NC + m) * T3Y + YO * yseg + i) * T3X + col];
-            S[i][m] = TreeSum<WW>::of(t);
+    for (int q = 0; q < NM * Box<R>::WW; ++q) mem[q * kSlot] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  // plane h of niter from its buffer of W sums: waits for it and hands it back once read
+  __device__ __forceinline__ void plane(const float* sx2, int h, int niter, int col, int row) {
+    using B = Box<R>;
+    bar_sync(kBarFull + (h & 1), B::NT);
+    const float* sx = sx2 + (h & 1) * B::sx_floats(NM) + row * B::PS + col;
+    float a[NM][kYO];
+#pragma unroll
+    for (int m = 0; m < NM; ++m) {
+      float v[kYO + 2 * R];
+#pragma unroll
+      for (int k = 0; k < kYO + 2 * R; ++k) v[k] = sx[(m * B::RY + k) * B::PS];
+#pragma unroll
+      for (int i = 0; i < kYO; i += 2) runsum<B::WW, 2>(v + i, a[m] + i);
+    }
+    if (h + 2 < niter) bar_arrive(kBarEmpty + (h & 1), B::NT);
+#pragma unroll
+    for (int m = 0; m < NM; ++m) {
+      float4* rp = mem + (j * NM + m) * kSlot;
+      const float4 old = *rp;
+      S[m][0] += a[m][0] - old.x;
+      S[m][1] += a[m][1] - old.y;
+      S[m][2] += a[m][2] - old.z;
+      S[m][3] += a[m][3] - old.w;
+      *rp = make_float4(a[m][0], a[m][1], a[m][2], a[m][3]);
+    }
+    if (++j == B::WW) {  // exact re-sum bounds the drift of the running sums
+      j = 0;
+#pragma unroll
+      for (int m = 0; m < NM; ++m) {
+        float t[kYO][B::WW];
+#pragma unroll
+        for (int q = 0; q < B::WW; ++q) {
+          const float4 r = mem[(q * NM + m) * kSlot];
+          t[0][q] = r.x, t[1][q] = r.y, t[2][q] = r.z, t[3][q] = r.w;
+        }
+#pragma unroll
+        for (int i = 0; i < kYO; ++i) {
+          if (SEQ) {
+            S[m][i] = t[i][0];
+#pragma unroll
+            for (int q = 1; q < B::WW; ++q) S[m][i] += t[i][q];
+          } else {
+            S[m][i] = TreeSum<B::WW>::of(t[i]);
           }
-      }
-      if (it >= 2 * R) {
-        const int pz = zin;
-        const int czn = max(0, min(pz, mz) - max(0, pz - 2 * R) + 1);
-#pragma unroll
-        for (int i = 0; i < YO; ++i) {
-          const int py = y0 + YO * yseg + i;
-          if (px >= n.n2 || py >= n.n1) continue;
-          const int o = pz * plane + py * n.n2 + px;
-          const float wv = wv_c[i], fv = fv_c[i];
-          float g;
-          if (KIND == 0)
-            g = scale * (cnt_xy[i] * (float)czn * wv - fv * S[i][0] - S[i][1]);
-          else
-            g = scale * (wv * S[i][0] - fv * S[i][1] - S[i][2]);
-          out[o] = g;
         }
       }
     }
-    j = (j + 1 == WW) ? 0 : j + 1;
   }
+};
+
+// number of window corners in [0, last] that hold offset k (0 when last < 0)
+__device__ __forceinline__ int corners_holding(int k, int last, int reach) {
+  return max(0, min(k, last) - max(0, k - reach) + 1);
 }
 
-// ---------------------------------------------------------------------------
-// The same two kernels with the input planes staged by the tensor memory
-// accelerator: one thread issues a 4-D tile copy (x, y, z, volume) per array and
-// plane into one of two shared-memory stages, completion is tracked by an
-// mbarrier per stage, and the copy of plane z+2 is issued as soon as every
-// thread is past the W pass of plane z (the only reader of a stage). The W sums
-// are double-buffered: one iteration runs the W pass of plane z and the H and D
-// passes of plane z-1, so a plane costs one barrier. The D ring keeps a thread's two
-// rows side by side (one 8-byte load and store per moment and plane). Boxes that
-// reach outside a volume are filled with zeros by the copy engine. Waits are
-// bounded: a wait that runs out sets *err and the kernel carries on (its results
-// are then reported as invalid by the host), so no CTA can hang.
-// floats of one staged plane (box RXS x RY), rounded up to 128-byte multiples
-template <int R, int NM>
-__host__ __device__ constexpr int stage_floats() {
-  return ((Geo3<R, NM>::RY * Geo3<R, NM>::RXS) + 31) & ~31;
-}
+// CTAs per SM the register budget is cut for (shared memory allows 4 for w <= 7)
+constexpr int kMinCtas = 4;
 
-template <int R, int KIND>
-__global__ void __launch_bounds__(NT3) k_sim_fwd3t(const __grid_constant__ SimMaps maps, const PairDesc* __restrict__ pd,
-                                                   const float* __restrict__ Wb, size_t Wstride,
-                                                   float* __restrict__ coef, size_t cstride,
-                                                   double* __restrict__ part, Dims n, float eps, int tz, int nzc,
-                                                   int* __restrict__ err) {
-  using G = Geo3<R, 3>;
-  constexpr int WW = G::WW, RY = G::RY, RXS = G::RXS, NV = G::NV;
-  constexpr int NC = KIND == 0 ? 2 : 3;
-  constexpr int TS = stage_floats<R, 3>();
-  constexpr unsigned kBytes = 2u * RY * RXS * 4u;  // F and W boxes of one plane
-  extern __shared__ __align__(128) float smem_raw[];
-  float* smem = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
-  float* stage = smem;                      // [2 stages][F, W][TS]
-  float* sx2 = stage + 4 * TS;              // [2 planes][3][RY][T3X]
-  // [WW][3][T3Y / YO][T3X] pairs: a thread's YO = 2 rows side by side (one 8-byte access)
-  float2* ring2 = reinterpret_cast<float2*>(sx2 + 2 * G::sx_floats());
+// Forward of one pair (see the head of the file).
+template <int R, int KIND, bool TMA>
+__global__ void __launch_bounds__(Box<R>::NT, kMinCtas)
+    k_sim_fwd(const __grid_constant__ SimMaps maps, const PairDesc* __restrict__ pd, const float* __restrict__ Wb,
+              size_t Wstride, float* __restrict__ coef, size_t cstride, double* __restrict__ part, Dims n, Tiles g,
+              float eps, int* __restrict__ err) {
+  using B = Box<R>;
+  constexpr int NM = KIND == 0 ? 2 : 3, NC = KIND == 0 ? 2 : 3;
+  extern __shared__ __align__(128) float smem[];
+  float* sx2 = smem + 4 * B::TS;  // stages: [2][F, W][TS]
   __shared__ __align__(8) uint64_t bar[2];
-  __shared__ float sh[2 * (NT3 / 32)];
-  const int pair = blockIdx.z / nzc, zc = blockIdx.z - pair * nzc;
-  const int x0 = blockIdx.x * T3X, y0 = blockIdx.y * T3Y, z0 = zc * tz;
-  const int tid = threadIdx.x;
-  const PairDesc d = pd[pair];
-  const float* __restrict__ F = d.Ii;
-  const float* __restrict__ Fs = d.Fs;
-  const float* __restrict__ W = Wb + (size_t)pair * Wstride;
-  float* __restrict__ C = coef + (size_t)pair * NC * cstride;
+  __shared__ float sh[2 * (B::NT / 32)];
+  const Tile t = tile_of(g);
   const int plane = n.n1 * n.n2;
-  const int zend = min(z0 + tz, n.n0);
-  const int niter = (zend - z0) + 2 * R;
-  if (tid == 0) {
+  const PairDesc d = pd[t.pair];
+  const float* __restrict__ F = d.Ii;
+  const float* __restrict__ W = Wb + (size_t)t.pair * Wstride;
+  const int zend = min(t.z0 + g.tz, n.n0), niter = (zend - t.z0) + 2 * R;
+  const int mx = n.n2 - B::WW, my = n.n1 - B::WW, mz = n.n0 - B::WW;
+  const int so = min(t.z0 + R, n.n0 - 1) * plane + min(t.y0 + R, n.n1 - 1) * n.n2 + min(t.x0 + R, n.n2 - 1);
+  const float shF = F[so], shW = W[so];
+  const int wt = (int)threadIdx.x - kHD;  // W thread, or an H/D thread when negative
+  if (TMA && wt == 0) {
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
     mbar_fence_init();
   }
   __syncthreads();
-  auto issue = [&](int it) {  // one thread: plane z0 + it of F and W into stage it & 1
-    const int st = it & 1;
-    mbar_expect_tx(&bar[st], kBytes);
-    tma_load4(stage + (2 * st) * TS, &maps.F, x0, y0, z0 + it, d.fi, &bar[st]);
-    tma_load4(stage + (2 * st + 1) * TS, &maps.W, x0, y0, z0 + it, pair, &bar[st]);
-  };
-  if (tid == 0) {
-    issue(0);
-    if (niter > 1) issue(1);
-  }
-  const int so = min(z0 + R, n.n0 - 1) * plane + min(y0 + R, n.n1 - 1) * n.n2 + min(x0 + R, n.n2 - 1);
-  const float shF = F[so], shW = W[so];
-  const float inv_nw = 1.f / (float)(WW * WW * WW);
-  const int mx = n.n2 - WW, my = n.n1 - WW, mz = n.n0 - WW;
-  const int col = tid & 31, yseg = tid >> 5;
-  float S[YO][3];
+  // SiLNCC: W threads sum_p cnt(p) W'(p)^2, H/D threads sum_R ((sum W')^2/|R| + beta S_FW);
+  // LNCC: H/D threads sum_R Sim_R
+  KSum acc;
+  if (wt >= 0) {
+    Stages<R, 2, TMA> st{smem, bar, {&maps.F, &maps.W}, {d.fi, t.pair}, {F, W}, t.x0, t.y0, t.z0, niter, wt, n, true};
+    st.start();
+    const bool on = wt < B::NTASK;
+    const int row = wt >> 2, xs = kXO * (wt & 3);
+    // how many of the tile's windows hold a voxel of this row, per axis (along W: valid corners
+    // of this task, all kXO of them except at the volume's end)
+    const int cnt_y = on ? corners_holding(row, min(kTY - 1, my - t.y0), 2 * R) : 0;
+    const int last_x = min(kXO - 1, mx - t.x0 - xs), last_z = min(zend - 1, mz) - t.z0;
+    for (int it = 0; it < niter; ++it) {
+      if (it >= 2) bar_sync(kBarEmpty + (it & 1), B::NT);
+      st.wait(it);
+      float f[4 * B::NV], w[4 * B::NV];
+      if (on) {
+        const float4* pF = reinterpret_cast<const float4*>(smem + 2 * (it & 1) * B::TS + row * B::PX + xs);
+        const float4* pW = pF + B::TS / 4;
 #pragma unroll
-  for (int i = 0; i < YO; ++i)
-#pragma unroll
-    for (int m = 0; m < 3; ++m) S[i][m] = 0.f;
-  for (int j = 0; j < WW; ++j)
-#pragma unroll
-    for (int m = 0; m < 3; ++m) ring2[((j * 3 + m) * (T3Y / YO) + yseg) * T3X + col] = make_float2(0.f, 0.f);
-  float lsum = 0.f, lcomp = 0.f;
-  const bool xin = x0 + col <= mx;
-  int j = 0;
-  bool ok = true;
-  // Iteration it runs the W pass of input plane it (into sx buffer it & 1) and the H and
-  // D passes of plane it - 1 (from the other buffer): one barrier per plane, and warps
-  // without a W-pass task go straight on to their H pass.
-  for (int it = 0; it <= niter; ++it) {
-    const int h = it - 1;  // plane of the H and D passes
-    // mu_F and S_FF of this thread's windows of the output plane (corner plane h - 2R),
-    // loaded now and used after the W pass
-    float muF_c[YO], Sff_c[YO];
-    const bool outp = h >= 2 * R;
-#pragma unroll
-    for (int i = 0; i < YO; ++i) {
-      const int cy = y0 + YO * yseg + i, cz = z0 + h - 2 * R;
-      muF_c[i] = 0.f;
-      Sff_c[i] = 0.f;
-      if (outp && xin && cy <= my && cz <= mz) {
-        const int o = cz * plane + cy * n.n2 + x0 + col;
-        muF_c[i] = Fs[o];
-        Sff_c[i] = Fs[(size_t)plane * n.n0 + o];
-      }
-    }
-    if (it < niter) {
-      const int st = it & 1;
-      ok = ok && mbar_wait(&bar[st], (unsigned)(it >> 1) & 1u);  // after a failure, stop waiting
-      const float* sF = stage + (2 * st) * TS;
-      const float* sW = sF + TS;
-      float* sx = sx2 + st * G::sx_floats();
-      for (int task = tid; task < 8 * RY; task += NT3) {
-        const int xrow = task >> 3, xseg = task & 7;
-        float f[4 * NV], w[4 * NV];
-        const float4* pF = reinterpret_cast<const float4*>(sF + xrow * RXS + 4 * xseg);
-        const float4* pW = reinterpret_cast<const float4*>(sW + xrow * RXS + 4 * xseg);
-#pragma unroll
-        for (int q = 0; q < NV; ++q) {
+        for (int q = 0; q < (B::NI + 3) / 4; ++q) {
           const float4 a = pF[q], b = pW[q];
           f[4 * q] = a.x - shF, f[4 * q + 1] = a.y - shF, f[4 * q + 2] = a.z - shF, f[4 * q + 3] = a.w - shF;
           w[4 * q] = b.x - shW, w[4 * q + 1] = b.y - shW, w[4 * q + 2] = b.z - shW, w[4 * q + 3] = b.w - shW;
         }
-        float ww[4 + 2 * R], fw[4 + 2 * R];
-#pragma unroll
-        for (int k = 0; k < 4 + 2 * R; ++k) {
-          ww[k] = w[k] * w[k];
-          fw[k] = f[k] * w[k];
-        }
-        float o0[4], o1[4], o2[4];
-        runsum<WW, 4>(w, o0);
-        runsum<WW, 4>(ww, o1);
-        runsum<WW, 4>(fw, o2);
-        float4* dst = reinterpret_cast<float4*>(sx + xrow * T3X + 4 * xseg);
-        dst[0] = make_float4(o0[0], o0[1], o0[2], o0[3]);
-        dst[RY * T3X / 4] = make_float4(o1[0], o1[1], o1[2], o1[3]);
-        dst[2 * RY * T3X / 4] = make_float4(o2[0], o2[1], o2[2], o2[3]);
+        float* sx = sx2 + (it & 1) * B::sx_floats(NM) + row * B::PS + xs;
+        w_sums<R>(w, sx);
+        w_sums<R>(f, w, sx + (NM - 1) * B::RY * B::PS);
+        if (KIND == 1) w_sums<R>(w, w, sx + B::RY * B::PS);
       }
-    }
-    if (h >= 0) {
-      const float* sx = sx2 + (h & 1) * G::sx_floats();
+      bar_arrive(kBarFull + (it & 1), B::NT);
+      if (KIND == 0) {
+        // a voxel that no window holds adds nothing, whatever it is (0 * Inf)
+        const int c = cnt_y * corners_holding(it, last_z, 2 * R);
+        if (c > 0 && last_x >= 0) {
+          float a = 0.f;
+          if (last_x == kXO - 1) {
 #pragma unroll
-      for (int m = 0; m < 3; ++m) {
-        float v[YO + 2 * R], a[YO];
-#pragma unroll
-        for (int k = 0; k < YO + 2 * R; ++k) v[k] = sx[(m * RY + YO * yseg + k) * T3X + col];
-        runsum<WW, YO>(v, a);
-        float2* rp = ring2 + ((j * 3 + m) * (T3Y / YO) + yseg) * T3X + col;
-        const float2 old = *rp;
-        S[0][m] += a[0] - old.x;
-        S[1][m] += a[1] - old.y;
-        *rp = make_float2(a[0], a[1]);
-      }
-      if (j == WW - 1) {
-#pragma unroll
-        for (int m = 0; m < 3; ++m) {
-          float t0[WW], t1[WW];
-#pragma unroll
-          for (int q = 0; q < WW; ++q) {
-            const float2 r = ring2[((q * 3 + m) * (T3Y / YO) + yseg) * T3X + col];
-            t0[q] = r.x;
-            t1[q] = r.y;
-          }
-          S[0][m] = TreeSum<WW>::of(t0);
-          S[1][m] = TreeSum<WW>::of(t1);
-        }
-      }
-      if (outp) {
-        const int cz = z0 + h - 2 * R, cx = x0 + col;
-#pragma unroll
-        for (int i = 0; i < YO; ++i) {
-          const int cy = y0 + YO * yseg + i;
-          if (cx >= n.n2 || cy >= n.n1) continue;
-          const int o = cz * plane + cy * n.n2 + cx;
-          float c0 = 0.f, c1 = 0.f, c2 = 0.f;
-          if (cx <= mx && cy <= my && cz <= mz) {
-            const float muF = muF_c[i], Sff = Sff_c[i];
-            const float Sww = fmaxf(S[i][1] - S[i][0] * S[i][0] * inv_nw, 0.f);
-            const float Sfw = S[i][2] - (muF - shF) * S[i][0];
-            const float muW = S[i][0] * inv_nw + shW;
-            float val;
-            if (KIND == 0) {
-              const float beta = Sfw * Sff;  // Sff holds 1 / (S_FF + eps) for SiLNCC
-              val = (Sww - Sfw * beta) * inv_nw;
-              c0 = beta;
-              c1 = muW - beta * muF;
-            } else {
-              const float Q = Sff * Sww + eps;
-              const float rq = 1.f / sqrtf(Q);
-              val = 1.f - Sfw * rq;
-              c0 = Sfw * Sff * rq * rq * rq;
-              c1 = rq;
-              c2 = c0 * muW - c1 * muF;
+            for (int k = 0; k < B::NI; ++k) {
+              const int q = (k < kXO - 1 ? k : kXO - 1) - (k > 2 * R ? k - 2 * R : 0) + 1;
+              a = fmaf((float)q * w[k], w[k], a);
             }
-            const float yk = val - lcomp;
-            const float tk = lsum + yk;
-            lcomp = (tk - lsum) - yk;
-            lsum = tk;
+          } else {
+#pragma unroll
+            for (int k = 0; k < B::NI; ++k) a = fmaf((float)corners_holding(k, last_x, 2 * R) * w[k], w[k], a);
           }
-          C[o] = c0;
-          C[cstride + o] = c1;
-          if (KIND == 1) C[2 * cstride + o] = c2;
+          acc.add((float)c * a);
         }
       }
-      j = (j + 1 == WW) ? 0 : j + 1;
+      st.next(it);
     }
-    // the W pass of this plane is done with its stage (refilled below) and the H pass of
-    // the previous plane with its sx buffer (rewritten by the next W pass)
-    __syncthreads();
-    if (tid == 0 && it + 2 < niter) {
-      fence_proxy_async();
-      issue(it + 2);
+    st.finish(err);
+  } else {
+    const float inv_nw = 1.f / (float)(B::WW * B::WW * B::WW);
+    const int col = threadIdx.x & 31, row = (threadIdx.x >> 5) * kYO;
+    const int cx = t.x0 + col, cy = t.y0 + row;
+    const int rows = cx < n.n2 ? min(kYO, n.n1 - cy) : 0;            // rows inside the volume
+    const int live_rows = cx <= mx ? min(rows, my - cy + 1) : 0;     // rows whose window is inside (H and W)
+    const ptrdiff_t o0 = (ptrdiff_t)t.z0 * plane + (ptrdiff_t)cy * n.n2 + cx;
+    const float* __restrict__ mu_p = d.Fs + o0;
+    const float* __restrict__ sf_p = mu_p + (size_t)plane * n.n0;
+    float* __restrict__ c_p = coef + (size_t)t.pair * NC * cstride + o0;
+    Ring<R, NM, !TMA> ring;
+    ring.init(sx2 + 2 * B::sx_floats(NM));
+    // coefficients of row i's window and its term of the loss
+    auto window = [&](int i, float muF, float Sff, float& c0, float& c1, float& c2) -> float {
+      const float s0 = ring.S[0][i];
+      const float Sfw = ring.S[NM - 1][i] - (muF - shF) * s0;
+      const float muW = s0 * inv_nw + shW;
+      if (KIND == 0) {
+        const float beta = Sfw * Sff;  // Sff holds 1 / (S_FF + eps) for SiLNCC
+        c0 = beta;
+        c1 = muW - beta * muF;
+        return fmaf(Sfw, beta, s0 * s0 * inv_nw);
+      }
+      const float Sww = fmaxf(ring.S[1][i] - s0 * s0 * inv_nw, 0.f);
+      const float Q = Sff * Sww + eps;
+      const float rq = 1.f / sqrtf(Q);
+      c0 = Sfw * Sff * rq * rq * rq;
+      c1 = rq;
+      c2 = c0 * muW - c1 * muF;
+      return 1.f - Sfw * rq;
+    };
+    for (int h = 0; h < niter; ++h) {
+      // mu_F and S_FF of this thread's windows of the output plane (corner plane h - 2R), loaded
+      // now and used after the passes
+      const bool outp = h >= 2 * R;
+      const int nl = outp && t.z0 + h - 2 * R <= mz ? live_rows : 0;
+      float mu[kYO], sf[kYO];
+      if (nl == kYO) {
+#pragma unroll
+        for (int i = 0; i < kYO; ++i) {
+          mu[i] = __ldg(mu_p + i * n.n2);
+          sf[i] = __ldg(sf_p + i * n.n2);
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < kYO; ++i)
+          if (i < nl) {
+            mu[i] = __ldg(mu_p + i * n.n2);
+            sf[i] = __ldg(sf_p + i * n.n2);
+          }
+      }
+      ring.plane(sx2, h, niter, col, row);
+      if (outp) {
+        if (nl == kYO) {
+          float val[kYO];
+#pragma unroll
+          for (int i = 0; i < kYO; ++i) {
+            float c0, c1, c2;
+            val[i] = window(i, mu[i], sf[i], c0, c1, c2);
+            c_p[i * n.n2] = c0;
+            c_p[cstride + i * n.n2] = c1;
+            if (KIND == 1) c_p[2 * cstride + i * n.n2] = c2;
+          }
+          acc.add((val[0] + val[1]) + (val[2] + val[3]));
+        } else {
+#pragma unroll
+          for (int i = 0; i < kYO; ++i)
+            if (i < rows) {
+              float c0 = 0.f, c1 = 0.f, c2 = 0.f;
+              if (i < nl) acc.add(window(i, mu[i], sf[i], c0, c1, c2));
+              c_p[i * n.n2] = c0;
+              c_p[cstride + i * n.n2] = c1;
+              if (KIND == 1) c_p[2 * cstride + i * n.n2] = c2;
+            }
+        }
+        mu_p += plane, sf_p += plane, c_p += plane;
+      }
     }
   }
-  if (!ok) {
-    // report, then give the copies still in flight into this CTA's stages one more bounded
-    // wait (the last use of each stage) before the CTA's shared memory is released
-    if (err) atomicOr(err, 1);
-    for (int st = 0; st < 2 && st < niter; ++st) {
-      const int last = niter - 1 - ((niter - 1 - st) & 1);  // last iteration that used stage st
-      mbar_wait(&bar[st], (unsigned)(last >> 1) & 1u);
-    }
-  }
-  const double sum = block_sum(FF{lsum, -lcomp}, sh);
-  if (threadIdx.x == 0) part[((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = sum;
+  const float sgn = KIND == 0 && wt < 0 ? -1.f : 1.f;
+  const double sum = block_sum<B::NT>(FF{sgn * acc.s, -sgn * acc.c}, sh);
+  if (threadIdx.x == 0) part[t.part] = KIND == 0 ? sum / (double)(B::WW * B::WW * B::WW) : sum;
 }
 
-// x offset of the adjoint's staged box: its first column x0 - 2R is rounded down to a
-// multiple of 4 (16-byte aligned tile coordinate), so the box starts XOFF columns early
-template <int R>
-__host__ __device__ constexpr int bwd_xoff() {
-  return (2 * R) & 3;
-}
-
-template <int R, int KIND>
-__global__ void __launch_bounds__(NT3) k_sim_bwd3t(const __grid_constant__ SimMaps maps, const PairDesc* __restrict__ pd,
-                                                   const float* __restrict__ Wb, size_t Wstride,
-                                                   float* __restrict__ dLdW, Dims n, float scale, int tz, int nzc,
-                                                   int* __restrict__ err) {
-  constexpr int NC = KIND == 0 ? 2 : 3;
-  using G = Geo3<R, NC>;
-  constexpr int WW = G::WW, RY = G::RY, RXS = G::RXS;
-  constexpr int XOFF = bwd_xoff<R>();
-  constexpr int TS = stage_floats<R, NC>();
-  constexpr unsigned kBytes = (unsigned)NC * RY * RXS * 4u;
-  static_assert(XOFF + 4 * 7 + 4 + 2 * R <= RXS, "staged box too narrow for the W pass");
-  static_assert((2 * R + XOFF) % 4 == 0, "the staged adjoint box must start at a multiple of 4 floats");
-  extern __shared__ __align__(128) float smem_raw[];
-  float* smem = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
-  float* stage = smem;                      // [2 stages][NC][TS]
-  float* sx2 = stage + 2 * NC * TS;         // [2 planes][NC][RY][T3X]
-  // [WW][NC][T3Y / YO][T3X] pairs: a thread's YO = 2 rows side by side (one 8-byte access)
-  float2* ring2 = reinterpret_cast<float2*>(sx2 + 2 * G::sx_floats());
+template <int R, int KIND, bool TMA>
+__global__ void __launch_bounds__(Box<R>::NT, kMinCtas)
+    k_sim_bwd(const __grid_constant__ SimMaps maps, const PairDesc* __restrict__ pd, const float* __restrict__ Wb,
+              size_t Wstride, const float* __restrict__ coef, size_t cstride, float* __restrict__ dLdW, Dims n, Tiles g,
+              float scale, int* __restrict__ err) {
+  using B = Box<R>;
+  constexpr int NC = KIND == 0 ? 2 : 3, XOFF = TMA ? bwd_xoff<R>() : 0;
+  static_assert(!TMA || (2 * R + XOFF) % 4 == 0, "the staged adjoint box must start at a multiple of 4 floats");
+  extern __shared__ __align__(128) float smem[];
+  float* sx2 = smem + 2 * NC * B::TS;  // stages: [2][NC][TS]
   __shared__ __align__(8) uint64_t bar[2];
-  const int pair = blockIdx.z / nzc, zc = blockIdx.z - pair * nzc;
-  const int x0 = blockIdx.x * T3X, y0 = blockIdx.y * T3Y, z0 = zc * tz;
-  const int tid = threadIdx.x;
-  const float* __restrict__ F = pd[pair].Ii;
-  const float* __restrict__ W = Wb + (size_t)pair * Wstride;
-  float* __restrict__ out = dLdW + (size_t)pair * Wstride;
+  const Tile t = tile_of(g);
   const int plane = n.n1 * n.n2;
-  const int zend = min(z0 + tz, n.n0);
-  const int niter = (zend - z0) + 2 * R;
-  if (tid == 0) {
+  const int zend = min(t.z0 + g.tz, n.n0), niter = (zend - t.z0) + 2 * R;
+  const int wt = (int)threadIdx.x - kHD;  // W thread, or an H/D thread when negative
+  if (TMA && wt == 0) {
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
     mbar_fence_init();
   }
   __syncthreads();
-  auto issue = [&](int it) {  // coefficient planes of corner plane z0 - 2R + it into stage it & 1
-    const int st = it & 1;
-    mbar_expect_tx(&bar[st], kBytes);
+  if (wt >= 0) {
+    Stages<R, NC, TMA> st;
+    st.stage = smem, st.bar = bar, st.niter = niter, st.wt = wt, st.n = n;
+    st.x0 = t.x0 - 2 * R - XOFF, st.y0 = t.y0 - 2 * R, st.z0 = t.z0 - 2 * R;
 #pragma unroll
-    for (int m = 0; m < NC; ++m)
-      tma_load4(stage + (st * NC + m) * TS, &maps.C, x0 - 2 * R - XOFF, y0 - 2 * R, z0 - 2 * R + it, pair * NC + m,
-                &bar[st]);
+    for (int m = 0; m < NC; ++m) {
+      st.map[m] = &maps.C;
+      st.vol[m] = t.pair * NC + m;
+      st.src[m] = coef + ((size_t)t.pair * NC + m) * cstride;
+    }
+    st.start();
+    const bool on = wt < B::NTASK;
+    const int row = wt >> 2, xs = kXO * (wt & 3);
+    for (int it = 0; it < niter; ++it) {
+      if (it >= 2) bar_sync(kBarEmpty + (it & 1), B::NT);
+      st.wait(it);
+      if (on) {
+        float* sx = sx2 + (it & 1) * B::sx_floats(NC) + row * B::PS + xs;
+#pragma unroll
+        for (int m = 0; m < NC; ++m) {
+          float v[4 * B::NV];
+          const float4* src = reinterpret_cast<const float4*>(smem + (NC * (it & 1) + m) * B::TS + row * B::PX + xs);
+#pragma unroll
+          for (int q = 0; q < (B::NI + XOFF + 3) / 4; ++q) {
+            const float4 a = src[q];
+            v[4 * q] = a.x, v[4 * q + 1] = a.y, v[4 * q + 2] = a.z, v[4 * q + 3] = a.w;
+          }
+          w_sums<R>(v + XOFF, sx + m * B::RY * B::PS);
+        }
+      }
+      bar_arrive(kBarFull + (it & 1), B::NT);
+      st.next(it);
+    }
+    st.finish(err);
+    return;
+  }
+  const int mx = n.n2 - B::WW, my = n.n1 - B::WW, mz = n.n0 - B::WW;
+  const int col = threadIdx.x & 31, row = (threadIdx.x >> 5) * kYO;
+  const int px = t.x0 + col, py = t.y0 + row;
+  const int rows = px < n.n2 ? min(kYO, n.n1 - py) : 0;
+  float cnt_xy[kYO];  // valid windows that hold the voxel, in the plane
+#pragma unroll
+  for (int i = 0; i < kYO; ++i)
+    cnt_xy[i] = (float)(corners_holding(px, mx, 2 * R) * corners_holding(py + i, my, 2 * R));
+  const ptrdiff_t o0 = (ptrdiff_t)t.z0 * plane + (ptrdiff_t)py * n.n2 + px;
+  const float* __restrict__ F_p = pd[t.pair].Ii + o0;
+  const float* __restrict__ W_p = Wb + (size_t)t.pair * Wstride + o0;
+  float* __restrict__ out = dLdW + (size_t)t.pair * Wstride + o0;
+  Ring<R, NC> ring;
+  ring.init(sx2 + 2 * B::sx_floats(NC));
+  auto gradient = [&](int i, float czn, float wv, float fv) {
+    if (KIND == 0) return scale * (cnt_xy[i] * czn * wv - fv * ring.S[0][i] - ring.S[1][i]);
+    return scale * (wv * ring.S[0][i] - fv * ring.S[1][i] - ring.S[NC - 1][i]);
   };
-  if (tid == 0) {
-    issue(0);
-    if (niter > 1) issue(1);
-  }
-  const int mx = n.n2 - WW, my = n.n1 - WW, mz = n.n0 - WW;
-  const int col = tid & 31, yseg = tid >> 5;
-  const int px = x0 + col;
-  float cnt_xy[YO];
+  for (int h = 0; h < niter; ++h) {
+    // W and F at this thread's voxels of the output plane, loaded now, used after the passes
+    const int nr = h >= 2 * R ? rows : 0;
+    float wv[kYO], fv[kYO];
+    if (nr == kYO) {
 #pragma unroll
-  for (int i = 0; i < YO; ++i) {
-    const int py = y0 + YO * yseg + i;
-    const int cxn = max(0, min(px, mx) - max(0, px - 2 * R) + 1);
-    const int cyn = max(0, min(py, my) - max(0, py - 2 * R) + 1);
-    cnt_xy[i] = (float)(cxn * cyn);
-  }
-  float S[YO][NC];
-#pragma unroll
-  for (int i = 0; i < YO; ++i)
-#pragma unroll
-    for (int m = 0; m < NC; ++m) S[i][m] = 0.f;
-  for (int j = 0; j < WW; ++j)
-#pragma unroll
-    for (int m = 0; m < NC; ++m) ring2[((j * NC + m) * (T3Y / YO) + yseg) * T3X + col] = make_float2(0.f, 0.f);
-  const bool xin = px < n.n2;
-  int j = 0;
-  bool ok = true;
-  // Iteration it runs the W pass of corner plane it (into sx buffer it & 1) and the H and
-  // D passes of corner plane it - 1 (from the other buffer): one barrier per plane.
-  // two planes per loop body: 2 % faster for this kernel (the forward one is faster rolled)
-#pragma unroll 2
-  for (int it = 0; it <= niter; ++it) {
-    const int h = it - 1;               // corner plane of the H and D passes
-    const int pz = z0 - 2 * R + h;      // output plane completed by it
-    const bool outp = h >= 2 * R;
-    // W and F at this thread's voxels of the output plane, loaded now, used after the W pass
-    float wv_c[YO], fv_c[YO];
-#pragma unroll
-    for (int i = 0; i < YO; ++i) {
-      const int py = y0 + YO * yseg + i;
-      wv_c[i] = 0.f;
-      fv_c[i] = 0.f;
-      if (outp && xin && py < n.n1) {
-        const int o = pz * plane + py * n.n2 + px;
-        wv_c[i] = W[o];
-        fv_c[i] = F[o];
+      for (int i = 0; i < kYO; ++i) {
+        wv[i] = __ldg(W_p + i * n.n2);
+        fv[i] = __ldg(F_p + i * n.n2);
       }
-    }
-    if (it < niter) {
-      const int st = it & 1;
-      ok = ok && mbar_wait(&bar[st], (unsigned)(it >> 1) & 1u);  // after a failure, stop waiting
-      float* sx = sx2 + st * G::sx_floats();
-      for (int task = tid; task < 8 * RY; task += NT3) {
-        const int xrow = task >> 3, xseg = task & 7;
+    } else {
 #pragma unroll
-        for (int m = 0; m < NC; ++m) {
-          float v[4 + 2 * R];  // the 4 + 2R inputs of 4 running outputs, as 2 + R 8-byte loads
-          const float2* src =
-              reinterpret_cast<const float2*>(stage + (st * NC + m) * TS + xrow * RXS + XOFF + 4 * xseg);
-#pragma unroll
-          for (int q = 0; q < 2 + R; ++q) {
-            const float2 a = src[q];
-            v[2 * q] = a.x, v[2 * q + 1] = a.y;
-          }
-          float o[4];
-          runsum<WW, 4>(v, o);
-          *reinterpret_cast<float4*>(sx + (m * RY + xrow) * T3X + 4 * xseg) = make_float4(o[0], o[1], o[2], o[3]);
+      for (int i = 0; i < kYO; ++i)
+        if (i < nr) {
+          wv[i] = __ldg(W_p + i * n.n2);
+          fv[i] = __ldg(F_p + i * n.n2);
         }
-      }
     }
-    if (h >= 0) {
-      const float* sx = sx2 + (h & 1) * G::sx_floats();
+    ring.plane(sx2, h, niter, col, row);
+    if (h >= 2 * R) {
+      const float czn = (float)corners_holding(t.z0 - 2 * R + h, mz, 2 * R);
+      if (nr == kYO) {
 #pragma unroll
-      for (int m = 0; m < NC; ++m) {
-        float v[YO + 2 * R], a[YO];
+        for (int i = 0; i < kYO; ++i) out[i * n.n2] = gradient(i, czn, wv[i], fv[i]);
+      } else {
 #pragma unroll
-        for (int k = 0; k < YO + 2 * R; ++k) v[k] = sx[(m * RY + YO * yseg + k) * T3X + col];
-        runsum<WW, YO>(v, a);
-        float2* rp = ring2 + ((j * NC + m) * (T3Y / YO) + yseg) * T3X + col;
-        const float2 old = *rp;
-        S[0][m] += a[0] - old.x;
-        S[1][m] += a[1] - old.y;
-        *rp = make_float2(a[0], a[1]);
+        for (int i = 0; i < kYO; ++i)
+          if (i < nr) out[i * n.n2] = gradient(i, czn, wv[i], fv[i]);
       }
-      if (j == WW - 1) {
-#pragma unroll
-        for (int m = 0; m < NC; ++m) {
-          float t0[WW], t1[WW];
-#pragma unroll
-          for (int q = 0; q < WW; ++q) {
-            const float2 r = ring2[((q * NC + m) * (T3Y / YO) + yseg) * T3X + col];
-            t0[q] = r.x;
-            t1[q] = r.y;
-          }
-          S[0][m] = TreeSum<WW>::of(t0);
-          S[1][m] = TreeSum<WW>::of(t1);
-        }
-      }
-      if (outp) {
-        const int czn = max(0, min(pz, mz) - max(0, pz - 2 * R) + 1);
-#pragma unroll
-        for (int i = 0; i < YO; ++i) {
-          const int py = y0 + YO * yseg + i;
-          if (px >= n.n2 || py >= n.n1) continue;
-          const int o = pz * plane + py * n.n2 + px;
-          const float wv = wv_c[i], fv = fv_c[i];
-          float g;
-          if (KIND == 0)
-            g = scale * (cnt_xy[i] * (float)czn * wv - fv * S[i][0] - S[i][1]);
-          else
-            g = scale * (wv * S[i][0] - fv * S[i][1] - S[i][2]);
-          out[o] = g;
-        }
-      }
-      j = (j + 1 == WW) ? 0 : j + 1;
-    }
-    // the W pass of this plane is done with its stage (refilled below) and the H pass of
-    // the previous plane with its sx buffer (rewritten by the next W pass)
-    __syncthreads();
-    if (tid == 0 && it + 2 < niter) {
-      fence_proxy_async();
-      issue(it + 2);
-    }
-  }
-  if (!ok) {
-    // report, then give the copies still in flight into this CTA's stages one more bounded
-    // wait (the last use of each stage) before the CTA's shared memory is released
-    if (err) atomicOr(err, 1);
-    for (int st = 0; st < 2 && st < niter; ++st) {
-      const int last = niter - 1 - ((niter - 1 - st) & 1);  // last iteration that used stage st
-      mbar_wait(&bar[st], (unsigned)(last >> 1) & 1u);
+      W_p += plane, F_p += plane, out += plane;
     }
   }
 }
@@ -955,77 +766,38 @@ template <typename Kern>
 cudaError_t set_smem(Kern k, size_t bytes) {
   return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
-
-template <int R>
-constexpr size_t fwd3_bytes() {
-  return sizeof(float) * (Geo3<R, 3>::in_floats(2) + Geo3<R, 3>::sx_floats() + Geo3<R, 3>::ring_floats());
-}
-template <int R, int KIND>
-constexpr size_t bwd3_bytes() {
-  return sizeof(float) * (Geo3<R, KIND == 0 ? 2 : 3>::in_floats(KIND == 0 ? 2 : 3) +
-                          Geo3<R, KIND == 0 ? 2 : 3>::sx_floats() + Geo3<R, KIND == 0 ? 2 : 3>::ring_floats());
-}
-template <int R>
-constexpr size_t fwd3t_bytes() {
-  return 128 + sizeof(float) * (4 * stage_floats<R, 3>() + 2 * Geo3<R, 3>::sx_floats() + Geo3<R, 3>::ring_floats());
-}
-template <int R, int KIND>
-constexpr size_t bwd3t_bytes() {
-  return 128 + sizeof(float) * (2 * (KIND == 0 ? 2 : 3) * stage_floats<R, KIND == 0 ? 2 : 3>() +
-                                2 * Geo3<R, KIND == 0 ? 2 : 3>::sx_floats() + Geo3<R, KIND == 0 ? 2 : 3>::ring_floats());
-}
-template <int R, int KIND>
-void fwd3(dim3 g, const PairDesc* pd, const float* W, size_t Ws, float* coef, size_t cs, double* part, Dims n,
-          float eps, int tz, int nzc, cudaStream_t s) {
-  k_sim_fwd3<R, KIND><<<g, NT3, fwd3_bytes<R>(), s>>>(pd, W, Ws, coef, cs, part, n, eps, tz, nzc);
-}
-template <int R, int KIND>
-void bwd3(dim3 g, const PairDesc* pd, const float* W, size_t Ws, const float* coef, size_t cs, float* dLdW, Dims n,
-          float scale, int tz, int nzc, cudaStream_t s) {
-  k_sim_bwd3<R, KIND><<<g, NT3, bwd3_bytes<R, KIND>(), s>>>(pd, W, Ws, coef, cs, dLdW, n, scale, tz, nzc);
+template <int R, int KIND, bool TMA>
+cudaError_t prepare_one() {
+  constexpr int NC = KIND == 0 ? 2 : 3;
+  const cudaError_t a = set_smem(k_sim_fwd<R, KIND, TMA>, Box<R>::bytes(2, NC)),
+                    b = set_smem(k_sim_bwd<R, KIND, TMA>, Box<R>::bytes(NC, NC));
+  return a != cudaSuccess ? a : b;
 }
 template <int R>
 cudaError_t prepare_r() {
-  const cudaError_t e[8] = {set_smem(k_sim_fwd3<R, 0>, fwd3_bytes<R>()),   set_smem(k_sim_fwd3<R, 1>, fwd3_bytes<R>()),
-                            set_smem(k_sim_bwd3<R, 0>, bwd3_bytes<R, 0>()), set_smem(k_sim_bwd3<R, 1>, bwd3_bytes<R, 1>()),
-                            set_smem(k_sim_fwd3t<R, 0>, fwd3t_bytes<R>()), set_smem(k_sim_fwd3t<R, 1>, fwd3t_bytes<R>()),
-                            set_smem(k_sim_bwd3t<R, 0>, bwd3t_bytes<R, 0>()),
-                            set_smem(k_sim_bwd3t<R, 1>, bwd3t_bytes<R, 1>())};
+  const cudaError_t e[4] = {prepare_one<R, 0, false>(), prepare_one<R, 0, true>(), prepare_one<R, 1, false>(),
+                            prepare_one<R, 1, true>()};
   for (cudaError_t x : e)
     if (x != cudaSuccess) return x;
   return cudaSuccess;
 }
-template <int R, int KIND>
-void fwd3t(dim3 g, const SimMaps& m, const PairDesc* pd, const float* W, size_t Ws, float* coef, size_t cs,
-           double* part, Dims n, float eps, int tz, int nzc, int* err, cudaStream_t s) {
-  k_sim_fwd3t<R, KIND><<<g, NT3, fwd3t_bytes<R>(), s>>>(m, pd, W, Ws, coef, cs, part, n, eps, tz, nzc, err);
-}
-template <int R, int KIND>
-void bwd3t(dim3 g, const SimMaps& m, const PairDesc* pd, const float* W, size_t Ws, float* dLdW, Dims n,
-           float scale, int tz, int nzc, int* err, cudaStream_t s) {
-  k_sim_bwd3t<R, KIND><<<g, NT3, bwd3t_bytes<R, KIND>(), s>>>(m, pd, W, Ws, dLdW, n, scale, tz, nzc, err);
-}
-template <int KIND>
-void fwd_dispatch_t(int R, dim3 g, const SimMaps& m, const PairDesc* pd, const float* W, size_t Ws, float* coef,
-                    size_t cs, double* part, Dims n, float eps, int tz, int nzc, int* err, cudaStream_t s) {
+
+// f(radius, kind, tma) with the three as compile-time constants
+template <class Fn>
+void dispatch(int R, int kind, bool tma, Fn f) {
+  auto with_r = [&](auto r) {
+    using std::integral_constant;
+    if (kind == 0)
+      tma ? f(r, integral_constant<int, 0>{}, std::true_type{}) : f(r, integral_constant<int, 0>{}, std::false_type{});
+    else
+      tma ? f(r, integral_constant<int, 1>{}, std::true_type{}) : f(r, integral_constant<int, 1>{}, std::false_type{});
+  };
   switch (R) {
-    case 1: fwd3t<1, KIND>(g, m, pd, W, Ws, coef, cs, part, n, eps, tz, nzc, err, s); break;
-    case 2: fwd3t<2, KIND>(g, m, pd, W, Ws, coef, cs, part, n, eps, tz, nzc, err, s); break;
-    case 3: fwd3t<3, KIND>(g, m, pd, W, Ws, coef, cs, part, n, eps, tz, nzc, err, s); break;
-    case 4: fwd3t<4, KIND>(g, m, pd, W, Ws, coef, cs, part, n, eps, tz, nzc, err, s); break;
-    case 5: fwd3t<5, KIND>(g, m, pd, W, Ws, coef, cs, part, n, eps, tz, nzc, err, s); break;
-    default: break;
-  }
-}
-template <int KIND>
-void bwd_dispatch_t(int R, dim3 g, const SimMaps& m, const PairDesc* pd, const float* W, size_t Ws, float* dLdW,
-                    Dims n, float scale, int tz, int nzc, int* err, cudaStream_t s) {
-  switch (R) {
-    case 1: bwd3t<1, KIND>(g, m, pd, W, Ws, dLdW, n, scale, tz, nzc, err, s); break;
-    case 2: bwd3t<2, KIND>(g, m, pd, W, Ws, dLdW, n, scale, tz, nzc, err, s); break;
-    case 3: bwd3t<3, KIND>(g, m, pd, W, Ws, dLdW, n, scale, tz, nzc, err, s); break;
-    case 4: bwd3t<4, KIND>(g, m, pd, W, Ws, dLdW, n, scale, tz, nzc, err, s); break;
-    case 5: bwd3t<5, KIND>(g, m, pd, W, Ws, dLdW, n, scale, tz, nzc, err, s); break;
+    case 1: with_r(std::integral_constant<int, 1>{}); break;
+    case 2: with_r(std::integral_constant<int, 2>{}); break;
+    case 3: with_r(std::integral_constant<int, 3>{}); break;
+    case 4: with_r(std::integral_constant<int, 4>{}); break;
+    case 5: with_r(std::integral_constant<int, 5>{}); break;
     default: break;
   }
 }
@@ -1067,45 +839,21 @@ bool encode_volumes(CUtensorMap* m, const float* base, Dims n, int n_vol, int bo
 }
 
 namespace {
-int staged_row(int R) {  // RXS of Geo3<R, *>
+int staged_row(int R) {  // row pitch of the staged planes, Box<R>::PX
   switch (R) {
-    case 1: return Geo3<1, 2>::RXS;
-    case 2: return Geo3<2, 2>::RXS;
-    case 3: return Geo3<3, 2>::RXS;
-    case 4: return Geo3<4, 2>::RXS;
-    case 5: return Geo3<5, 2>::RXS;
+    case 1: return Box<1>::PX;
+    case 2: return Box<2>::PX;
+    case 3: return Box<3>::PX;
+    case 4: return Box<4>::PX;
+    case 5: return Box<5>::PX;
     default: return 0;
-  }
-}
-
-template <int KIND>
-void fwd_dispatch(int R, dim3 g, const PairDesc* pd, const float* W, size_t Ws, float* coef, size_t cs, double* part,
-                  Dims n, float eps, int tz, int nzc, cudaStream_t s) {
-  switch (R) {
-    case 1: fwd3<1, KIND>(g, pd, W, Ws, coef, cs, part, n, eps, tz, nzc, s); break;
-    case 2: fwd3<2, KIND>(g, pd, W, Ws, coef, cs, part, n, eps, tz, nzc, s); break;
-    case 3: fwd3<3, KIND>(g, pd, W, Ws, coef, cs, part, n, eps, tz, nzc, s); break;
-    case 4: fwd3<4, KIND>(g, pd, W, Ws, coef, cs, part, n, eps, tz, nzc, s); break;
-    case 5: fwd3<5, KIND>(g, pd, W, Ws, coef, cs, part, n, eps, tz, nzc, s); break;
-    default: break;
-  }
-}
-template <int KIND>
-void bwd_dispatch(int R, dim3 g, const PairDesc* pd, const float* W, size_t Ws, const float* coef, size_t cs,
-                  float* dLdW, Dims n, float scale, int tz, int nzc, cudaStream_t s) {
-  switch (R) {
-    case 1: bwd3<1, KIND>(g, pd, W, Ws, coef, cs, dLdW, n, scale, tz, nzc, s); break;
-    case 2: bwd3<2, KIND>(g, pd, W, Ws, coef, cs, dLdW, n, scale, tz, nzc, s); break;
-    case 3: bwd3<3, KIND>(g, pd, W, Ws, coef, cs, dLdW, n, scale, tz, nzc, s); break;
-    case 4: bwd3<4, KIND>(g, pd, W, Ws, coef, cs, dLdW, n, scale, tz, nzc, s); break;
-    case 5: bwd3<5, KIND>(g, pd, W, Ws, coef, cs, dLdW, n, scale, tz, nzc, s); break;
-    default: break;
   }
 }
 
 // D chunk of one CTA: every chunk streams 2R planes more than it covers, so D is split only
 // while one pair has fewer than 16384 threads and the launch (batch pairs) fewer than 1824
-// CTAs (four waves of three CTAs on each of 152 SMs), and halved only while above min_chunk planes
+// CTAs (four waves of three CTAs on each of 152 SMs), and halved only while above min_chunk planes.
+// The chunks are where the D sums restart, so this rule is part of the results.
 int chunk_for(int ntiles, int depth, int min_chunk, int threads, int batch) {
   int tz = depth;
   for (;;) {
@@ -1116,19 +864,18 @@ int chunk_for(int ntiles, int depth, int min_chunk, int threads, int batch) {
   return tz < 1 ? 1 : tz;
 }
 
-dim3 sim_grid(Dims ni, int window, int n_pairs, int batch, SimGeom* geo) {
-  (void)window;
-  const int gx = (ni.n2 + T3X - 1) / T3X, gy = (ni.n1 + T3Y - 1) / T3Y;
-  SimGeom g;
-  g.tz = chunk_for(gx * gy, ni.n0, 8, NT3, batch);
+Tiles sim_tiles(Dims ni, int n_pairs, int batch, int group) {
+  Tiles g;
+  g.np = n_pairs;
+  g.grp = std::max(1, std::min(group, n_pairs));
+  g.gx = (ni.n2 + kTX - 1) / kTX;
+  g.gy = (ni.n1 + kTY - 1) / kTY;
+  g.tz = chunk_for(g.gx * g.gy, ni.n0, 8, 256, batch);
   g.nzc = (ni.n0 + g.tz - 1) / g.tz;
-  g.ctas = gx * gy * g.nzc;
-  if (geo) *geo = g;
-  return dim3(gx, gy, g.nzc * n_pairs);
+  return g;
 }
-}  // namespace
+unsigned ctas(const Tiles& g) { return (unsigned)g.gx * g.gy * g.nzc * g.np; }
 
-namespace {
 template <int KIND>
 void fixed_stats(dim3 g, const float* imgs, Dims ni, int window, float eps, float* stats, int tz, int nzc,
                  cudaStream_t s) {
@@ -1167,57 +914,40 @@ cudaError_t prepare_kernels() {
 }
 
 SimGeom sim_geom(Dims ni, int window, int batch) {
-  SimGeom g;
-  sim_grid(ni, window, 1, batch, &g);
-  return g;
+  (void)window;
+  const Tiles g = sim_tiles(ni, 1, batch, 1);
+  return SimGeom{g.nzc, g.tz, (int)ctas(g)};
 }
 int sim_ncoef(int kind) { return kind == 0 ? 2 : 3; }
 
 void make_sim_maps(SimMaps* m, const float* W, int n_pairs, const float* imgs, int n_images, const float* coef,
                    Dims ni, int window, int kind) {
   memset(m, 0, sizeof(*m));
-  const int R = window / 2, rxs = staged_row(R), ry = T3Y + 2 * R;
-  if (!rxs) return;
+  const int R = window / 2, px = staged_row(R), ry = kTY + 2 * R;
+  if (!px) return;
   m->fwd_ok =
-      encode_volumes(&m->W, W, ni, n_pairs, rxs, ry, 1) && encode_volumes(&m->F, imgs, ni, n_images, rxs, ry, 1);
-  m->bwd_ok = encode_volumes(&m->C, coef, ni, n_pairs * sim_ncoef(kind), rxs, ry, 1);
+      encode_volumes(&m->W, W, ni, n_pairs, px, ry, 1) && encode_volumes(&m->F, imgs, ni, n_images, px, ry, 1);
+  m->bwd_ok = encode_volumes(&m->C, coef, ni, n_pairs * sim_ncoef(kind), px, ry, 1);
 }
 
-void launch_sim_fwd(const PairDesc* pd, int n_pairs, int batch, const float* W, size_t Wstride, float* coef,
+void launch_sim_fwd(const PairDesc* pd, int n_pairs, int batch, int group, const float* W, size_t Wstride, float* coef,
                     size_t cs, double* partials, Dims ni, int window, int kind, float eps, const SimMaps* maps,
                     int* err, cudaStream_t s) {
-  SimGeom g;
-  const dim3 grid = sim_grid(ni, window, n_pairs, batch, &g);
-  const int R = window / 2;
-  if (maps && maps->fwd_ok) {
-    if (kind == 0)
-      fwd_dispatch_t<0>(R, grid, *maps, pd, W, Wstride, coef, cs, partials, ni, eps, g.tz, g.nzc, err, s);
-    else
-      fwd_dispatch_t<1>(R, grid, *maps, pd, W, Wstride, coef, cs, partials, ni, eps, g.tz, g.nzc, err, s);
-    return;
-  }
-  if (kind == 0)
-    fwd_dispatch<0>(R, grid, pd, W, Wstride, coef, cs, partials, ni, eps, g.tz, g.nzc, s);
-  else
-    fwd_dispatch<1>(R, grid, pd, W, Wstride, coef, cs, partials, ni, eps, g.tz, g.nzc, s);
+  const Tiles g = sim_tiles(ni, n_pairs, batch, group);
+  dispatch(window / 2, kind, maps && maps->fwd_ok, [&](auto r, auto k, auto t) {
+    k_sim_fwd<r(), k(), t()><<<ctas(g), Box<r()>::NT, Box<r()>::bytes(2, k() == 0 ? 2 : 3), s>>>(
+        maps ? *maps : SimMaps{}, pd, W, Wstride, coef, cs, partials, ni, g, eps, err);
+  });
 }
-void launch_sim_bwd(const PairDesc* pd, int n_pairs, int batch, const float* W, size_t Wstride, const float* coef,
-                    size_t cs, float* dLdW, Dims ni, int window, int kind, float scale, const SimMaps* maps, int* err,
-                    cudaStream_t s) {
-  SimGeom g;
-  const dim3 grid = sim_grid(ni, window, n_pairs, batch, &g);
-  const int R = window / 2;
-  if (maps && maps->bwd_ok) {
-    if (kind == 0)
-      bwd_dispatch_t<0>(R, grid, *maps, pd, W, Wstride, dLdW, ni, scale, g.tz, g.nzc, err, s);
-    else
-      bwd_dispatch_t<1>(R, grid, *maps, pd, W, Wstride, dLdW, ni, scale, g.tz, g.nzc, err, s);
-    return;
-  }
-  if (kind == 0)
-    bwd_dispatch<0>(R, grid, pd, W, Wstride, coef, cs, dLdW, ni, scale, g.tz, g.nzc, s);
-  else
-    bwd_dispatch<1>(R, grid, pd, W, Wstride, coef, cs, dLdW, ni, scale, g.tz, g.nzc, s);
+void launch_sim_bwd(const PairDesc* pd, int n_pairs, int batch, int group, const float* W, size_t Wstride,
+                    const float* coef, size_t cs, float* dLdW, Dims ni, int window, int kind, float scale,
+                    const SimMaps* maps, int* err, cudaStream_t s) {
+  const Tiles g = sim_tiles(ni, n_pairs, batch, group);
+  dispatch(window / 2, kind, maps && maps->bwd_ok, [&](auto r, auto k, auto t) {
+    constexpr int nc = k() == 0 ? 2 : 3;
+    k_sim_bwd<r(), k(), t()><<<ctas(g), Box<r()>::NT, Box<r()>::bytes(nc, nc), s>>>(
+        maps ? *maps : SimMaps{}, pd, W, Wstride, coef, cs, dLdW, ni, g, scale, err);
+  });
 }
 
 }  // namespace muster
