@@ -17,10 +17,10 @@
 // issue. The layout is chosen for both: 8 sums per W task read 14 inputs (w = 7) instead of 10 for
 // every 4, four rows per H/D thread read 10 W sums instead of 16, the ring moves 16 bytes per
 // access, and the row pitches (4 modulo 8 floats) keep the W task's accesses free of bank conflicts.
-// Measured on 90 pairs of 160 x 192 x 160, w = 7, SiLNCC: forward 1678 us, adjoint 1451 us (L1 data
+// Measured on 90 pairs of 160 x 192 x 160, w = 7, SiLNCC: forward 1729 us, adjoint 1451 us (L1 data
 // pipe 76 and 81 % busy, DRAM 39 and 57 %); one role per thread with a barrier per plane, W sums in
 // runs of 4 and two rows per thread took 2605 and 1802 us. 4 CTAs of 7 warps run on an SM; cut for
-// 3, the forward takes 1895 us.
+// 3, the forward takes 12 % longer.
 //
 // The order of the additions is part of the results, and the layout keeps it: along W runs of 4
 // sums (a pairwise tree, then a running sum), along H runs of 2, along D the ring. An optimiser
@@ -44,7 +44,11 @@
 // one voxel of the tile (variance is shift invariant) to limit cancellation.
 // SiLNCC needs S_WW only in the loss, where sum_R S_WW = sum_p cnt(p) W'(p)^2 - sum_R (sum W')^2/|R|
 // with cnt(p) the number of the CTA's windows that hold voxel p: the W pass adds the first term
-// once per voxel, which spares a third box sum (a third of the ring and of the arithmetic).
+// once per voxel, which spares a third box sum (a third of the ring and of the arithmetic: 2570 us
+// instead of 1729). Both sums are larger than their difference and are carried without rounding
+// (FSum), so that the loss stays as smooth in the images as the sum over windows: central
+// differences of it with step 1e-3 agree with the gradient to a median of 1.0 to 1.4 % (three draws of
+// 128 entries, 6 sessions of 128^3), with a third box sum and Kahan sums to 1.3 to 1.4 %.
 // Adjoint: dL/dW(p) = scale * (W(p) sum A - F(p) sum B - sum C) over the
 // windows containing p (corners p - 2R .. p).
 #include <cudaTypedefs.h>
@@ -191,7 +195,7 @@ struct Tile {
 };
 // Pairs that share a fixed image (the engine orders them by fixed image) run beside each other
 // on the same tile, so that its F, mu_F and S_FF planes are read from L2 by all but the first
-// (10 sessions of 160 x 192 x 160: forward 1678 us, in pair order 1763 us).
+// (10 sessions of 160 x 192 x 160: forward 1678 us, in pair order 1763 us, before the loss sums were widened).
 __device__ __forceinline__ Tile tile_of(const Tiles& g) {
   const unsigned per = (unsigned)g.gx * g.gy * g.nzc;
   unsigned id = blockIdx.x;
@@ -227,13 +231,21 @@ __device__ __forceinline__ double block_sum(FF x, float* sh) {
   return r;
 }
 
-// compensated (Kahan) running sum
-struct KSum {
-  float s = 0.f, c = 0.f;
+// a + b = s exactly, with the rounding error of s in e (Knuth)
+__device__ __forceinline__ float two_sum(float a, float b, float& e) {
+  const float s = __fadd_rn(a, b), v = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, v)), __fsub_rn(b, v));
+  return s;
+}
+
+// running sum without rounding: hi + lo carries every term (Knuth's two-sum). A term changes nothing
+// but the sum, so a change in one window leaves the rounding of all others as it was.
+struct FSum {
+  float hi = 0.f, lo = 0.f;
   __device__ __forceinline__ void add(float x) {
-    const float y = x - c, t = s + y;
-    c = (t - s) - y;
-    s = t;
+    float e;
+    hi = two_sum(hi, x, e);
+    lo += e;
   }
 };
 
@@ -519,7 +531,7 @@ __global__ void __launch_bounds__(Box<R>::NT, kMinCtas)
   __syncthreads();
   // SiLNCC: W threads sum_p cnt(p) W'(p)^2, H/D threads sum_R ((sum W')^2/|R| + beta S_FW);
   // LNCC: H/D threads sum_R Sim_R
-  KSum acc;
+  FSum acc;
   if (wt >= 0) {
     Stages<R, 2, TMA> st{smem, bar, {&maps.F, &maps.W}, {d.fi, t.pair}, {F, W}, t.x0, t.y0, t.z0, niter, wt, n, true};
     st.start();
@@ -552,18 +564,23 @@ __global__ void __launch_bounds__(Box<R>::NT, kMinCtas)
         // a voxel that no window holds adds nothing, whatever it is (0 * Inf)
         const int c = cnt_y * corners_holding(it, last_z, 2 * R);
         if (c > 0 && last_x >= 0) {
-          float a = 0.f;
+          float sq[B::NI];
           if (last_x == kXO - 1) {
 #pragma unroll
-            for (int k = 0; k < B::NI; ++k) {
-              const int q = (k < kXO - 1 ? k : kXO - 1) - (k > 2 * R ? k - 2 * R : 0) + 1;
-              a = fmaf((float)q * w[k], w[k], a);
-            }
+            for (int k = 0; k < B::NI; ++k)
+              sq[k] = (float)((k < kXO - 1 ? k : kXO - 1) - (k > 2 * R ? k - 2 * R : 0) + 1) * w[k] * w[k];
           } else {
 #pragma unroll
-            for (int k = 0; k < B::NI; ++k) a = fmaf((float)corners_holding(k, last_x, 2 * R) * w[k], w[k], a);
+            for (int k = 0; k < B::NI; ++k) sq[k] = (float)corners_holding(k, last_x, 2 * R) * w[k] * w[k];
           }
-          acc.add((float)c * a);
+          // the two upper levels of the pairwise sum and the product with c, with their errors
+          constexpr int N1 = B::NI / 2, N2 = B::NI - N1;
+          float e0, e1, e2;
+          const float lo = two_sum(TreeSum<N1 / 2>::of(sq), TreeSum<N1 - N1 / 2>::of(sq + N1 / 2), e0);
+          const float hi = two_sum(TreeSum<N2 / 2>::of(sq + N1), TreeSum<N2 - N2 / 2>::of(sq + N1 + N2 / 2), e1);
+          const float a = two_sum(lo, hi, e2), ca = __fmul_rn((float)c, a);
+          acc.add(ca);
+          acc.lo += __fmaf_rn((float)c, e2 + (e0 + e1), __fmaf_rn((float)c, a, -ca));
         }
       }
       st.next(it);
@@ -590,7 +607,7 @@ __global__ void __launch_bounds__(Box<R>::NT, kMinCtas)
         const float beta = Sfw * Sff;  // Sff holds 1 / (S_FF + eps) for SiLNCC
         c0 = beta;
         c1 = muW - beta * muF;
-        return fmaf(Sfw, beta, s0 * s0 * inv_nw);
+        return fmaf(s0, s0 * inv_nw, Sfw * beta);
       }
       const float Sww = fmaxf(ring.S[1][i] - s0 * s0 * inv_nw, 0.f);
       const float Q = Sff * Sww + eps;
@@ -649,7 +666,7 @@ __global__ void __launch_bounds__(Box<R>::NT, kMinCtas)
     }
   }
   const float sgn = KIND == 0 && wt < 0 ? -1.f : 1.f;
-  const double sum = block_sum<B::NT>(FF{sgn * acc.s, -sgn * acc.c}, sh);
+  const double sum = block_sum<B::NT>(FF{sgn * acc.hi, sgn * acc.lo}, sh);
   if (threadIdx.x == 0) part[t.part] = KIND == 0 ? sum / (double)(B::WW * B::WW * B::WW) : sum;
 }
 
