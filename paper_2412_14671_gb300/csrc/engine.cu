@@ -104,6 +104,7 @@ struct muster_ctx {
   std::string err;
   std::vector<Dims> ni, nf;
   std::vector<float*> imgs;
+  std::vector<float2*> cells;  // per level: the cells of every image (moving images of the warp)
   std::vector<float*> fstats;  // per level: window statistics (mu_F, S_FF or 1/(S_FF+eps)) of every session
   std::vector<double> times;
   bool have_images = false;
@@ -405,7 +406,7 @@ int build_all_tables(muster_ctx* ctx) {
       for (int k = 0; k < N; ++k) {
         if (k == i) continue;
         PairDesc d;
-        d.Ik = im + (size_t)k * Vi;
+        d.Ic = ctx->cells[l] + (size_t)k * image_cells(ctx->ni[l]);
         d.Ii = im + (size_t)i * Vi;
         d.Fs = ctx->fstats[l] + (size_t)i * 2 * Vi;
         d.fi = i;
@@ -967,7 +968,9 @@ int create_impl(const int64_t shape[3], int n_sessions, const double spacing[3],
   const int L = ctx->L;
   ctx->imgs.resize(L);
   ctx->fstats.resize(L);
+  ctx->cells.resize(L);
   for (int l = 0; l < L; ++l) {
+    ctx->cells[l] = (float2*)A(sizeof(float2) * ctx->N * image_cells(ctx->ni[l]));
     ctx->imgs[l] = (float*)A(sizeof(float) * ctx->N * nvox(ctx->ni[l]));
     ctx->fstats[l] = (float*)A(sizeof(float) * 2 * ctx->N * nvox(ctx->ni[l]));
   }
@@ -1146,6 +1149,7 @@ int muster_set_images(muster_ctx* ctx, const float* imgs, int on_device, const d
     Scope s(ctx, KK_DOWN2, (double)N * (nvox(ctx->ni[l + 1]) + nvox(ctx->ni[l])) * 4.0);
     launch_down2(ctx->imgs[l + 1], ctx->ni[l + 1], ctx->imgs[l], ctx->ni[l], N, ctx->stream);
   }
+  for (int l = 0; l < L; ++l) launch_image_cells(ctx->imgs[l], N, ctx->ni[l], ctx->cells[l], ctx->stream);
   // window statistics of every session as a fixed image, per level (images do not change)
   for (int l = 0; l < L; ++l) launch_fixed_stats(ctx->imgs[l], N, ctx->ni[l], ctx->p.window, ctx->p.similarity, ctx->p.sim_eps,
                                             ctx->fstats[l], ctx->stream);

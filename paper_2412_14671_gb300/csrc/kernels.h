@@ -46,7 +46,7 @@ struct PairGradTab {
   int slot_pair[kMaxDescPerLaunch];
 };
 struct PairDesc {   // ordered pair (k -> i): pulls image k onto grid i
-  const float* Ik;  // moving image (level grid)
+  const float2* Ic; // cells of the moving image (launch_image_cells)
   const float* Ii;  // fixed image
   const float* Fs;  // window statistics of the fixed image: mu_F then S_FF planes
   const float4* U;  // pair displacement on the flow grid
@@ -129,6 +129,9 @@ void launch_planar_to_f4(const float* in, float4* out, int n_fields, size_t V, c
 
 // ---- image-grid kernels (image_kernels.cu) ----
 void launch_down2(const float* in, Dims n, float* out, Dims m, int n_images, cudaStream_t s);
+// images as cells along W with a replicated border, as the forward warp samples them (warp_kernels.cu)
+size_t image_cells(Dims n);
+void launch_image_cells(const float* in, int n_images, Dims n, float2* out, cudaStream_t s);
 // warp_kernels.cu; both require nf = ceil(ni / 2) per axis
 // W: n_pairs volumes at stride Wstride; gI (nullable): grad I_k at the sample points, 3 planes per pair
 void launch_warp(const PairDesc* pd, int n_pairs, Dims ni, Dims nf, float* W, float* gI, size_t Wstride,
