@@ -65,17 +65,30 @@ __global__ void k_rigid_table(const float* __restrict__ rho, float* __restrict__
   if (i < a.N) table_row(rho, i, a, tab + 12 * i);
 }
 
-// one thread per session i >= 1: pairs (k -> i) are i*(N-1) + r, r = 0..N-2
-__global__ void k_rigid_grad(const float* __restrict__ rpart, const float* __restrict__ rho,
-                             float* __restrict__ grad, RigidArgs a) {
-  const int i = threadIdx.x + 1;
-  if (i >= a.N) return;
-  double S[12] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-  for (int r = 0; r < a.N - 1; ++r) {
-    const float* p = rpart + ((size_t)(i * (a.N - 1) + r) * a.per_pair) * 12;
-    for (int c = 0; c < a.per_pair; ++c)
-      for (int e = 0; e < 12; ++e) S[e] += (double)p[(size_t)c * 12 + e];
+// one CTA per session i >= 1. Its pairs are i*(N-1) .. i*(N-1) + N-2, so their CTA sums are one array of
+// rows of 12: thread (e, l) adds entry e of rows l, l + 32, ... in double, and the 32 partial sums of
+// an entry are added in order. One thread per session took 639 us for 30 pairs of 128^3 (a serial
+// chain of 12 loads per row), this takes 19 us.
+constexpr int kRigidLanes = 32;
+__global__ void __launch_bounds__(12 * kRigidLanes) k_rigid_grad(const float* __restrict__ rpart,
+                                                                 const float* __restrict__ rho, float* __restrict__ grad,
+                                                                 RigidArgs a) {
+  __shared__ double sh[kRigidLanes][12];
+  __shared__ double S[12];
+  const int i = blockIdx.x + 1, e = threadIdx.x % 12, l = threadIdx.x / 12;
+  const size_t rows = (size_t)(a.N - 1) * a.per_pair;
+  const float* p = rpart + (size_t)i * rows * 12;
+  double sum = 0.0;
+  for (size_t r = l; r < rows; r += kRigidLanes) sum += (double)p[r * 12 + e];
+  sh[l][e] = sum;
+  __syncthreads();
+  if (l == 0) {
+    double t = 0.0;
+    for (int k = 0; k < kRigidLanes; ++k) t += sh[k][e];
+    S[e] = t;
   }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
   double R[9], dR[27];
   rotation(rho + 6 * (i - 1), R, dR);
   const double c[3] = {a.c0, a.c1, a.c2};
@@ -127,7 +140,7 @@ void launch_rigid_table(const float* rho, float* tab, const RigidArgs& a, cudaSt
   k_rigid_table<<<1, 32, 0, s>>>(rho, tab, a);
 }
 void launch_rigid_grad(const float* rpart, const float* rho, float* grad, const RigidArgs& a, cudaStream_t s) {
-  k_rigid_grad<<<1, 32, 0, s>>>(rpart, rho, grad, a);
+  k_rigid_grad<<<a.N - 1, 12 * kRigidLanes, 0, s>>>(rpart, rho, grad, a);
 }
 void launch_rigid_step(float* rho, float* m, float* v, const float* grad, const float* sched, const int* step,
                        float* tab, const RigidArgs& a, cudaStream_t s) {
