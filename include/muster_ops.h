@@ -9,6 +9,11 @@
  * legacy default stream). Functions returning host values synchronise `stream`.
  * Return value: MUSTER_OK or a negative MUSTER_E* code of muster.h; the message
  * is muster_ops_last_error() (per thread).
+ *
+ * Scratch comes from a memory pool of the library on the current device and is released in
+ * the order of `stream`. The pool keeps up to 256 MiB of unused scratch between calls (so that
+ * a call does not map memory anew) and gives it back when a device allocation of the
+ * library fails; while `stream` is being captured, the graph owns the scratch instead.
  */
 #ifndef MUSTER_OPS_H
 #define MUSTER_OPS_H
@@ -30,7 +35,7 @@ int muster_op_downsample(const float* in, int n_images, int64_t D, int64_t H, in
 /* Exp of Alg. 1 in the displacement form of its comment: u = Exp(sign * phi) - identity
    after K squarings u <- u + u o (x + u) from u = sign * phi / 2^K, trilinear
    sampling with clamp-to-edge. phi, u: (3, D, H, W); sign is +1 or -1.
-   Allocates and frees device scratch of 20 * D*H*W floats on `stream`. */
+   Takes device scratch of 8 * D*H*W floats. */
 int muster_op_exp(const float* phi, int64_t D, int64_t H, int64_t W, int K, float sign,
                   float* u, void* stream);
 
@@ -38,7 +43,7 @@ int muster_op_exp(const float* phi, int64_t D, int64_t H, int64_t W, int K, floa
    w^3 windows of SiLNCC_R (kind MUSTER_SILNCC) or LNCC_R (MUSTER_LNCC) between
    fixed F and moving W, and (dLdW, nullable) its gradient with respect to W.
    loss: host double. eps: the guard of muster_params.sim_eps. Returns 0 loss and
-   a zero gradient when no window fits. Allocates and frees device scratch of
+   a zero gradient when no window fits. Takes device scratch of
    about 5 * D*H*W floats on `stream`. */
 int muster_op_similarity(const float* F, const float* W, int64_t D, int64_t H, int64_t Wd,
                          int window, int kind, float eps, double* loss, float* dLdW,
@@ -86,7 +91,7 @@ int muster_op_jacobian_det(const float* u, int64_t D, int64_t H, int64_t W, floa
    each thread's running sums are double-float values (a pair of floats, about 48
    significant bits); the per-CTA and final sums are FP64 in a fixed order over a grid of
    three CTAs per SM (at most 768), so a device gives the same result on every run.
-   Allocates and frees about 150 KB of device scratch on `stream`; synchronises it. */
+   Takes about 150 KB of device scratch; synchronises `stream`. */
 int muster_op_deformation_metrics(const float* u_true, const float* u_est, const uint8_t* roi, int64_t D,
                                   int64_t H, int64_t W, double out[16], void* stream);
 

@@ -225,7 +225,11 @@ void* dalloc(muster_ctx* ctx, size_t bytes) {
     ptr = ctx->p.alloc(bytes, ctx->p.alloc_user);
   } else if (cudaMalloc(&ptr, bytes) != cudaSuccess) {
     cudaGetLastError();
-    ptr = nullptr;
+    trim_op_pools();
+    if (cudaMalloc(&ptr, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      ptr = nullptr;
+    }
   }
   if (ptr) ctx->allocs.push_back(ptr);
   return ptr;
@@ -550,7 +554,7 @@ int forward_adjoint(muster_ctx* ctx, int l, const float4* th) {
   const int F = ctx->F, P = ctx->P, K = ctx->p.n_squarings, NC = ctx->NC;
   forward_fields(ctx, l, th);
   const int64_t NR = count_NR(ni, ctx->p.window);
-  const SimGeom g = sim_geom(ni, ctx->p.window, ctx->Bc);
+  const SimGeom g = sim_geom(ni, ctx->p.window, ctx->Bc, ctx->p.similarity);
   const int det = ctx->p.deterministic;
   // det: the step's largest-gradient word was zeroed by the exp launch of forward_fields
   if (NR == 0) {
@@ -698,7 +702,7 @@ int forward_adjoint(muster_ctx* ctx, int l, const float4* th) {
 int reduce_loss(muster_ctx* ctx, int l, int advance) {
   const Dims ni = ctx->ni[l], nf = ctx->nf[l];
   const int64_t NR = count_NR(ni, ctx->p.window);
-  const SimGeom g = sim_geom(ni, ctx->p.window, ctx->Bc);
+  const SimGeom g = sim_geom(ni, ctx->p.window, ctx->Bc, ctx->p.similarity);
   const int nreg = reg_blocks(nf) * ctx->F;
   Scope s(ctx, KK_LOSS, 0.0);
   launch_loss_reduce(ctx->sim_part, g.ctas * ctx->P, ctx->reg_part, nreg, NR ? 1.0 / (double)NR : 0.0,
@@ -878,7 +882,7 @@ int create_impl(const int64_t shape[3], int n_sessions, const double spacing[3],
     ctx->sched_off[l] = hist_len;
     hist_len += params->steps_per_level[l];
     // batch 1 splits D the most: an upper bound for any pair batch
-    max_sim_part = std::max(max_sim_part, (size_t)sim_geom(d, params->window, 1).ctas * ctx->P);
+    max_sim_part = std::max(max_sim_part, (size_t)sim_geom(d, params->window, 1, params->similarity).ctas * ctx->P);
     max_reg = std::max(max_reg, (size_t)reg_blocks(ctx->nf[l]) * ctx->F);
   }
   ctx->hist_len = std::max(hist_len, 1);
@@ -898,7 +902,7 @@ int create_impl(const int64_t shape[3], int n_sessions, const double spacing[3],
   {
     int zmax = 1;
     for (int l = 0; l < ctx->L; ++l)
-      zmax = std::max({zmax, ctx->nf[l].n0, sim_geom(ctx->ni[l], params->window, 1).nzc,
+      zmax = std::max({zmax, ctx->nf[l].n0, sim_geom(ctx->ni[l], params->window, 1, params->similarity).nzc,
                        warp_bwd_zchunks(ctx->nf[l], 1)});
     ctx->B = std::max(1, std::min(ctx->B, 65535 / zmax));
   }
@@ -1151,7 +1155,7 @@ int muster_set_images(muster_ctx* ctx, const float* imgs, int on_device, const d
   }
   for (int l = 0; l < L; ++l) launch_image_cells(ctx->imgs[l], N, ctx->ni[l], ctx->cells[l], ctx->stream);
   // window statistics of every session as a fixed image, per level (images do not change)
-  for (int l = 0; l < L; ++l) launch_fixed_stats(ctx->imgs[l], N, ctx->ni[l], ctx->p.window, ctx->p.similarity, ctx->p.sim_eps,
+  for (int l = 0; l < L; ++l) launch_fixed_stats(ctx->imgs[l], N, 1, ctx->ni[l], ctx->p.window, ctx->p.similarity, ctx->p.sim_eps,
                                             ctx->fstats[l], ctx->stream);
   rc = check_launch(ctx, "pyramid");
   if (rc) return rc;

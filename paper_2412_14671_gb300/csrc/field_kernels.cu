@@ -73,6 +73,20 @@ __global__ void k_squaring(const float4* __restrict__ u, float4* __restrict__ un
   }
 }
 
+// one field, its squared map written planar (the end of a stateless exponential)
+__global__ void k_squaring_planar(const float4* __restrict__ u, float* __restrict__ un, Dims n) {
+  const int v = blockIdx.x * blockDim.x + threadIdx.x;
+  const int V = (int)vox(n);
+  if (v >= V) return;
+  int z, y, x;
+  unflat(n, v, z, y, x);
+  const float4 a = u[v];
+  const float4 s = f4add(a, sample4(u, n, z + a.x, y + a.y, x + a.z));
+  un[v] = s.x;
+  un[(size_t)V + v] = s.y;
+  un[2 * (size_t)V + v] = s.z;
+}
+
 // ---- Alg. 1, first line and first loop iteration in one launch: u_0 = sign phi / 2^K is
 // written (the adjoint reads it) and u_1 = u_0 + S[u_0](x + u_0(x)) is computed from phi.
 // sign / 2^K is a power of two, so scaling commutes with every rounding of the trilinear
@@ -553,11 +567,12 @@ __global__ void k_f4_to_planar(const float4* __restrict__ in, float* __restrict_
   out[(3 * f + 2) * V + v] = a.z;
 }
 
-__global__ void k_planar_to_f4(const float* __restrict__ in, float4* __restrict__ out, size_t V) {
+__global__ void k_planar_to_f4(const float* __restrict__ in, float4* __restrict__ out, size_t V, float scale) {
   const size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= V) return;
   const size_t f = blockIdx.y;
-  out[f * V + v] = make_float4(in[(3 * f + 0) * V + v], in[(3 * f + 1) * V + v], in[(3 * f + 2) * V + v], 0.f);
+  out[f * V + v] =
+      make_float4(scale * in[(3 * f + 0) * V + v], scale * in[(3 * f + 1) * V + v], scale * in[(3 * f + 2) * V + v], 0.f);
 }
 }  // namespace
 
@@ -579,6 +594,9 @@ void launch_squaring(const float4* u, float4* un, int n_fields2, Dims n, cudaStr
     k_squaring<1><<<g, kThreads, 0, s>>>(u, un, n, n_fields2);
   else
     k_squaring<2><<<g, kThreads, 0, s>>>(u, un, n, n_fields2);
+}
+void launch_squaring_planar(const float4* u, float* un, Dims n, cudaStream_t s) {
+  k_squaring_planar<<<blocks_for(vox(n)), kThreads, 0, s>>>(u, un, n);
 }
 void launch_squaring_first(const float4* theta, float4* u0, float4* u1, int n_fields, Dims n, float scale,
                            cudaStream_t s, int nf, unsigned* zero) {
@@ -696,8 +714,8 @@ void launch_adam(float4* theta, float4* m, float4* v, const float4* grad, size_t
 void launch_f4_to_planar(const float4* in, float* out, int n_fields, size_t V, cudaStream_t s) {
   k_f4_to_planar<<<dim3(blocks_for(V), n_fields), kThreads, 0, s>>>(in, out, V);
 }
-void launch_planar_to_f4(const float* in, float4* out, int n_fields, size_t V, cudaStream_t s) {
-  k_planar_to_f4<<<dim3(blocks_for(V), n_fields), kThreads, 0, s>>>(in, out, V);
+void launch_planar_to_f4(const float* in, float4* out, int n_fields, size_t V, cudaStream_t s, float scale) {
+  k_planar_to_f4<<<dim3(blocks_for(V), n_fields), kThreads, 0, s>>>(in, out, V, scale);
 }
 
 }  // namespace muster

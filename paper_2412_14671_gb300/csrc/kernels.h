@@ -100,6 +100,8 @@ void launch_exp_init(const float4* theta, float4* u0, int n_fields, Dims n, floa
 // nf: fields (or chains) per thread of the flow-grid gather kernels, 1 or 2 (launch
 // configuration only: the results are the same)
 void launch_squaring(const float4* u, float4* un, int n_fields2, Dims n, cudaStream_t s, int nf = 2);
+// the same for one field, written as a planar (3, D, H, W) displacement
+void launch_squaring_planar(const float4* u, float* un, Dims n, cudaStream_t s);
 // exp_init and the first squaring in one launch: u0 = +-scale theta (2 n_fields fields, the
 // second half negated) and u1 = its first squaring (scale a power of two)
 void launch_squaring_first(const float4* theta, float4* u0, float4* u1, int n_fields, Dims n, float scale,
@@ -125,7 +127,8 @@ void launch_adam(float4* theta, float4* m, float4* v, const float4* grad, size_t
                  const float* sched, const int* step, int sgd, float beta1, float beta2, float eps,
                  cudaStream_t s);
 void launch_f4_to_planar(const float4* in, float* out, int n_fields, size_t V, cudaStream_t s);
-void launch_planar_to_f4(const float* in, float4* out, int n_fields, size_t V, cudaStream_t s);
+// out = scale * in
+void launch_planar_to_f4(const float* in, float4* out, int n_fields, size_t V, cudaStream_t s, float scale = 1.f);
 
 // ---- image-grid kernels (image_kernels.cu) ----
 void launch_down2(const float* in, Dims n, float* out, Dims m, int n_images, cudaStream_t s);
@@ -146,15 +149,16 @@ struct SimGeom {
   int ctas;  // CTAs per pair
 };
 // batch: the most pairs one launch of the caller takes; it sets the D chunking (fewer,
-// longer chunks for larger batches), so every launch of a context must pass the same value
-SimGeom sim_geom(Dims ni, int window, int batch);  // sim_kernels.cu
+// longer chunks for larger batches), so every launch of a context must pass the same value;
+// 0 for a stateless call, whose one pair should fill the device
+SimGeom sim_geom(Dims ni, int window, int batch, int kind = 0);  // sim_kernels.cu
 // kernel attributes (dynamic shared memory limits), set once per device; call with the
 // device current before any launch or capture on it
 cudaError_t prepare_kernels();
 // mu_F and S_FF of every window corner of each image: stats = n_images x 2 planes; with
 // kind 0 (SiLNCC) the second plane holds 1 / (S_FF + eps) instead of S_FF
-void launch_fixed_stats(const float* imgs, int n_images, Dims ni, int window, int kind, float eps, float* stats,
-                        cudaStream_t s);
+void launch_fixed_stats(const float* imgs, int n_images, int batch, Dims ni, int window, int kind, float eps,
+                        float* stats, cudaStream_t s);
 int sim_ncoef(int kind);
 // maps for W (capacity n_pairs volumes), the n_images fixed images and the coefficient
 // buffer (n_pairs * NC volumes), all with stride nvox(ni) between volumes
@@ -214,6 +218,8 @@ void launch_jacobian_det(const float* u, Dims n, float* J, cudaStream_t s);
 size_t metrics_scratch_doubles();
 void launch_deformation_metrics(const float* ut, const float* ue, const unsigned char* roi, Dims n, double* scratch,
                                 double* out, cudaStream_t s);
+// ops.cu: gives the unused scratch that the stateless calls keep back to the device
+void trim_op_pools();
 // single-CTA deterministic loss reduction; writes out[0..4], hist[*step], flag, ++*step
 void launch_loss_reduce(const double* sim_part, int n_sim, const double* reg_part, int n_reg,
                         double inv_NR, double inv_F, double inv_Nm2, float a_ss, float a_l2,

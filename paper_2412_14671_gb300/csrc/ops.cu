@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <cstring>
+#include <mutex>
 #include <string>
 
 #include "kernels.h"
@@ -32,7 +34,59 @@ bool dims_ok(int64_t D, int64_t H, int64_t W) {
 }
 }  // namespace
 
+// ---- scratch of the stateless calls: a memory pool of the library per device. The default pool gives
+// everything back at each synchronisation, so a call that returns a number to the host paid for
+// mapping its scratch again every time (about 200 us of the 290 us of a 48^3 similarity). This one
+// keeps at most kPoolKeep bytes of unused scratch; a failed allocation, of a call here or of a
+// context, gives all of it back first. Allocation and release are ordered by the caller's stream.
+namespace {
+constexpr uint64_t kPoolKeep = (uint64_t)256 << 20;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pool[kMaxDevices] = {};
+
+cudaMemPool_t op_pool() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  if (!g_pool[dev]) {
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.handleTypes = cudaMemHandleTypeNone;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t p = nullptr;
+    uint64_t keep = kPoolKeep;
+    if (cudaMemPoolCreate(&p, &props) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
+    g_pool[dev] = p;
+  }
+  return g_pool[dev];
+}
+cudaError_t op_alloc(void** out, size_t bytes, cudaStream_t s) {
+  // in a capture the graph owns the scratch, as an allocation node of the default pool
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
+  const cudaMemPool_t pool = cap == cudaStreamCaptureStatusNone ? op_pool() : nullptr;
+  if (!pool) return cudaMallocAsync(out, bytes, s);
+  cudaError_t e = cudaMallocFromPoolAsync(out, bytes, pool, s);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    muster::trim_op_pools();
+    e = cudaMallocFromPoolAsync(out, bytes, pool, s);
+  }
+  return e;
+}
+}  // namespace
+
 namespace muster {
+void trim_op_pools() {
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  for (cudaMemPool_t p : g_pool)
+    if (p) cudaMemPoolTrimTo(p, 0);
+}
 void set_ops_error(const std::string& m) { g_err = m; }
 }  // namespace muster
 
@@ -57,18 +111,19 @@ int muster_op_exp(const float* phi, int64_t D, int64_t H, int64_t W, int K, floa
   cudaStream_t s = (cudaStream_t)stream;
   const Dims n{(int)D, (int)H, (int)W};
   const size_t V = vox(n);
+  // u_0 = sign phi / 2^K, then K squarings, the last one into the caller's planar field
   float4* buf = nullptr;
-  OK_(cudaMallocAsync((void**)&buf, sizeof(float4) * 5 * V, s));
-  float4 *th = buf, *a = buf + V, *b = buf + 3 * V;
-  launch_planar_to_f4(phi, th, 1, V, s);
-  launch_exp_init(th, a, 1, n, ldexpf(1.f, -K), s);  // a[0] = +phi/2^K, a[1] = -phi/2^K
-  for (int t = 0; t < K; ++t) {
-    launch_squaring(a, b, 2, n, s);
-    float4* tmp = a;
-    a = b;
-    b = tmp;
+  OK_(op_alloc((void**)&buf, sizeof(float4) * 2 * V, s));
+  float4 *a = buf, *b = buf + V;
+  launch_planar_to_f4(phi, a, 1, V, s, sign * ldexpf(1.f, -K));
+  for (int t = 0; t + 1 < K; ++t) {
+    launch_squaring(a, b, 1, n, s, 1);
+    std::swap(a, b);
   }
-  launch_f4_to_planar(a + (sign > 0.f ? 0 : V), u, 1, V, s);
+  if (K > 0)
+    launch_squaring_planar(a, u, n, s);
+  else
+    launch_f4_to_planar(a, u, 1, V, s);
   cudaError_t e = cudaGetLastError();
   cudaFreeAsync(buf, s);
   if (e != cudaSuccess) return op_cuda(e, "exp launches");
@@ -97,50 +152,50 @@ int muster_op_similarity(const float* F, const float* W, int64_t D, int64_t H, i
     return MUSTER_OK;
   }
   const int NC = sim_ncoef(kind);
-  const SimGeom g = sim_geom(n, window, 1);
-  // scratch: [out 8 doubles | step, flag ints | partials | descriptor | coefficients | F statistics]
-  const size_t off_part = 64, off_desc = off_part + sizeof(double) * (size_t)g.ctas;
-  const size_t off_coef = (off_desc + sizeof(PairDesc) + 255) / 256 * 256;
+  const SimGeom g = sim_geom(n, window, 0, kind);
+  // scratch: [head: out 6 doubles, step, flag and wait-failure ints, descriptor | partials | coefficients |
+  // F statistics]; the head starts as zeros and the descriptor, in one copy
+  struct Head {
+    double out[6];
+    int ints[4];
+    PairDesc pd;
+  };
+  const size_t off_part = (sizeof(Head) + 255) / 256 * 256;
+  const size_t off_coef = (off_part + sizeof(double) * (size_t)g.ctas + 255) / 256 * 256;
   const size_t off_stat = off_coef + sizeof(float) * NC * V;
   const size_t bytes = off_stat + sizeof(float) * 2 * V;
   char* buf = nullptr;
-  OK_(cudaMallocAsync((void**)&buf, bytes, s));
-  double* out = (double*)buf;
-  int* ints = (int*)(buf + 48);
+  OK_(op_alloc((void**)&buf, bytes, s));
+  Head* d = (Head*)buf;
   double* part = (double*)(buf + off_part);
-  PairDesc* pd = (PairDesc*)(buf + off_desc);
   float* coef = (float*)(buf + off_coef);
   float* stat = (float*)(buf + off_stat);
-  PairDesc h{};
-  h.Ii = F;
-  h.Fs = stat;
-  cudaError_t e = cudaMemsetAsync(buf, 0, 64, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(pd, &h, sizeof(h), cudaMemcpyHostToDevice, s);
+  Head h{};
+  h.pd.Ii = F;
+  h.pd.Fs = stat;
+  cudaError_t e = cudaMemcpyAsync(d, &h, sizeof(h), cudaMemcpyHostToDevice, s);
   SimMaps maps;
   make_sim_maps(&maps, W, 1, F, 1, coef, n, window, kind);
   if (e == cudaSuccess) e = prepare_kernels();
   if (e == cudaSuccess) {
-    launch_fixed_stats(F, 1, n, window, kind, eps, stat, s);
-    launch_sim_fwd(pd, 1, 1, 1, W, V, coef, V, part, n, window, kind, eps, &maps, ints + 2, s);
-    launch_loss_reduce(part, g.ctas, nullptr, 0, 1.0 / (double)NR, 0.0, 0.0, 0.f, 0.f, 0.f, out, nullptr, ints,
-                       ints + 1, 0, s);
+    launch_fixed_stats(F, 1, 0, n, window, kind, eps, stat, s);
+    launch_sim_fwd(&d->pd, 1, 0, 1, W, V, coef, V, part, n, window, kind, eps, &maps, d->ints + 2, s);
     if (dLdW) {
       const int nw = window * window * window;
       const float scale = kind == MUSTER_SILNCC ? (float)(2.0 / ((double)nw * (double)NR)) : (float)(1.0 / (double)NR);
-      launch_sim_bwd(pd, 1, 1, 1, W, V, coef, V, dLdW, n, window, kind, scale, &maps, ints + 2, s);
+      launch_sim_bwd(&d->pd, 1, 0, 1, W, V, coef, V, dLdW, n, window, kind, scale, &maps, d->ints + 2, s);
     }
+    launch_loss_reduce(part, g.ctas, nullptr, 0, 1.0 / (double)NR, 0.0, 0.0, 0.f, 0.f, 0.f, d->out, nullptr, d->ints,
+                       d->ints + 1, 0, s);
     e = cudaGetLastError();
   }
-  double host_out[2] = {0.0, 0.0};
-  int host_err = 0;
-  if (e == cudaSuccess && loss) e = cudaMemcpyAsync(host_out, out, sizeof(double) * 2, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess && loss) e = cudaMemcpyAsync(&host_err, ints + 2, sizeof(int), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess && loss) e = cudaMemcpyAsync(&h, d, offsetof(Head, pd), cudaMemcpyDeviceToHost, s);
   cudaFreeAsync(buf, s);
   if (e != cudaSuccess) return op_cuda(e, "similarity launches");
   if (loss) {
     OK_(cudaStreamSynchronize(s));
-    if (host_err) return op_fail(MUSTER_ETIMEOUT, "a bounded wait for an input copy ran out");
-    *loss = host_out[1];
+    if (h.ints[2]) return op_fail(MUSTER_ETIMEOUT, "a bounded wait for an input copy ran out");
+    *loss = h.out[1];
   }
   return MUSTER_OK;
 }
@@ -161,7 +216,7 @@ int muster_op_deformation_metrics(const float* u_true, const float* u_est, const
   cudaStream_t s = (cudaStream_t)stream;
   const size_t nd = metrics_scratch_doubles();
   double* buf = nullptr;
-  OK_(cudaMallocAsync((void**)&buf, sizeof(double) * (nd + 16), s));
+  OK_(op_alloc((void**)&buf, sizeof(double) * (nd + 16), s));
   launch_deformation_metrics(u_true, u_est, roi, Dims{(int)D, (int)H, (int)Wd}, buf, buf + nd, s);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaMemcpyAsync(out, buf + nd, sizeof(double) * 16, cudaMemcpyDeviceToHost, s);

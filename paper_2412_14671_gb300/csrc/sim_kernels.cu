@@ -881,13 +881,40 @@ int chunk_for(int ntiles, int depth, int min_chunk, int threads, int batch) {
   return tz < 1 ? 1 : tz;
 }
 
-Tiles sim_tiles(Dims ni, int n_pairs, int batch, int group) {
+// D chunks of a launch of `tiles` tiles that should fill the device on its own (one pair of a
+// stateless call). Every chunk streams 2R planes more than it covers, so fewer chunks do less work;
+// more chunks fill more SMs. The cost of a chunking is its planes per CTA times the time of a plane at
+// its CTAs per SM: c <= 4 resident CTAs take about 0.55 + 0.21 c us per plane (one 160 x 192 x 160
+// pair, w = 7, forward: 0.97 us at 2, 1.39 us at 4), and more than 4 follow one another. That pair runs
+// in 10 chunks (forward and adjoint 57 us), where the rule above takes 2 (148 us).
+int filling_chunks(long tiles, int depth, int reach) {
+  const long sms = device_sm_count();
+  auto wave = [](long c) { return c ? 26 + 10 * c : 0; };
+  int best = 1;
+  long cost = 0;
+  for (int c = 1; c <= depth && (c == 1 || tiles * c <= 8 * sms); ++c) {
+    const long tz = (depth + c - 1) / c, per_sm = (tiles * c + sms - 1) / sms;
+    const long k = (tz + reach + 1) * (per_sm / 4 * wave(4) + wave(per_sm % 4));
+    if (c == 1 || k < cost) best = c, cost = k;
+  }
+  return best;
+}
+
+// batch 0: a stateless call. Its chunks may lie elsewhere than the engine's, for SiLNCC: LNCC's
+// gradient follows the rounding of the window sums in flat regions, so it keeps the one rule.
+int chunk_planes(int ntiles, Dims ni, int window, int kind, int min_chunk, int threads, int batch) {
+  if (batch > 0 || kind != 0) return chunk_for(ntiles, ni.n0, min_chunk, threads, std::max(batch, 1));
+  const int c = filling_chunks(ntiles, ni.n0, window - 1);
+  return (ni.n0 + c - 1) / c;
+}
+
+Tiles sim_tiles(Dims ni, int window, int kind, int n_pairs, int batch, int group) {
   Tiles g;
   g.np = n_pairs;
   g.grp = std::max(1, std::min(group, n_pairs));
   g.gx = (ni.n2 + kTX - 1) / kTX;
   g.gy = (ni.n1 + kTY - 1) / kTY;
-  g.tz = chunk_for(g.gx * g.gy, ni.n0, 8, 256, batch);
+  g.tz = chunk_planes(g.gx * g.gy, ni, window, kind, 8, 256, batch);
   g.nzc = (ni.n0 + g.tz - 1) / g.tz;
   return g;
 }
@@ -907,10 +934,10 @@ void fixed_stats(dim3 g, const float* imgs, Dims ni, int window, float eps, floa
 }
 }  // namespace
 
-void launch_fixed_stats(const float* imgs, int n_images, Dims ni, int window, int kind, float eps, float* stats,
-                        cudaStream_t s) {
+void launch_fixed_stats(const float* imgs, int n_images, int batch, Dims ni, int window, int kind, float eps,
+                        float* stats, cudaStream_t s) {
   const int gx = (ni.n2 + TX - 1) / TX, gy = (ni.n1 + 7) / 8;
-  const int tz = chunk_for(gx * gy, ni.n0, 16, 128, 1), nzc = (ni.n0 + tz - 1) / tz;
+  const int tz = chunk_planes(gx * gy, ni, window, kind, 16, 128, batch), nzc = (ni.n0 + tz - 1) / tz;
   const dim3 g(gx, gy, nzc * n_images);
   if (kind == 0)
     fixed_stats<0>(g, imgs, ni, window, eps, stats, tz, nzc, s);
@@ -930,9 +957,8 @@ cudaError_t prepare_kernels() {
   });
 }
 
-SimGeom sim_geom(Dims ni, int window, int batch) {
-  (void)window;
-  const Tiles g = sim_tiles(ni, 1, batch, 1);
+SimGeom sim_geom(Dims ni, int window, int batch, int kind) {
+  const Tiles g = sim_tiles(ni, window, kind, 1, batch, 1);
   return SimGeom{g.nzc, g.tz, (int)ctas(g)};
 }
 int sim_ncoef(int kind) { return kind == 0 ? 2 : 3; }
@@ -950,7 +976,7 @@ void make_sim_maps(SimMaps* m, const float* W, int n_pairs, const float* imgs, i
 void launch_sim_fwd(const PairDesc* pd, int n_pairs, int batch, int group, const float* W, size_t Wstride, float* coef,
                     size_t cs, double* partials, Dims ni, int window, int kind, float eps, const SimMaps* maps,
                     int* err, cudaStream_t s) {
-  const Tiles g = sim_tiles(ni, n_pairs, batch, group);
+  const Tiles g = sim_tiles(ni, window, kind, n_pairs, batch, group);
   dispatch(window / 2, kind, maps && maps->fwd_ok, [&](auto r, auto k, auto t) {
     k_sim_fwd<r(), k(), t()><<<ctas(g), Box<r()>::NT, Box<r()>::bytes(2, k() == 0 ? 2 : 3), s>>>(
         maps ? *maps : SimMaps{}, pd, W, Wstride, coef, cs, partials, ni, g, eps, err);
@@ -959,7 +985,7 @@ void launch_sim_fwd(const PairDesc* pd, int n_pairs, int batch, int group, const
 void launch_sim_bwd(const PairDesc* pd, int n_pairs, int batch, int group, const float* W, size_t Wstride,
                     const float* coef, size_t cs, float* dLdW, Dims ni, int window, int kind, float scale,
                     const SimMaps* maps, int* err, cudaStream_t s) {
-  const Tiles g = sim_tiles(ni, n_pairs, batch, group);
+  const Tiles g = sim_tiles(ni, window, kind, n_pairs, batch, group);
   dispatch(window / 2, kind, maps && maps->bwd_ok, [&](auto r, auto k, auto t) {
     constexpr int nc = k() == 0 ? 2 : 3;
     k_sim_bwd<r(), k(), t()><<<ctas(g), Box<r()>::NT, Box<r()>::bytes(nc, nc), s>>>(
