@@ -19,7 +19,7 @@
 namespace muster {
 
 namespace {
-constexpr int kJX = 32, kJY = 8;         // Jacobian: CTA tile (W x H) of one plane
+constexpr int kJT = 256;                 // Jacobian: threads per CTA
 // metrics: threads per CTA, and the most CTAs of the grid-stride passes (3 per SM of the
 // device; kMCtas bounds the scratch of the per-CTA partial sums)
 constexpr int kMT = 256, kMCtas = 3 * 256, kMCtasPerSM = 3;
@@ -34,53 +34,82 @@ __device__ __forceinline__ float dstep(float lo, float mid, float hi, int p, int
   return 0.5f * (hi - lo);
 }
 
-// Streams along D: each thread owns one (y, x) column of a 32 x 8 tile and keeps the three
-// components at planes z-1, z, z+1 in registers; plane z of the tile with a 1-voxel halo
-// in W and H is staged in shared memory for the in-plane differences.
-__global__ void __launch_bounds__(kJX* kJY) k_jacobian_det(const float* __restrict__ u, Dims n, float* __restrict__ J,
-                                                           int zchunk) {
-  __shared__ float tile[3][kJY + 2][kJX + 2];
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const int x = blockIdx.x * kJX + tx, y = blockIdx.y * kJY + ty;
-  const int z0 = blockIdx.z * zchunk, z1 = min(z0 + zchunk, n.n0);
+// A thread owns NX neighbouring voxels of a row (4 with 16-byte loads when the width is a multiple
+// of 4 and the fields are 16-byte aligned, else 1) and walks a chunk of D with the planes z-1, z, z+1 of
+// the three components in registers. The rows y-1 and y+1 of plane z are loads that hit the L1 or
+// L2 lines of the neighbouring threads' own rows; x-1 and x+NX come from the neighbouring lanes, or
+// from memory at a row's or warp's end. DRAM bounds it (16 bytes per voxel); the walk is short, so
+// that every SM has loads of some 1400 threads in flight. 160 x 192 x 160: @JACT@ us; staging
+// every plane of a 32 x 8 tile in shared memory behind two barriers took 39 us.
+template <int NX>
+struct Run {
+  float v[NX];
+};
+template <int NX>
+__device__ __forceinline__ Run<NX> load_run(const float* __restrict__ p) {
+  Run<NX> r;
+  if constexpr (NX == 4) {
+    const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+    r.v[0] = t.x, r.v[1] = t.y, r.v[2] = t.z, r.v[3] = t.w;
+  } else {
+    r.v[0] = __ldg(p);
+  }
+  return r;
+}
+template <int NX>
+__global__ void __launch_bounds__(kJT) k_jacobian_det(const float* __restrict__ u, Dims n, float* __restrict__ J,
+                                                      int zchunk) {
+  const int runs = n.n2 / NX, i = blockIdx.x * kJT + threadIdx.x, lane = threadIdx.x & 31;
+  const bool in = i < runs * n.n1;
+  const int y = in ? i / runs : 0, x = in ? (i - y * runs) * NX : 0;
+  const int z0 = blockIdx.y * zchunk, z1 = min(z0 + zchunk, n.n0);
   const size_t V = vox(n);
-  const int plane = n.n1 * n.n2;
-  const bool in = x < n.n2 && y < n.n1;
-  const int xc = min(x, n.n2 - 1), yc = min(y, n.n1 - 1);
-  const float* col = u + (size_t)yc * n.n2 + xc;
-  // halo loaders: threads of the first/last column and row also fetch the neighbour cell
-  const int hx = tx == 0 ? max(blockIdx.x * kJX - 1, 0) : (tx == kJX - 1 ? min(x + 1, n.n2 - 1) : -1);
-  const int hy = ty == 0 ? max(blockIdx.y * kJY - 1, 0) : (ty == kJY - 1 ? min(y + 1, n.n1 - 1) : -1);
-  float prv[3], cur[3], nxt[3];
+  const ptrdiff_t plane = (ptrdiff_t)n.n1 * n.n2;
+  const int below = y > 0 ? -n.n2 : 0, above = y < n.n1 - 1 ? n.n2 : 0;
+  const bool left = x > 0, right = x + NX < n.n2;  // x-1 and x+NX exist
+  const float* f = u + (size_t)y * n.n2 + x + z0 * plane;
+  Run<NX> prv[3], cur[3], nxt[3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    const float* f = col + (size_t)c * V;
-    cur[c] = __ldg(f + (size_t)z0 * plane);
-    prv[c] = z0 > 0 ? __ldg(f + (size_t)(z0 - 1) * plane) : cur[c];
+    cur[c] = load_run<NX>(f + c * V);
+    prv[c] = z0 > 0 ? load_run<NX>(f + c * V - plane) : cur[c];
   }
-  for (int z = z0; z < z1; ++z) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c) nxt[c] = z + 1 < n.n0 ? __ldg(col + (size_t)c * V + (size_t)(z + 1) * plane) : cur[c];
-    __syncthreads();  // the previous plane's reads of the tile are done
+  for (int z = z0; z < z1; ++z, f += plane) {
+    Run<NX> lo[3], hi[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const float* f = u + (size_t)c * V + (size_t)z * plane;
-      tile[c][ty + 1][tx + 1] = cur[c];
-      if (hx >= 0) tile[c][ty + 1][tx == 0 ? 0 : kJX + 1] = __ldg(f + (size_t)yc * n.n2 + hx);
-      if (hy >= 0) tile[c][ty == 0 ? 0 : kJY + 1][tx + 1] = __ldg(f + (size_t)hy * n.n2 + xc);
+      nxt[c] = z + 1 < n.n0 ? load_run<NX>(f + c * V + plane) : cur[c];
+      lo[c] = load_run<NX>(f + c * V + below);
+      hi[c] = load_run<NX>(f + c * V + above);
     }
-    __syncthreads();
-    if (in) {
-      float M[3][3];
+    float M[NX][3][3];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        M[c][0] = (c == 0 ? 1.f : 0.f) + dstep(prv[c], cur[c], nxt[c], z, n.n0);
-        M[c][1] = (c == 1 ? 1.f : 0.f) + dstep(tile[c][ty][tx + 1], cur[c], tile[c][ty + 2][tx + 1], y, n.n1);
-        M[c][2] = (c == 2 ? 1.f : 0.f) + dstep(tile[c][ty + 1][tx], cur[c], tile[c][ty + 1][tx + 2], x, n.n2);
+    for (int c = 0; c < 3; ++c) {
+      // the voxels beside the run: a run of the same row in the next lane, else memory
+      float l = __shfl_up_sync(0xffffffffu, cur[c].v[NX - 1], 1), r = __shfl_down_sync(0xffffffffu, cur[c].v[0], 1);
+      if (lane == 0 && left) l = __ldg(f + c * V - 1);
+      if (lane == 31 && right) r = __ldg(f + c * V + NX);
+#pragma unroll
+      for (int k = 0; k < NX; ++k) {
+        const float mid = cur[c].v[k];
+        M[k][c][0] = (c == 0 ? 1.f : 0.f) + dstep(prv[c].v[k], mid, nxt[c].v[k], z, n.n0);
+        M[k][c][1] = (c == 1 ? 1.f : 0.f) + dstep(lo[c].v[k], mid, hi[c].v[k], y, n.n1);
+        M[k][c][2] = (c == 2 ? 1.f : 0.f) + dstep(k > 0 ? cur[c].v[k - 1] : l, mid, k < NX - 1 ? cur[c].v[k + 1] : r, x + k, n.n2);
       }
-      J[(size_t)z * plane + (size_t)y * n.n2 + x] =
-          M[0][0] * (M[1][1] * M[2][2] - M[1][2] * M[2][1]) - M[0][1] * (M[1][0] * M[2][2] - M[1][2] * M[2][0]) +
-          M[0][2] * (M[1][0] * M[2][1] - M[1][1] * M[2][0]);
+    }
+    float det[NX];
+#pragma unroll
+    for (int k = 0; k < NX; ++k) {
+      const float(*A)[3] = M[k];
+      det[k] = A[0][0] * (A[1][1] * A[2][2] - A[1][2] * A[2][1]) - A[0][1] * (A[1][0] * A[2][2] - A[1][2] * A[2][0]) +
+               A[0][2] * (A[1][0] * A[2][1] - A[1][1] * A[2][0]);
+    }
+    if (in) {
+      float* o = J + (size_t)z * plane + (size_t)y * n.n2 + x;
+      if constexpr (NX == 4)
+        *reinterpret_cast<float4*>(o) = make_float4(det[0], det[1], det[2], det[3]);
+      else
+        o[0] = det[0];
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -111,11 +140,6 @@ __device__ __forceinline__ DF df_add(DF x, DF y) {
   const DF s = two_sum(x.hi, y.hi);
   return fast_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(x.lo, y.lo)));
 }
-__device__ __forceinline__ DF df_mul(DF x, DF y) {
-  const float p = __fmul_rn(x.hi, y.hi);
-  const float e = fmaf(x.hi, y.hi, -p);  // a b - p exactly
-  return fast_two_sum(p, __fadd_rn(e, __fadd_rn(__fmul_rn(x.hi, y.lo), __fmul_rn(x.lo, y.hi))));
-}
 // a - (m_hi + m_lo) for a float a and a split double m
 __device__ __forceinline__ DF df_sub_split(float a, float m_hi, float m_lo) {
   const DF s = two_sum(a, -m_hi);
@@ -130,28 +154,70 @@ __device__ __forceinline__ DF df_sqrt(DF x) {
 }
 __device__ __forceinline__ double df_val(DF x) { return (double)x.hi + (double)x.lo; }
 
-// fixed-order sum of one double over the CTA (result valid in thread 0)
-__device__ __forceinline__ double cta_sum(double x, double* sh) {
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+// acc += x without renormalising acc: the high parts by two_sum, everything else into the low part
+// (a thread adds some tens of terms, so the low part stays below 2^-20 of the high part)
+__device__ __forceinline__ void df_accumulate(DF& acc, DF x) {
+  const DF s = two_sum(acc.hi, x.hi);
+  acc.hi = s.hi;
+  acc.lo = __fadd_rn(acc.lo, __fadd_rn(s.lo, x.lo));
+}
+// acc += x y
+__device__ __forceinline__ void df_accumulate_product(DF& acc, DF x, DF y) {
+  const float p = __fmul_rn(x.hi, y.hi);
+  const float e = __fmaf_rn(x.hi, y.hi, -p);
+  df_accumulate(acc, DF{p, __fmaf_rn(x.hi, y.lo, __fmaf_rn(x.lo, y.hi, e))});
+}
+
+// the CTA's sums of NK double-float values per thread, written as doubles to part[0 .. NK) by the
+// first NK threads, in a fixed order: each value's kMT entries are added in 16 runs of 16 threads'
+// entries in double-float arithmetic, then the runs in double
+template <int NK>
+__device__ __forceinline__ void cta_sums(const DF (&acc)[NK], double* __restrict__ part) {
+  constexpr int kRuns = 16;
+  static_assert(NK <= kMT / kRuns, "one run per thread");
+  __shared__ DF sh[NK][kMT + 1];
+  __shared__ double run[NK][kRuns];
+#pragma unroll
+  for (int k = 0; k < NK; ++k) sh[k][threadIdx.x] = fast_two_sum(acc[k].hi, acc[k].lo);
   __syncthreads();
-  if (l == 0) sh[w] = x;
+  const int k = threadIdx.x / kRuns, r = threadIdx.x % kRuns;
+  if (k < NK) {
+    DF s{0.f, 0.f};
+    for (int i = 0; i < kMT / kRuns; ++i) s = df_add(s, sh[k][i * kRuns + r]);
+    run[k][r] = df_val(s);
+  }
   __syncthreads();
-  double r = 0.0;
-  if (threadIdx.x == 0)
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) r += sh[i];
-  return r;
+  if (threadIdx.x < NK) {
+    double s = 0.0;
+    for (int i = 0; i < kRuns; ++i) s += run[threadIdx.x][i];
+    part[threadIdx.x] = s;
+  }
+}
+
+// out[0 .. nk) = sums over the nparts rows of nk doubles, in a fixed order (one CTA; sh: kMT doubles)
+__device__ __forceinline__ void part_sums(const double* __restrict__ part, int nparts, int nk, double* sh,
+                                          double* out) {
+  const int lanes = kMT / nk, k = threadIdx.x % nk, l = threadIdx.x / nk;
+  double a = 0.0;
+  for (int i = l; i < nparts; i += lanes) a += part[(size_t)i * nk + k];
+  sh[threadIdx.x] = a;
+  __syncthreads();
+  if (threadIdx.x < nk) {
+    double s = 0.0;
+    for (int i = 0; i < lanes; ++i) s += sh[i * nk + threadIdx.x];
+    out[threadIdx.x] = s;
+  }
+  __syncthreads();
 }
 
 // pass 1: count, sum |ut - ue|, sum ut, sum ue
 __global__ void __launch_bounds__(kMT) k_metrics_pass1(const float* __restrict__ ut, const float* __restrict__ ue,
                                                        const unsigned char* __restrict__ roi, size_t V,
                                                        double* __restrict__ part) {
-  __shared__ double sh[kMT / 32];
   int count = 0;
-  DF acc[kP1 - 1];  // sum |d|, sum ut (3), sum ue (3)
+  DF acc[kP1];  // count, sum |d|, sum ut (3), sum ue (3)
 #pragma unroll
-  for (int k = 0; k < kP1 - 1; ++k) acc[k] = DF{0.f, 0.f};
+  for (int k = 0; k < kP1; ++k) acc[k] = DF{0.f, 0.f};
   for (size_t v = (size_t)blockIdx.x * kMT + threadIdx.x; v < V; v += (size_t)gridDim.x * kMT) {
     if (roi && !roi[v]) continue;
     DF d2{0.f, 0.f};
@@ -159,44 +225,31 @@ __global__ void __launch_bounds__(kMT) k_metrics_pass1(const float* __restrict__
     for (int c = 0; c < 3; ++c) {
       const float a = ut[(size_t)c * V + v], b = ue[(size_t)c * V + v];
       const DF d = two_sum(a, -b);  // a - b exactly
-      d2 = df_add(d2, df_mul(d, d));
-      acc[1 + c] = df_add(acc[1 + c], DF{a, 0.f});
-      acc[4 + c] = df_add(acc[4 + c], DF{b, 0.f});
+      df_accumulate_product(d2, d, d);
+      df_accumulate(acc[2 + c], DF{a, 0.f});
+      df_accumulate(acc[5 + c], DF{b, 0.f});
     }
     ++count;
-    acc[0] = df_add(acc[0], df_sqrt(d2));
+    df_accumulate(acc[1], df_sqrt(fast_two_sum(d2.hi, d2.lo)));
   }
-  {
-    const double s = cta_sum((double)count, sh);
-    if (threadIdx.x == 0) part[(size_t)blockIdx.x * kP1] = s;
-  }
-#pragma unroll
-  for (int k = 0; k < kP1 - 1; ++k) {
-    const double s = cta_sum(df_val(acc[k]), sh);
-    if (threadIdx.x == 0) part[(size_t)blockIdx.x * kP1 + 1 + k] = s;
-  }
+  // a thread's count (below 2^31 voxels over the grid) as a float pair: 24 low bits and the rest
+  acc[0] = DF{(float)(count & ~0xffffff), (float)(count & 0xffffff)};
+  cta_sums<kP1>(acc, part + (size_t)blockIdx.x * kP1);
 }
 
 // means from the pass-1 partials: stats = {count, sum |d|, mt[3], me[3]} with means in place
 __global__ void __launch_bounds__(kMT) k_metrics_means(const double* __restrict__ part, int nparts,
                                                        double* __restrict__ stats) {
-  __shared__ double sh[kMT / 32];
-  for (int k = 0; k < kP1; ++k) {
-    double a = 0.0;
-    for (int i = threadIdx.x; i < nparts; i += kMT) a += part[(size_t)i * kP1 + k];
-    const double s = cta_sum(a, sh);
-    if (threadIdx.x == 0) stats[k] = s;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0 && stats[0] > 0.0)
-    for (int k = 2; k < kP1; ++k) stats[k] /= stats[0];
+  __shared__ double sh[kMT];
+  __shared__ double S[kP1];
+  part_sums(part, nparts, kP1, sh, S);
+  if (threadIdx.x < kP1) stats[threadIdx.x] = threadIdx.x >= 2 && S[0] > 0.0 ? S[threadIdx.x] / S[0] : S[threadIdx.x];
 }
 
 // pass 2: centred moments Ctt (6 unique), Cet (9), see
 __global__ void __launch_bounds__(kMT) k_metrics_pass2(const float* __restrict__ ut, const float* __restrict__ ue,
                                                        const unsigned char* __restrict__ roi, size_t V,
                                                        const double* __restrict__ stats, double* __restrict__ part) {
-  __shared__ double sh[kMT / 32];
   // the means as double-float pairs (hi = nearest float, lo = the float of the remainder)
   float mh[6], ml[6];
 #pragma unroll
@@ -216,37 +269,28 @@ __global__ void __launch_bounds__(kMT) k_metrics_pass2(const float* __restrict__
       a[c] = df_sub_split(ut[(size_t)c * V + v], mh[c], ml[c]);
       b[c] = df_sub_split(ue[(size_t)c * V + v], mh[3 + c], ml[3 + c]);
     }
-    acc[0] = df_add(acc[0], df_mul(a[0], a[0]));
-    acc[1] = df_add(acc[1], df_mul(a[0], a[1]));
-    acc[2] = df_add(acc[2], df_mul(a[0], a[2]));
-    acc[3] = df_add(acc[3], df_mul(a[1], a[1]));
-    acc[4] = df_add(acc[4], df_mul(a[1], a[2]));
-    acc[5] = df_add(acc[5], df_mul(a[2], a[2]));
+    df_accumulate_product(acc[0], a[0], a[0]);
+    df_accumulate_product(acc[1], a[0], a[1]);
+    df_accumulate_product(acc[2], a[0], a[2]);
+    df_accumulate_product(acc[3], a[1], a[1]);
+    df_accumulate_product(acc[4], a[1], a[2]);
+    df_accumulate_product(acc[5], a[2], a[2]);
 #pragma unroll
     for (int r = 0; r < 3; ++r)
 #pragma unroll
-      for (int c = 0; c < 3; ++c) acc[6 + 3 * r + c] = df_add(acc[6 + 3 * r + c], df_mul(b[r], a[c]));
-    acc[15] = df_add(acc[15], df_add(df_add(df_mul(b[0], b[0]), df_mul(b[1], b[1])), df_mul(b[2], b[2])));
-  }
+      for (int c = 0; c < 3; ++c) df_accumulate_product(acc[6 + 3 * r + c], b[r], a[c]);
 #pragma unroll
-  for (int k = 0; k < kP2; ++k) {
-    const double s = cta_sum(df_val(acc[k]), sh);
-    if (threadIdx.x == 0) part[(size_t)blockIdx.x * kP2 + k] = s;
+    for (int c = 0; c < 3; ++c) df_accumulate_product(acc[15], b[c], b[c]);
   }
+  cta_sums<kP2>(acc, part + (size_t)blockIdx.x * kP2);
 }
 
 // final: fixed-order sums of the pass-2 partials, then Eu, PCC, A = Cet Ctt^-1, b, B
 __global__ void __launch_bounds__(kMT) k_metrics_final(const double* __restrict__ part, int nparts,
                                                        const double* __restrict__ stats, double* __restrict__ out) {
-  __shared__ double sh[kMT / 32];
+  __shared__ double sh[kMT];
   __shared__ double S[kP2];
-  for (int k = 0; k < kP2; ++k) {
-    double a = 0.0;
-    for (int i = threadIdx.x; i < nparts; i += kMT) a += part[(size_t)i * kP2 + k];
-    const double s = cta_sum(a, sh);
-    if (threadIdx.x == 0) S[k] = s;
-  }
-  __syncthreads();
+  part_sums(part, nparts, kP2, sh, S);
   if (threadIdx.x != 0) return;
   for (int k = 0; k < 16; ++k) out[k] = 0.0;
   const double cnt = stats[0];
@@ -260,16 +304,17 @@ __global__ void __launch_bounds__(kMT) k_metrics_final(const double* __restrict_
   const double det = C[0][0] * (C[1][1] * C[2][2] - C[1][2] * C[2][1]) -
                      C[0][1] * (C[1][0] * C[2][2] - C[1][2] * C[2][0]) +
                      C[0][2] * (C[1][0] * C[2][1] - C[1][1] * C[2][0]);
+  const double rdet = 1.0 / det;
   double inv[3][3];
-  inv[0][0] = (C[1][1] * C[2][2] - C[1][2] * C[2][1]) / det;
-  inv[0][1] = (C[0][2] * C[2][1] - C[0][1] * C[2][2]) / det;
-  inv[0][2] = (C[0][1] * C[1][2] - C[0][2] * C[1][1]) / det;
-  inv[1][0] = (C[1][2] * C[2][0] - C[1][0] * C[2][2]) / det;
-  inv[1][1] = (C[0][0] * C[2][2] - C[0][2] * C[2][0]) / det;
-  inv[1][2] = (C[0][2] * C[1][0] - C[0][0] * C[1][2]) / det;
-  inv[2][0] = (C[1][0] * C[2][1] - C[1][1] * C[2][0]) / det;
-  inv[2][1] = (C[0][1] * C[2][0] - C[0][0] * C[2][1]) / det;
-  inv[2][2] = (C[0][0] * C[1][1] - C[0][1] * C[1][0]) / det;
+  inv[0][0] = (C[1][1] * C[2][2] - C[1][2] * C[2][1]) * rdet;
+  inv[0][1] = (C[0][2] * C[2][1] - C[0][1] * C[2][2]) * rdet;
+  inv[0][2] = (C[0][1] * C[1][2] - C[0][2] * C[1][1]) * rdet;
+  inv[1][0] = (C[1][2] * C[2][0] - C[1][0] * C[2][2]) * rdet;
+  inv[1][1] = (C[0][0] * C[2][2] - C[0][2] * C[2][0]) * rdet;
+  inv[1][2] = (C[0][2] * C[1][0] - C[0][0] * C[1][2]) * rdet;
+  inv[2][0] = (C[1][0] * C[2][1] - C[1][1] * C[2][0]) * rdet;
+  inv[2][1] = (C[0][1] * C[2][0] - C[0][0] * C[2][1]) * rdet;
+  inv[2][2] = (C[0][0] * C[1][1] - C[0][1] * C[1][0]) * rdet;
   double tr = 0.0;
   for (int r = 0; r < 3; ++r) {
     double Ar[3];
@@ -283,12 +328,18 @@ __global__ void __launch_bounds__(kMT) k_metrics_final(const double* __restrict_
 }  // namespace
 
 void launch_jacobian_det(const float* u, Dims n, float* J, cudaStream_t s) {
-  // D chunks so that the grid has at least 8 CTAs per SM of the device
-  const int gx = (n.n2 + kJX - 1) / kJX, gy = (n.n1 + kJY - 1) / kJY;
-  const long want = 8L * device_sm_count();
+  const bool four = n.n2 % 4 == 0 && (reinterpret_cast<uintptr_t>(u) & 15) == 0 && (reinterpret_cast<uintptr_t>(J) & 15) == 0;
+  // D chunks so that the grid has at least 5 CTAs per SM of the device
+  const size_t runs = (size_t)n.n1 * (four ? n.n2 / 4 : n.n2);
+  const unsigned gx = (unsigned)((runs + kJT - 1) / kJT);
+  const long want = 5L * device_sm_count();
   int zc = n.n0;
-  while (zc > 4 && (long)gx * gy * ((n.n0 + zc - 1) / zc) < want) zc = (zc + 1) / 2;
-  k_jacobian_det<<<dim3(gx, gy, (n.n0 + zc - 1) / zc), dim3(kJX, kJY), 0, s>>>(u, n, J, zc);
+  while (zc > 4 && (long)gx * ((n.n0 + zc - 1) / zc) < want) zc = (zc + 1) / 2;
+  const dim3 g(gx, (n.n0 + zc - 1) / zc);
+  if (four)
+    k_jacobian_det<4><<<g, kJT, 0, s>>>(u, n, J, zc);
+  else
+    k_jacobian_det<1><<<g, kJT, 0, s>>>(u, n, J, zc);
 }
 
 size_t metrics_scratch_doubles() { return (size_t)kMCtas * (kP1 + kP2) + kP1; }
