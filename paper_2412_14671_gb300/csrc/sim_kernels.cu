@@ -602,7 +602,7 @@ __global__ void __launch_bounds__(Box<R>::NT, kMinCtas)
     auto window = [&](int i, float muF, float Sff, float& c0, float& c1, float& c2) -> float {
       const float s0 = ring.S[0][i];
       const float Sfw = ring.S[NM - 1][i] - (muF - shF) * s0;
-      const float muW = s0 * inv_nw + shW;
+      const float muW = __fmaf_rn(s0, inv_nw, shW);  // s0 * inv_nw is used again below: fused all the same
       if (KIND == 0) {
         const float beta = Sfw * Sff;  // Sff holds 1 / (S_FF + eps) for SiLNCC
         c0 = beta;
