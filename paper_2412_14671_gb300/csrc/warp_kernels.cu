@@ -201,6 +201,30 @@ __global__ void __launch_bounds__(BX* BY, kWarpCtas) k_warp(const PairDesc* __re
   }
 }
 
+// racc += sums of dL/dq and dL/dq p^T over the block of node (mz, my, mx), g = 2 dL/dq: with p = 2 m + d
+// the products reduce to 2 m sum g + sum over d_a = 1 of g, per axis a
+template <int NR>
+__device__ __forceinline__ void rigid_sums(const float3 (&g)[2][2][2], int mz, int my, int mx, float (&racc)[NR]) {
+  if constexpr (NR == 12) {
+    const float m2[3] = {(float)(2 * mz), (float)(2 * my), (float)(2 * mx)};
+    auto add = [](float3 a, float3 b) { return make_float3(a.x + b.x, a.y + b.y, a.z + b.z); };
+    const float3 z0y0 = add(g[0][0][0], g[0][0][1]), z0y1 = add(g[0][1][0], g[0][1][1]);
+    const float3 z1y0 = add(g[1][0][0], g[1][0][1]), z1y1 = add(g[1][1][0], g[1][1][1]);
+    const float3 hi[3] = {add(z1y0, z1y1), add(z0y1, z1y1),
+                          add(add(g[0][0][1], g[0][1][1]), add(g[1][0][1], g[1][1][1]))};
+    const float3 all = add(add(z0y0, z0y1), hi[0]);
+    const float s[3] = {0.5f * all.x, 0.5f * all.y, 0.5f * all.z};
+#pragma unroll
+    for (int q = 0; q < 3; ++q) racc[q] += s[q];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      racc[3 + a] += fmaf(m2[a], s[0], 0.5f * hi[a].x);
+      racc[6 + a] += fmaf(m2[a], s[1], 0.5f * hi[a].y);
+      racc[9 + a] += fmaf(m2[a], s[2], 0.5f * hi[a].z);
+    }
+  }
+}
+
 // ---- adjoint: g(p) = 2 dL/dW(p) grad S[I_k](p + U~(p)) at every image voxel (the image
 // gradient at the sample point was stored by the forward warp), then
 // dL/dU(node) = sum over the image voxels of the node's stencil with the same
@@ -275,23 +299,7 @@ __global__ void __launch_bounds__(RX* RY) k_warp_bwd2(const PairDesc* __restrict
     if (RIGID && writer && mz >= Z0 && mz < Z1) {
       // g holds 2 dL/dq (the 2 of the flow-to-image scale); image voxels outside the
       // grid were left at 0
-#pragma unroll
-      for (int dz = 0; dz < 2; ++dz)
-#pragma unroll
-        for (int dy = 0; dy < 2; ++dy)
-#pragma unroll
-          for (int dx = 0; dx < 2; ++dx) {
-            const float3 q = g[dz][dy][dx];
-            const float gx = 0.5f * q.x, gy = 0.5f * q.y, gz = 0.5f * q.z;
-            const float pz = (float)(2 * mz + dz), py = (float)(2 * my + dy), px = (float)(2 * mx + dx);
-            float* r = racc;
-            r[0] += gx, r[1 % (RIGID ? 12 : 1)] += gy, r[2 % (RIGID ? 12 : 1)] += gz;
-            if (RIGID) {
-              r[3] += gx * pz, r[4] += gx * py, r[5] += gx * px;
-              r[6] += gy * pz, r[7] += gy * py, r[8] += gy * px;
-              r[9] += gz * pz, r[10] += gz * py, r[11] += gz * px;
-            }
-          }
+      rigid_sums(g, mz, my, mx, racc);
     }
     // transpose along W: node mx gets 0.75 (g0 + g1) of its block, 0.25 g1 of block mx-1
     // and 0.25 g0 of block mx+1 (neighbouring lanes); edge nodes keep their folded share
@@ -455,23 +463,7 @@ __global__ void __launch_bounds__(RX* RY) k_warp_bwd3t(const __grid_constant__ W
     if (RIGID && writer && mz >= Z0 && mz < Z1) {
       // g holds 2 dL/dq (the 2 of the flow-to-image scale); image voxels outside the
       // grid arrived as 0
-#pragma unroll
-      for (int dz = 0; dz < 2; ++dz)
-#pragma unroll
-        for (int dy = 0; dy < 2; ++dy)
-#pragma unroll
-          for (int dx = 0; dx < 2; ++dx) {
-            const float3 q = g[dz][dy][dx];
-            const float gx = 0.5f * q.x, gy = 0.5f * q.y, gz = 0.5f * q.z;
-            const float pz = (float)(2 * mz + dz), py = (float)(2 * my + dy), px = (float)(2 * mx + dx);
-            float* r = racc;
-            r[0] += gx, r[1 % (RIGID ? 12 : 1)] += gy, r[2 % (RIGID ? 12 : 1)] += gz;
-            if (RIGID) {
-              r[3] += gx * pz, r[4] += gx * py, r[5] += gx * px;
-              r[6] += gy * pz, r[7] += gy * py, r[8] += gy * px;
-              r[9] += gz * pz, r[10] += gz * py, r[11] += gz * px;
-            }
-          }
+      rigid_sums(g, mz, my, mx, racc);
     }
     // transpose along W (neighbouring lanes), as in k_warp_bwd2
     float hx[2][2][3];
