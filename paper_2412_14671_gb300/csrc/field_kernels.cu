@@ -436,11 +436,11 @@ __global__ void k_add(const __grid_constant__ AddTab t, int V) {
   a.dst[v] = f4add(a.dst[v], a.src[v]);
 }
 
-// The CTA's sums of three per-thread values, written to out[0..2] by thread 0: float-float
-// sums within each warp, then the warp sums in double.
-__device__ __forceinline__ void block_sum3(float a, float b, float c, double* out) {
+// The CTA's sums of three per-thread float-float values, written to out[0..2] by threads 0..2:
+// float-float sums within each warp, then the warp sums in double.
+__device__ __forceinline__ void block_sum3(FF a, FF b, FF c, double* out) {
   __shared__ float sh[3][2][kThreads / 32];
-  const FF s[3] = {warp_sum_ff(FF{a, 0.f}), warp_sum_ff(FF{b, 0.f}), warp_sum_ff(FF{c, 0.f})};
+  const FF s[3] = {warp_sum_ff(a), warp_sum_ff(b), warp_sum_ff(c)};
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   if (l == 0)
     for (int k = 0; k < 3; ++k) {
@@ -448,28 +448,34 @@ __device__ __forceinline__ void block_sum3(float a, float b, float c, double* ou
       sh[k][1][w] = s[k].lo;
     }
   __syncthreads();
-  if (threadIdx.x == 0)
-    for (int k = 0; k < 3; ++k) {
-      double r = 0.0;
-      for (int i = 0; i < kThreads / 32; ++i) r += (double)sh[k][0][i] + (double)sh[k][1][i];
-      out[k] = r;
-    }
+  if (threadIdx.x < 3) {
+    const int k = threadIdx.x;
+    double r = 0.0;
+    for (int i = 0; i < kThreads / 32; ++i) r += (double)sh[k][0][i] + (double)sh[k][1][i];
+    out[k] = r;
+  }
 }
 
 // ---- Eq. reg_ss / the L2 term / Eq. reg_ts (means over the flow grid) and the
 // total gradient dL/dphi = (G0+ - G0-) / 2^K + dL_reg/dphi.
 // With fx.ain (deterministic mode) G0 is completed with its fixed-point sums, which are cleared.
 // CLEAR: G0 read through G0clr (the same buffer) and cleared after the read (see
-// k_squaring_bwd's Gclr)
+// k_squaring_bwd's Gclr).
+// A CTA takes kRegRuns runs of 256 voxels: its three sums (float-float shuffle trees, then double) cost
+// about as much as a voxel's whole gradient, so several voxels per thread share them. 9 fields of
+// 80 x 96 x 80: 104 us; one voxel per thread and one thread for the double sums took 157 us.
+constexpr int kRegRuns = 4;
 template <bool CLEAR>
 __global__ void k_reg_grad(const float4* __restrict__ th, const float4* __restrict__ G0,
                            float4* __restrict__ grad, double* __restrict__ part, Dims n, RegArgs a, FxArgs fx,
                            float4* G0clr) {
-  const int v = blockIdx.x * blockDim.x + threadIdx.x;
   const int V = (int)vox(n);
   const int f = blockIdx.y, F = a.n_fields;
-  float lss = 0.f, ll2 = 0.f, lts = 0.f;
-  if (v < V) {
+  FF sss{0.f, 0.f}, sl2{0.f, 0.f}, sts{0.f, 0.f};
+  for (int run = 0; run < kRegRuns; ++run) {
+    const int v = (blockIdx.x * kRegRuns + run) * blockDim.x + threadIdx.x;
+    if (v >= V) break;
+    float lss = 0.f, ll2 = 0.f, lts = 0.f;
     const float4* T = th + (size_t)f * V;
     int z, y, x;
     unflat(n, v, z, y, x);
@@ -522,9 +528,12 @@ __global__ void k_reg_grad(const float4* __restrict__ th, const float4* __restri
       clear_fx(fx.ain + (size_t)2 * f * V, V, v);
       clear_fx(fx.ain + (size_t)2 * (F + f) * V, V, v);
     }
+    sss = ff_add(sss, FF{lss, 0.f});
+    sl2 = ff_add(sl2, FF{ll2, 0.f});
+    sts = ff_add(sts, FF{lts, 0.f});
   }
   const size_t b = (size_t)blockIdx.y * gridDim.x + blockIdx.x;
-  block_sum3(lss, ll2, lts, part + 3 * b);
+  block_sum3(sss, sl2, sts, part + 3 * b);
 }
 
 // ---- Adam (PyTorch update rule) or SGD with the per-step schedule
@@ -690,10 +699,10 @@ void launch_add(const AddDesc* d, int n, Dims dims, cudaStream_t s) {
     k_add<<<dim3(blocks_for(vox(dims)), cnt), kThreads, 0, s>>>(t, (int)vox(dims));
   }
 }
-int reg_blocks(Dims n) { return (int)blocks_for(vox(n)); }
+int reg_blocks(Dims n) { return (int)((vox(n) + kRegRuns * kThreads - 1) / (kRegRuns * kThreads)); }
 void launch_reg_grad(const float4* theta, const float4* G0, float4* grad, double* partials, Dims n,
                      const RegArgs& a, const FxArgs* fx, cudaStream_t s, bool clear_g0) {
-  const dim3 g(blocks_for(vox(n)), a.n_fields);
+  const dim3 g(reg_blocks(n), a.n_fields);
   if (clear_g0 && G0)
     k_reg_grad<true><<<g, kThreads, 0, s>>>(theta, G0, grad, partials, n, a, fx ? *fx : FxArgs{},
                                              const_cast<float4*>(G0));
