@@ -1054,6 +1054,7 @@ int create_impl(const int64_t shape[3], int n_sessions, const double spacing[3],
   {
     cudaError_t e = prepare_kernels();
     if (e == cudaSuccess) e = prepare_warp_kernels();
+    if (e == cudaSuccess) e = prepare_field_kernels();
     if (e != cudaSuccess) {
       muster_destroy(ctx);
       return fail(nullptr, MUSTER_ECUDA, std::string("kernel attributes: ") + cudaGetErrorString(e));

@@ -11,6 +11,7 @@
 // fields/chains; the deterministic scatter adjoints take 16 x 16 voxel tiles of a plane (or
 // of a pair of planes) in x and y, and planes x fields/chains in z.
 #include <algorithm>
+#include <mutex>
 
 #include "kernels.h"
 
@@ -403,30 +404,95 @@ __global__ void k_compose_bwd_dz(const __grid_constant__ ComposeBwdTab t, Dims n
 
 // ---- Appendix Gaussian Smoothing along one axis: circular convolution of every field with
 // the taps (inverse DFT of the Gaussian response, symmetric: taps[d] = taps[m - d]) over
-// the offsets lo..hi (either the whole circle or the taps above FP32 resolution)
+// the offsets lo..hi (either the whole circle or the taps above FP32 resolution).
+// A thread computes kSO neighbouring outputs along the axis and walks their nodes downwards, so a
+// node loaded once serves kSO outputs, each of which adds its offsets in ascending order. Along D
+// and H the lanes lie along W. Along W they lie along rows, staged in shared memory with an odd
+// pitch (no bank conflicts), and the results leave through the same buffer. FMAs bound the whole
+// circle (64 taps), DRAM short ranges. 5 fields of 64^3 with 64 taps: 32 us an axis; one output per
+// thread with a load, a wrap test and a tap look-up per offset took 62 us.
+constexpr int kSO = 8;
+constexpr int kStagedTaps = 4096;  // more taps (an axis of that many nodes) are read from memory
+// outputs p0 .. p0 + kSO - 1 from at(q), the node of position q (0 <= q < m), and tap(d), the tap of offset d
+template <class Tap, class At>
+__device__ __forceinline__ void smooth_run(float4 (&acc)[kSO], int p0, int m, int lo, int hi, Tap tap, At at) {
+  float t[kSO];  // taps of the node under way for every output: offset p0 + j - q
+#pragma unroll
+  for (int j = 0; j < kSO; ++j) acc[j] = make_float4(0.f, 0.f, 0.f, 0.f), t[j] = 0.f;
+  int q = p0 + kSO - 1 - lo;  // position of the node under way, wrapped into the grid
+  while (q >= m) q -= m;
+  for (int d = lo - (kSO - 1); d <= hi; ++d) {  // d: offset of output 0
+#pragma unroll
+    for (int j = 0; j < kSO - 1; ++j) t[j] = t[j + 1];
+    t[kSO - 1] = d + kSO - 1 <= hi ? tap(d + kSO - 1) : 0.f;
+    const float4 s = at(q);
+    if (d >= lo && d + kSO - 1 <= hi) {
+#pragma unroll
+      for (int j = 0; j < kSO; ++j) {
+        acc[j].x = fmaf(t[j], s.x, acc[j].x);
+        acc[j].y = fmaf(t[j], s.y, acc[j].y);
+        acc[j].z = fmaf(t[j], s.z, acc[j].z);
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < kSO; ++j)
+        if (d + j >= lo && d + j <= hi) {
+          acc[j].x = fmaf(t[j], s.x, acc[j].x);
+          acc[j].y = fmaf(t[j], s.y, acc[j].y);
+          acc[j].z = fmaf(t[j], s.z, acc[j].z);
+        }
+    }
+    q = q == 0 ? m - 1 : q - 1;
+  }
+}
+__device__ __forceinline__ void load_taps(float* w, const float* __restrict__ taps, int m, int lo, int hi) {
+  for (int d = lo + (int)threadIdx.x; d <= hi; d += blockDim.x) w[d - lo] = __ldg(taps + (d < 0 ? d + m : d));
+}
+// along axis 0 or 1: a thread per column of `inner` consecutive voxels and run of kSO positions
 __global__ void k_smooth_axis(const float4* __restrict__ in, float4* __restrict__ out, Dims n, int axis,
                               const float* __restrict__ taps, int lo, int hi) {
-  const int v = blockIdx.x * blockDim.x + threadIdx.x;
-  const int V = (int)vox(n);
-  if (v >= V) return;
-  const size_t off = (size_t)blockIdx.y * V;
-  int z, y, x;
-  unflat(n, v, z, y, x);
-  const int p = axis == 0 ? z : (axis == 1 ? y : x);
-  const int m = axis == 0 ? n.n0 : (axis == 1 ? n.n1 : n.n2);
-  const int stride = axis == 0 ? n.n1 * n.n2 : (axis == 1 ? n.n2 : 1);
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int d = lo; d <= hi; ++d) {
-    int q = p - d;
-    if (q < 0) q += m;
-    if (q >= m) q -= m;
-    const float w = __ldg(taps + (d < 0 ? d + m : d));
-    const float4 a = __ldg(in + off + v + (q - p) * stride);
-    acc.x = fmaf(w, a.x, acc.x);
-    acc.y = fmaf(w, a.y, acc.y);
-    acc.z = fmaf(w, a.z, acc.z);
+  extern __shared__ float w[];  // taps of the offsets lo .. hi
+  const int m = axis == 0 ? n.n0 : n.n1, inner = axis == 0 ? n.n1 * n.n2 : n.n2;
+  const bool staged = hi - lo < kStagedTaps;
+  if (staged) load_taps(w, taps, m, lo, hi);
+  __syncthreads();
+  const int runs = (m + kSO - 1) / kSO, outer = axis == 0 ? 1 : n.n0;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= inner * runs * outer) return;
+  const int c = i % inner, r = i / inner, p0 = r % runs * kSO, o = r / runs;
+  const size_t base = (size_t)blockIdx.y * vox(n) + (size_t)o * m * inner + c;
+  float4 acc[kSO];
+  smooth_run(
+      acc, p0, m, lo, hi, [&](int d) { return staged ? w[d - lo] : __ldg(taps + (d < 0 ? d + m : d)); },
+      [&](int q) { return __ldg(in + base + (size_t)q * inner); });
+#pragma unroll
+  for (int j = 0; j < kSO; ++j)
+    if (p0 + j < m) out[base + (size_t)(p0 + j) * inner] = acc[j];
+}
+// along axis 2: a CTA per kSR rows
+constexpr int kSR = 32, kSmoothRow = 256;  // rows per CTA, longest staged row (132 KB)
+__global__ void __launch_bounds__(kSR * kSmoothRow / kSO) k_smooth_rows(const float4* __restrict__ in, float4* __restrict__ out, Dims n,
+                              const float* __restrict__ taps, int lo, int hi, int pitch) {
+  extern __shared__ float4 row[];  // [kSR][pitch], then the taps
+  const int m = n.n2, rows = n.n0 * n.n1, r0 = blockIdx.x * kSR, nr = min(kSR, rows - r0);
+  float* w = reinterpret_cast<float*>(row + kSR * pitch);
+  load_taps(w, taps, m, lo, hi);
+  const size_t base = (size_t)blockIdx.y * vox(n) + (size_t)r0 * m;
+  for (int i = threadIdx.x; i < nr * m; i += blockDim.x) row[i / m * pitch + i % m] = __ldg(in + base + i);
+  __syncthreads();
+  const int r = threadIdx.x % kSR, p0 = threadIdx.x / kSR * kSO;  // one run per thread
+  float4* mine = row + r * pitch;
+  float4 acc[kSO];
+  if (r < nr)
+    smooth_run(acc, p0, m, lo, hi, [&](int d) { return w[d - lo]; }, [&](int q) { return mine[q]; });
+  __syncthreads();
+  if (r < nr) {
+#pragma unroll
+    for (int j = 0; j < kSO; ++j)
+      if (p0 + j < m) mine[p0 + j] = acc[j];
   }
-  out[off + v] = acc;
+  __syncthreads();
+  for (int i = threadIdx.x; i < nr * m; i += blockDim.x) out[base + i] = row[i / m * pitch + i % m];
 }
 
 __global__ void k_add(const __grid_constant__ AddTab t, int V) {
@@ -709,12 +775,39 @@ void launch_reg_grad(const float4* theta, const float4* G0, float4* grad, double
   else
     k_reg_grad<false><<<g, kThreads, 0, s>>>(theta, G0, grad, partials, n, a, fx ? *fx : FxArgs{}, nullptr);
 }
+cudaError_t prepare_field_kernels() {
+  static std::mutex mu;
+  static bool done[kMaxDevices] = {};
+  return once_per_device(done, mu, [] {
+    return cudaFuncSetAttribute(k_smooth_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)(sizeof(float4) * kSR * (kSmoothRow | 1) + sizeof(float) * kSmoothRow));
+  });
+}
 void launch_smooth(const float4* in, float4* out, float4* tmp_a, float4* tmp_b, int n_fields, Dims n,
                    const SmoothAxis axes[3], cudaStream_t s) {
-  const dim3 g(blocks_for(vox(n)), n_fields);
-  k_smooth_axis<<<g, kThreads, 0, s>>>(in, tmp_a, n, 0, axes[0].taps, axes[0].lo, axes[0].hi);
-  k_smooth_axis<<<g, kThreads, 0, s>>>(tmp_a, tmp_b, n, 1, axes[1].taps, axes[1].lo, axes[1].hi);
-  k_smooth_axis<<<g, kThreads, 0, s>>>(tmp_b, out, n, 2, axes[2].taps, axes[2].lo, axes[2].hi);
+  auto tap_bytes = [&](int a) { return sizeof(float) * (size_t)std::min(axes[a].hi - axes[a].lo + 1, kStagedTaps); };
+  auto strided = [&](int a, const float4* src, float4* dst) {
+    const int m = a == 0 ? n.n0 : n.n1;
+    const size_t threads = vox(n) / m * ((m + kSO - 1) / kSO);
+    k_smooth_axis<<<dim3(blocks_for(threads), n_fields), kThreads, tap_bytes(a), s>>>(src, dst, n, a, axes[a].taps,
+                                                                                      axes[a].lo, axes[a].hi);
+  };
+  strided(0, in, tmp_a);
+  strided(1, tmp_a, tmp_b);
+  // rows of up to kSmoothRow nodes fit the staged kernel (32 threads per run); longer ones take the
+  // strided kernel on a grid whose axis 1 is axis 2 of n, with lanes along the axis
+  const int pitch = n.n2 | 1, threads = kSR * ((n.n2 + kSO - 1) / kSO);
+  if (n.n2 <= kSmoothRow) {
+    const size_t rows = (size_t)n.n0 * n.n1;
+    k_smooth_rows<<<dim3((unsigned)((rows + kSR - 1) / kSR), n_fields), threads,
+                    sizeof(float4) * kSR * pitch + tap_bytes(2), s>>>(tmp_b, out, n, axes[2].taps, axes[2].lo, axes[2].hi,
+                                                                     pitch);
+  } else {
+    const Dims flat{n.n0 * n.n1, n.n2, 1};
+    const size_t runs = (size_t)flat.n0 * ((n.n2 + kSO - 1) / kSO);
+    k_smooth_axis<<<dim3(blocks_for(runs), n_fields), kThreads, tap_bytes(2), s>>>(tmp_b, out, flat, 1, axes[2].taps,
+                                                                                   axes[2].lo, axes[2].hi);
+  }
 }
 void launch_adam(float4* theta, float4* m, float4* v, const float4* grad, size_t count, const float* sched,
                  const int* step, int sgd, float beta1, float beta2, float eps, cudaStream_t s) {

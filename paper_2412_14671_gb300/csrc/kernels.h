@@ -210,6 +210,7 @@ struct SmoothAxis {
   const float* taps;  // m taps of the axis (device), symmetric
   int lo, hi;         // offsets summed: lo..hi
 };
+cudaError_t prepare_field_kernels();  // dynamic shared memory limit, once per device
 void launch_smooth(const float4* in, float4* out, float4* tmp_a, float4* tmp_b, int n_fields, Dims n,
                    const SmoothAxis axes[3], cudaStream_t s);
 // metrics_kernels.cu: det(I + grad u) of a planar displacement, and the deformation
