@@ -38,9 +38,10 @@ __device__ __forceinline__ float dstep(float lo, float mid, float hi, int p, int
 // of 4 and the fields are 16-byte aligned, else 1) and walks a chunk of D with the planes z-1, z, z+1 of
 // the three components in registers. The rows y-1 and y+1 of plane z are loads that hit the L1 or
 // L2 lines of the neighbouring threads' own rows; x-1 and x+NX come from the neighbouring lanes, or
-// from memory at a row's or warp's end. DRAM bounds it (16 bytes per voxel); the walk is short, so
-// that every SM has loads of some 1400 threads in flight. 160 x 192 x 160: @JACT@ us; staging
-// every plane of a 32 x 8 tile in shared memory behind two barriers took 39 us.
+// from memory at a row's or warp's end. DRAM is the floor (16 bytes per voxel, 12 us at 160 x 192 x 160);
+// the latency of a plane's nine loads per thread bounds it, so 3 CTAs of 80 registers share an SM and
+// the walk is short. 160 x 192 x 160: 28 us; with 2 CTAs per SM 36 us, with runs of 2 voxels 29 us, of 1 47 us;
+// staging every plane of a 32 x 8 tile in shared memory behind two barriers took 39 us.
 template <int NX>
 struct Run {
   float v[NX];
@@ -57,8 +58,8 @@ __device__ __forceinline__ Run<NX> load_run(const float* __restrict__ p) {
   return r;
 }
 template <int NX>
-__global__ void __launch_bounds__(kJT) k_jacobian_det(const float* __restrict__ u, Dims n, float* __restrict__ J,
-                                                      int zchunk) {
+__global__ void __launch_bounds__(kJT, 3) k_jacobian_det(const float* __restrict__ u, Dims n,
+                                                         float* __restrict__ J, int zchunk) {
   const int runs = n.n2 / NX, i = blockIdx.x * kJT + threadIdx.x, lane = threadIdx.x & 31;
   const bool in = i < runs * n.n1;
   const int y = in ? i / runs : 0, x = in ? (i - y * runs) * NX : 0;
@@ -329,10 +330,10 @@ __global__ void __launch_bounds__(kMT) k_metrics_final(const double* __restrict_
 
 void launch_jacobian_det(const float* u, Dims n, float* J, cudaStream_t s) {
   const bool four = n.n2 % 4 == 0 && (reinterpret_cast<uintptr_t>(u) & 15) == 0 && (reinterpret_cast<uintptr_t>(J) & 15) == 0;
-  // D chunks so that the grid has at least 5 CTAs per SM of the device
+  // D chunks so that the grid has at least 8 CTAs per SM of the device (5: 30 us, 8 to 30: 28 us)
   const size_t runs = (size_t)n.n1 * (four ? n.n2 / 4 : n.n2);
   const unsigned gx = (unsigned)((runs + kJT - 1) / kJT);
-  const long want = 5L * device_sm_count();
+  const long want = 8L * device_sm_count();
   int zc = n.n0;
   while (zc > 4 && (long)gx * ((n.n0 + zc - 1) / zc) < want) zc = (zc + 1) / 2;
   const dim3 g(gx, (n.n0 + zc - 1) / zc);
