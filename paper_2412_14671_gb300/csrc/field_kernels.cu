@@ -24,6 +24,7 @@ __host__ __device__ inline unsigned blocks_for(size_t V) { return (unsigned)((V 
 
 // ---- Sec. Implementation Details: velocity initialised from the previous stage
 __global__ void k_prolong(const float4* __restrict__ coarse, Dims nc, float4* __restrict__ fine, Dims nf) {
+  grid_begin();
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
   const size_t Vf = vox(nf);
   if (v >= (int)Vf) return;
@@ -38,6 +39,7 @@ __global__ void k_prolong(const float4* __restrict__ coarse, Dims nc, float4* __
 // ---- Alg. 1, first line: u_0 = sign * phi / 2^K; fields [0, F) are +phi, [F, 2F) are -phi
 __global__ void k_exp_init(const float4* __restrict__ theta, float4* __restrict__ u0, int F, int V,
                            float scale, unsigned* __restrict__ zero) {
+  grid_begin();
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
   if (zero && v == 0 && blockIdx.y == 0) *zero = 0u;  // a per-step word the step's later kernels set
   if (v >= V) return;
@@ -54,6 +56,7 @@ __global__ void k_exp_init(const float4* __restrict__ theta, float4* __restrict_
 // ---- Alg. 1, loop body in displacement form: u(x) <- u(x) + S[u](x + u(x))
 template <int NF>
 __global__ void k_squaring(const float4* __restrict__ u, float4* __restrict__ un, Dims n, int count) {
+  grid_begin();
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
   const int V = (int)vox(n);
   if (v >= V) return;
@@ -76,6 +79,7 @@ __global__ void k_squaring(const float4* __restrict__ u, float4* __restrict__ un
 
 // one field, its squared map written planar (the end of a stateless exponential)
 __global__ void k_squaring_planar(const float4* __restrict__ u, float* __restrict__ un, Dims n) {
+  grid_begin();
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
   const int V = (int)vox(n);
   if (v >= V) return;
@@ -95,6 +99,7 @@ __global__ void k_squaring_planar(const float4* __restrict__ u, float* __restric
 template <int NF>
 __global__ void k_squaring_first(const float4* __restrict__ th, float4* __restrict__ u0, float4* __restrict__ u1,
                                  Dims n, int count, int F, float scale, unsigned* __restrict__ zero) {
+  grid_begin();
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
   if (zero && v == 0 && blockIdx.y == 0) *zero = 0u;  // a per-step word the step's later kernels set
   const int V = (int)vox(n);
@@ -176,6 +181,7 @@ template <bool FX, int NF, bool CLEAR = false>
 __global__ void k_squaring_bwd(const float4* __restrict__ u, const float4* __restrict__ Gin,
                                float4* __restrict__ Gout, Dims n, int count, FxArgs fx,
                                const __grid_constant__ PairGradTab pg, float4* Gclr) {
+  grid_begin();
   const Place p = place<FX>(n);
   const int x = p.x, y = p.y, z = p.z, v = p.v, grp = p.grp;
   const bool vin = p.vin;
@@ -230,6 +236,7 @@ __global__ void k_squaring_bwd(const float4* __restrict__ u, const float4* __res
 // corners are merged along D as well as along W and H before their fixed-point reductions
 __global__ void k_squaring_bwd_dz(const float4* __restrict__ u, const float4* __restrict__ Gin, Dims n, FxArgs fx,
                                   const __grid_constant__ PairGradTab pg) {
+  grid_begin();
   const int nzp = (n.n0 + 1) / 2;
   const int zp = blockIdx.z % nzp, f = blockIdx.z / nzp;
   const Tile2 tl = tile2();
@@ -284,6 +291,7 @@ __global__ void k_squaring_bwd_dz(const float4* __restrict__ u, const float4* __
 // ---- Eq. cum_deformation: U_new(x) = U_prev(x) + S[u](x + U_prev(x))
 template <int NF>
 __global__ void __launch_bounds__(kThreads, 8) k_compose(const __grid_constant__ ComposeTab t, Dims n, int count) {
+  grid_begin();
   const ComposeDesc* d = t.d;
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= (int)vox(n)) return;
@@ -309,6 +317,7 @@ __global__ void __launch_bounds__(kThreads, 8) k_compose(const __grid_constant__
 template <bool FX, int NF>
 __global__ void __launch_bounds__(kThreads, 4)
     k_compose_bwd(const __grid_constant__ ComposeBwdTab t, Dims n, int count, FxArgs fx) {
+  grid_begin();
   const ComposeBwdDesc* d = t.d;
   const Place p = place<FX>(n);
   const int x = p.x, y = p.y, z = p.z, v = p.v, grp = p.grp;
@@ -356,6 +365,7 @@ __global__ void __launch_bounds__(kThreads, 4)
 // ---- the deterministic composition adjoint with two voxels of one column per lane (planes
 // 2 zp and 2 zp + 1 of one chain; grid z = planes / 2 x chains), merged along D as well
 __global__ void k_compose_bwd_dz(const __grid_constant__ ComposeBwdTab t, Dims n, FxArgs fx) {
+  grid_begin();
   const int nzp = (n.n0 + 1) / 2;
   const int zp = blockIdx.z % nzp, ci = blockIdx.z / nzp;
   const ComposeBwdDesc c = t.d[ci];
@@ -451,6 +461,7 @@ __device__ __forceinline__ void load_taps(float* w, const float* __restrict__ ta
 // along axis 0 or 1: a thread per column of `inner` consecutive voxels and run of kSO positions
 __global__ void k_smooth_axis(const float4* __restrict__ in, float4* __restrict__ out, Dims n, int axis,
                               const float* __restrict__ taps, int lo, int hi) {
+  grid_begin();
   extern __shared__ float w[];  // taps of the offsets lo .. hi
   const int m = axis == 0 ? n.n0 : n.n1, inner = axis == 0 ? n.n1 * n.n2 : n.n2;
   const bool staged = hi - lo < kStagedTaps;
@@ -473,6 +484,7 @@ __global__ void k_smooth_axis(const float4* __restrict__ in, float4* __restrict_
 constexpr int kSR = 32, kSmoothRow = 256;  // rows per CTA, longest staged row (132 KB)
 __global__ void __launch_bounds__(kSR * kSmoothRow / kSO) k_smooth_rows(const float4* __restrict__ in, float4* __restrict__ out, Dims n,
                               const float* __restrict__ taps, int lo, int hi, int pitch) {
+  grid_begin();
   extern __shared__ float4 row[];  // [kSR][pitch], then the taps
   const int m = n.n2, rows = n.n0 * n.n1, r0 = blockIdx.x * kSR, nr = min(kSR, rows - r0);
   float* w = reinterpret_cast<float*>(row + kSR * pitch);
@@ -496,6 +508,7 @@ __global__ void __launch_bounds__(kSR * kSmoothRow / kSO) k_smooth_rows(const fl
 }
 
 __global__ void k_add(const __grid_constant__ AddTab t, int V) {
+  grid_begin();
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= V) return;
   const AddDesc a = t.d[blockIdx.y];
@@ -535,6 +548,7 @@ template <bool CLEAR>
 __global__ void k_reg_grad(const float4* __restrict__ th, const float4* __restrict__ G0,
                            float4* __restrict__ grad, double* __restrict__ part, Dims n, RegArgs a, FxArgs fx,
                            float4* G0clr) {
+  grid_begin();
   const int V = (int)vox(n);
   const int f = blockIdx.y, F = a.n_fields;
   FF sss{0.f, 0.f}, sl2{0.f, 0.f}, sts{0.f, 0.f};
@@ -607,6 +621,7 @@ __global__ void k_reg_grad(const float4* __restrict__ th, const float4* __restri
 __global__ void k_adam(float4* __restrict__ th, float4* __restrict__ m, float4* __restrict__ v,
                        const float4* __restrict__ g, size_t count, const float* __restrict__ sched,
                        const int* __restrict__ step, int sgd, float b1, float b2, float eps) {
+  grid_begin();
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   const int s = *step;
@@ -633,6 +648,7 @@ __global__ void k_adam(float4* __restrict__ th, float4* __restrict__ m, float4* 
 }
 
 __global__ void k_f4_to_planar(const float4* __restrict__ in, float* __restrict__ out, size_t V) {
+  grid_begin();
   const size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= V) return;
   const size_t f = blockIdx.y;
@@ -643,6 +659,7 @@ __global__ void k_f4_to_planar(const float4* __restrict__ in, float* __restrict_
 }
 
 __global__ void k_planar_to_f4(const float* __restrict__ in, float4* __restrict__ out, size_t V, float scale) {
+  grid_begin();
   const size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= V) return;
   const size_t f = blockIdx.y;
@@ -652,11 +669,11 @@ __global__ void k_planar_to_f4(const float* __restrict__ in, float4* __restrict_
 }  // namespace
 
 void launch_prolong(const float4* coarse, Dims nc, float4* fine, Dims nf, int n_fields, cudaStream_t s) {
-  k_prolong<<<dim3(blocks_for(vox(nf)), n_fields), kThreads, 0, s>>>(coarse, nc, fine, nf);
+  launch(k_prolong, dim3(blocks_for(vox(nf)), n_fields), kThreads, 0, s)(coarse, nc, fine, nf);
 }
 void launch_exp_init(const float4* theta, float4* u0, int n_fields, Dims n, float scale, cudaStream_t s,
                      unsigned* zero) {
-  k_exp_init<<<dim3(blocks_for(vox(n)), 2 * n_fields), kThreads, 0, s>>>(theta, u0, n_fields, (int)vox(n), scale,
+  launch(k_exp_init, dim3(blocks_for(vox(n)), 2 * n_fields), kThreads, 0, s)(theta, u0, n_fields, (int)vox(n), scale,
                                                                           zero);
 }
 // fields (or chains) per thread of the flow-grid gather kernels: 1 or 2 (the launch
@@ -666,20 +683,20 @@ unsigned groups(int count, int nf) { return (unsigned)((count + nf - 1) / nf); }
 void launch_squaring(const float4* u, float4* un, int n_fields2, Dims n, cudaStream_t s, int nf) {
   const dim3 g(blocks_for(vox(n)), groups(n_fields2, nf));
   if (nf == 1)
-    k_squaring<1><<<g, kThreads, 0, s>>>(u, un, n, n_fields2);
+    launch(k_squaring<1>, g, kThreads, 0, s)(u, un, n, n_fields2);
   else
-    k_squaring<2><<<g, kThreads, 0, s>>>(u, un, n, n_fields2);
+    launch(k_squaring<2>, g, kThreads, 0, s)(u, un, n, n_fields2);
 }
 void launch_squaring_planar(const float4* u, float* un, Dims n, cudaStream_t s) {
-  k_squaring_planar<<<blocks_for(vox(n)), kThreads, 0, s>>>(u, un, n);
+  launch(k_squaring_planar, blocks_for(vox(n)), kThreads, 0, s)(u, un, n);
 }
 void launch_squaring_first(const float4* theta, float4* u0, float4* u1, int n_fields, Dims n, float scale,
                            cudaStream_t s, int nf, unsigned* zero) {
   const dim3 g(blocks_for(vox(n)), groups(2 * n_fields, nf));
   if (nf == 1)
-    k_squaring_first<1><<<g, kThreads, 0, s>>>(theta, u0, u1, n, 2 * n_fields, n_fields, scale, zero);
+    launch(k_squaring_first<1>, g, kThreads, 0, s)(theta, u0, u1, n, 2 * n_fields, n_fields, scale, zero);
   else
-    k_squaring_first<2><<<g, kThreads, 0, s>>>(theta, u0, u1, n, 2 * n_fields, n_fields, scale, zero);
+    launch(k_squaring_first<2>, g, kThreads, 0, s)(theta, u0, u1, n, 2 * n_fields, n_fields, scale, zero);
 }
 // grid of the 2-D layout: W tiles, H tiles, D planes x groups of fields
 dim3 grid2(Dims n, int count, int nf) {
@@ -689,13 +706,13 @@ template <int NF>
 void squaring_bwd_nf(const float4* u, const float4* Gin, float4* Gout, int n_fields2, Dims n, const FxArgs* fx,
                      const PairGradTab& pg, float4* Gclr, cudaStream_t s) {
   if (fx)
-    k_squaring_bwd<true, NF><<<grid2(n, n_fields2, NF), kThreads, 0, s>>>(u, Gin, Gout, n, n_fields2, *fx, pg,
+    launch(k_squaring_bwd<true, NF>, grid2(n, n_fields2, NF), kThreads, 0, s)(u, Gin, Gout, n, n_fields2, *fx, pg,
                                                                           nullptr);
   else if (Gclr)
-    k_squaring_bwd<false, NF, true><<<dim3(blocks_for(vox(n)), groups(n_fields2, NF)), kThreads, 0, s>>>(
+    launch(k_squaring_bwd<false, NF, true>, dim3(blocks_for(vox(n)), groups(n_fields2, NF)), kThreads, 0, s)(
         u, Gin, Gout, n, n_fields2, FxArgs{}, pg, Gclr);
   else
-    k_squaring_bwd<false, NF><<<dim3(blocks_for(vox(n)), groups(n_fields2, NF)), kThreads, 0, s>>>(
+    launch(k_squaring_bwd<false, NF>, dim3(blocks_for(vox(n)), groups(n_fields2, NF)), kThreads, 0, s)(
         u, Gin, Gout, n, n_fields2, FxArgs{}, pg, nullptr);
 }
 // the 2-D layout puts planes x field groups on grid z (at most 65535): one field per thread
@@ -714,7 +731,7 @@ void launch_squaring_bwd(const float4* u, const float4* Gin, float4* Gout, int n
   PairGradTab t{};
   if (pg && n_fields2 <= kMaxDescPerLaunch) t = *pg;
   if (fx && dz_fits(n, n_fields2)) {
-    k_squaring_bwd_dz<<<grid_dz(n, n_fields2), kThreads, 0, s>>>(u, Gin, n, *fx, t);
+    launch(k_squaring_bwd_dz, grid_dz(n, n_fields2), kThreads, 0, s)(u, Gin, n, *fx, t);
     return;
   }
   nf = fx_nf(fx, n, n_fields2, nf);
@@ -731,17 +748,17 @@ void launch_compose(const ComposeDesc* d, int n_chains, Dims n, cudaStream_t s, 
     for (int c = 0; c < cnt; ++c) t.d[c] = d[c0 + c];
     const dim3 g(blocks_for(vox(n)), groups(cnt, nf));
     if (nf == 1)
-      k_compose<1><<<g, kThreads, 0, s>>>(t, n, cnt);
+      launch(k_compose<1>, g, kThreads, 0, s)(t, n, cnt);
     else
-      k_compose<2><<<g, kThreads, 0, s>>>(t, n, cnt);
+      launch(k_compose<2>, g, kThreads, 0, s)(t, n, cnt);
   }
 }
 template <int NF>
 void compose_bwd_nf(const ComposeBwdTab& t, int n_chains, Dims n, const FxArgs* fx, cudaStream_t s) {
   if (fx)
-    k_compose_bwd<true, NF><<<grid2(n, n_chains, NF), kThreads, 0, s>>>(t, n, n_chains, *fx);
+    launch(k_compose_bwd<true, NF>, grid2(n, n_chains, NF), kThreads, 0, s)(t, n, n_chains, *fx);
   else
-    k_compose_bwd<false, NF><<<dim3(blocks_for(vox(n)), groups(n_chains, NF)), kThreads, 0, s>>>(t, n, n_chains,
+    launch(k_compose_bwd<false, NF>, dim3(blocks_for(vox(n)), groups(n_chains, NF)), kThreads, 0, s)(t, n, n_chains,
                                                                                                FxArgs{});
 }
 void launch_compose_bwd(const ComposeBwdDesc* d, int n_chains, Dims n, const FxArgs* fx, cudaStream_t s, int nf) {
@@ -750,7 +767,7 @@ void launch_compose_bwd(const ComposeBwdDesc* d, int n_chains, Dims n, const FxA
     ComposeBwdTab t;
     for (int c = 0; c < cnt; ++c) t.d[c] = d[c0 + c];
     if (fx && dz_fits(n, cnt))
-      k_compose_bwd_dz<<<grid_dz(n, cnt), kThreads, 0, s>>>(t, n, *fx);
+      launch(k_compose_bwd_dz, grid_dz(n, cnt), kThreads, 0, s)(t, n, *fx);
     else if (fx_nf(fx, n, cnt, nf) == 1)
       compose_bwd_nf<1>(t, cnt, n, fx, s);
     else
@@ -762,7 +779,7 @@ void launch_add(const AddDesc* d, int n, Dims dims, cudaStream_t s) {
     const int cnt = std::min(kMaxDescPerLaunch, n - c0);
     AddTab t;
     for (int c = 0; c < cnt; ++c) t.d[c] = d[c0 + c];
-    k_add<<<dim3(blocks_for(vox(dims)), cnt), kThreads, 0, s>>>(t, (int)vox(dims));
+    launch(k_add, dim3(blocks_for(vox(dims)), cnt), kThreads, 0, s)(t, (int)vox(dims));
   }
 }
 int reg_blocks(Dims n) { return (int)((vox(n) + kRegRuns * kThreads - 1) / (kRegRuns * kThreads)); }
@@ -770,10 +787,10 @@ void launch_reg_grad(const float4* theta, const float4* G0, float4* grad, double
                      const RegArgs& a, const FxArgs* fx, cudaStream_t s, bool clear_g0) {
   const dim3 g(reg_blocks(n), a.n_fields);
   if (clear_g0 && G0)
-    k_reg_grad<true><<<g, kThreads, 0, s>>>(theta, G0, grad, partials, n, a, fx ? *fx : FxArgs{},
+    launch(k_reg_grad<true>, g, kThreads, 0, s)(theta, G0, grad, partials, n, a, fx ? *fx : FxArgs{},
                                              const_cast<float4*>(G0));
   else
-    k_reg_grad<false><<<g, kThreads, 0, s>>>(theta, G0, grad, partials, n, a, fx ? *fx : FxArgs{}, nullptr);
+    launch(k_reg_grad<false>, g, kThreads, 0, s)(theta, G0, grad, partials, n, a, fx ? *fx : FxArgs{}, nullptr);
 }
 cudaError_t prepare_field_kernels() {
   static std::mutex mu;
@@ -789,7 +806,7 @@ void launch_smooth(const float4* in, float4* out, float4* tmp_a, float4* tmp_b, 
   auto strided = [&](int a, const float4* src, float4* dst) {
     const int m = a == 0 ? n.n0 : n.n1;
     const size_t threads = vox(n) / m * ((m + kSO - 1) / kSO);
-    k_smooth_axis<<<dim3(blocks_for(threads), n_fields), kThreads, tap_bytes(a), s>>>(src, dst, n, a, axes[a].taps,
+    launch(k_smooth_axis, dim3(blocks_for(threads), n_fields), kThreads, tap_bytes(a), s)(src, dst, n, a, axes[a].taps,
                                                                                       axes[a].lo, axes[a].hi);
   };
   strided(0, in, tmp_a);
@@ -799,25 +816,25 @@ void launch_smooth(const float4* in, float4* out, float4* tmp_a, float4* tmp_b, 
   const int pitch = n.n2 | 1, threads = kSR * ((n.n2 + kSO - 1) / kSO);
   if (n.n2 <= kSmoothRow) {
     const size_t rows = (size_t)n.n0 * n.n1;
-    k_smooth_rows<<<dim3((unsigned)((rows + kSR - 1) / kSR), n_fields), threads,
-                    sizeof(float4) * kSR * pitch + tap_bytes(2), s>>>(tmp_b, out, n, axes[2].taps, axes[2].lo, axes[2].hi,
-                                                                     pitch);
+    const size_t bytes = sizeof(float4) * kSR * pitch + tap_bytes(2);
+    launch(k_smooth_rows, dim3((unsigned)((rows + kSR - 1) / kSR), n_fields), threads, bytes, s)(
+        tmp_b, out, n, axes[2].taps, axes[2].lo, axes[2].hi, pitch);
   } else {
     const Dims flat{n.n0 * n.n1, n.n2, 1};
     const size_t runs = (size_t)flat.n0 * ((n.n2 + kSO - 1) / kSO);
-    k_smooth_axis<<<dim3(blocks_for(runs), n_fields), kThreads, tap_bytes(2), s>>>(tmp_b, out, flat, 1, axes[2].taps,
+    launch(k_smooth_axis, dim3(blocks_for(runs), n_fields), kThreads, tap_bytes(2), s)(tmp_b, out, flat, 1, axes[2].taps,
                                                                                    axes[2].lo, axes[2].hi);
   }
 }
 void launch_adam(float4* theta, float4* m, float4* v, const float4* grad, size_t count, const float* sched,
                  const int* step, int sgd, float beta1, float beta2, float eps, cudaStream_t s) {
-  k_adam<<<blocks_for(count), kThreads, 0, s>>>(theta, m, v, grad, count, sched, step, sgd, beta1, beta2, eps);
+  launch(k_adam, blocks_for(count), kThreads, 0, s)(theta, m, v, grad, count, sched, step, sgd, beta1, beta2, eps);
 }
 void launch_f4_to_planar(const float4* in, float* out, int n_fields, size_t V, cudaStream_t s) {
-  k_f4_to_planar<<<dim3(blocks_for(V), n_fields), kThreads, 0, s>>>(in, out, V);
+  launch(k_f4_to_planar, dim3(blocks_for(V), n_fields), kThreads, 0, s)(in, out, V);
 }
 void launch_planar_to_f4(const float* in, float4* out, int n_fields, size_t V, cudaStream_t s, float scale) {
-  k_planar_to_f4<<<dim3(blocks_for(V), n_fields), kThreads, 0, s>>>(in, out, V, scale);
+  launch(k_planar_to_f4, dim3(blocks_for(V), n_fields), kThreads, 0, s)(in, out, V, scale);
 }
 
 }  // namespace muster

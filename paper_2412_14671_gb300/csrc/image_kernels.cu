@@ -16,6 +16,7 @@ __host__ __device__ inline unsigned blocks_for(size_t V) { return (unsigned)((V 
 
 // ---- pyramid: 2x2x2 mean, last plane replicated for odd sizes
 __global__ void k_down2(const float* __restrict__ in, Dims n, float* __restrict__ out, Dims m) {
+  grid_begin();
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
   const int Vm = (int)vox(m);
   if (v >= Vm) return;
@@ -34,6 +35,7 @@ __global__ void k_down2(const float* __restrict__ in, Dims n, float* __restrict_
 __device__ __forceinline__ float centre(int p) { return 0.5f * (float)p - 0.25f; }
 
 __global__ void k_upsample_disp(const float4* __restrict__ U, Dims nf, Dims ni, float* __restrict__ out) {
+  grid_begin();
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
   const int Vi = (int)vox(ni);
   if (v >= Vi) return;
@@ -46,6 +48,7 @@ __global__ void k_upsample_disp(const float4* __restrict__ U, Dims nf, Dims ni, 
 }
 
 __global__ void k_count_nonfinite(const float* __restrict__ x, size_t n, int* __restrict__ count) {
+  grid_begin();
   int bad = 0;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
     bad += isfinite(x[i]) ? 0 : 1;
@@ -59,6 +62,7 @@ __global__ void k_loss_reduce(const double* __restrict__ sp, int nsp, const doub
                               double inv_NR, double inv_F, double inv_Nm2, float ass, float al2, float ats,
                               double* __restrict__ out, double* __restrict__ hist, int* __restrict__ step,
                               int* __restrict__ flag, int advance) {
+  grid_begin();
   __shared__ double sh[4][kThreads];
   double a = 0.0, b = 0.0, c = 0.0, e = 0.0;
   for (int i = threadIdx.x; i < nsp; i += kThreads) a += sp[i];
@@ -94,20 +98,20 @@ __global__ void k_loss_reduce(const double* __restrict__ sp, int nsp, const doub
 }  // namespace
 
 void launch_down2(const float* in, Dims n, float* out, Dims m, int n_images, cudaStream_t s) {
-  k_down2<<<dim3(blocks_for(vox(m)), n_images), kThreads, 0, s>>>(in, n, out, m);
+  launch(k_down2, dim3(blocks_for(vox(m)), n_images), kThreads, 0, s)(in, n, out, m);
 }
 void launch_count_nonfinite(const float* x, size_t n, int* count, cudaStream_t s) {
   const unsigned b = (unsigned)std::min<size_t>((n + kThreads - 1) / kThreads, (size_t)16 * device_sm_count());
-  if (b) k_count_nonfinite<<<b, kThreads, 0, s>>>(x, n, count);
+  if (b) launch(k_count_nonfinite, b, kThreads, 0, s)(x, n, count);
 }
 void launch_upsample_disp(const float4* U, Dims nf, Dims ni, float* out, cudaStream_t s) {
-  k_upsample_disp<<<blocks_for(vox(ni)), kThreads, 0, s>>>(U, nf, ni, out);
+  launch(k_upsample_disp, blocks_for(vox(ni)), kThreads, 0, s)(U, nf, ni, out);
 }
 
 void launch_loss_reduce(const double* sim_part, int n_sim, const double* reg_part, int n_reg, double inv_NR,
                         double inv_F, double inv_Nm2, float a_ss, float a_l2, float a_ts, double* out, double* hist,
                         int* step, int* flag, int advance, cudaStream_t s) {
-  k_loss_reduce<<<1, kThreads, 0, s>>>(sim_part, n_sim, reg_part, n_reg, inv_NR, inv_F, inv_Nm2, a_ss, a_l2, a_ts,
+  launch(k_loss_reduce, 1, kThreads, 0, s)(sim_part, n_sim, reg_part, n_reg, inv_NR, inv_F, inv_Nm2, a_ss, a_l2, a_ts,
                                        out, hist, step, flag, advance);
 }
 

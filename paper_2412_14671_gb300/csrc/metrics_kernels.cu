@@ -60,6 +60,7 @@ __device__ __forceinline__ Run<NX> load_run(const float* __restrict__ p) {
 template <int NX>
 __global__ void __launch_bounds__(kJT, 3) k_jacobian_det(const float* __restrict__ u, Dims n,
                                                          float* __restrict__ J, int zchunk) {
+  grid_begin();
   const int runs = n.n2 / NX, i = blockIdx.x * kJT + threadIdx.x, lane = threadIdx.x & 31;
   const bool in = i < runs * n.n1;
   const int y = in ? i / runs : 0, x = in ? (i - y * runs) * NX : 0;
@@ -215,6 +216,7 @@ __device__ __forceinline__ void part_sums(const double* __restrict__ part, int n
 __global__ void __launch_bounds__(kMT) k_metrics_pass1(const float* __restrict__ ut, const float* __restrict__ ue,
                                                        const unsigned char* __restrict__ roi, size_t V,
                                                        double* __restrict__ part) {
+  grid_begin();
   int count = 0;
   DF acc[kP1];  // count, sum |d|, sum ut (3), sum ue (3)
 #pragma unroll
@@ -241,6 +243,7 @@ __global__ void __launch_bounds__(kMT) k_metrics_pass1(const float* __restrict__
 // means from the pass-1 partials: stats = {count, sum |d|, mt[3], me[3]} with means in place
 __global__ void __launch_bounds__(kMT) k_metrics_means(const double* __restrict__ part, int nparts,
                                                        double* __restrict__ stats) {
+  grid_begin();
   __shared__ double sh[kMT];
   __shared__ double S[kP1];
   part_sums(part, nparts, kP1, sh, S);
@@ -251,6 +254,7 @@ __global__ void __launch_bounds__(kMT) k_metrics_means(const double* __restrict_
 __global__ void __launch_bounds__(kMT) k_metrics_pass2(const float* __restrict__ ut, const float* __restrict__ ue,
                                                        const unsigned char* __restrict__ roi, size_t V,
                                                        const double* __restrict__ stats, double* __restrict__ part) {
+  grid_begin();
   // the means as double-float pairs (hi = nearest float, lo = the float of the remainder)
   float mh[6], ml[6];
 #pragma unroll
@@ -289,6 +293,7 @@ __global__ void __launch_bounds__(kMT) k_metrics_pass2(const float* __restrict__
 // final: fixed-order sums of the pass-2 partials, then Eu, PCC, A = Cet Ctt^-1, b, B
 __global__ void __launch_bounds__(kMT) k_metrics_final(const double* __restrict__ part, int nparts,
                                                        const double* __restrict__ stats, double* __restrict__ out) {
+  grid_begin();
   __shared__ double sh[kMT];
   __shared__ double S[kP2];
   part_sums(part, nparts, kP2, sh, S);
@@ -338,9 +343,9 @@ void launch_jacobian_det(const float* u, Dims n, float* J, cudaStream_t s) {
   while (zc > 4 && (long)gx * ((n.n0 + zc - 1) / zc) < want) zc = (zc + 1) / 2;
   const dim3 g(gx, (n.n0 + zc - 1) / zc);
   if (four)
-    k_jacobian_det<4><<<g, kJT, 0, s>>>(u, n, J, zc);
+    launch(k_jacobian_det<4>, g, kJT, 0, s)(u, n, J, zc);
   else
-    k_jacobian_det<1><<<g, kJT, 0, s>>>(u, n, J, zc);
+    launch(k_jacobian_det<1>, g, kJT, 0, s)(u, n, J, zc);
 }
 
 size_t metrics_scratch_doubles() { return (size_t)kMCtas * (kP1 + kP2) + kP1; }
@@ -353,10 +358,10 @@ void launch_deformation_metrics(const float* ut, const float* ue, const unsigned
   double* p1 = scratch;
   double* p2 = scratch + (size_t)kMCtas * kP1;
   double* stats = p2 + (size_t)kMCtas * kP2;
-  k_metrics_pass1<<<ctas, kMT, 0, s>>>(ut, ue, roi, V, p1);
-  k_metrics_means<<<1, kMT, 0, s>>>(p1, ctas, stats);
-  k_metrics_pass2<<<ctas, kMT, 0, s>>>(ut, ue, roi, V, stats, p2);
-  k_metrics_final<<<1, kMT, 0, s>>>(p2, ctas, stats, out);
+  launch(k_metrics_pass1, ctas, kMT, 0, s)(ut, ue, roi, V, p1);
+  launch(k_metrics_means, 1, kMT, 0, s)(p1, ctas, stats);
+  launch(k_metrics_pass2, ctas, kMT, 0, s)(ut, ue, roi, V, stats, p2);
+  launch(k_metrics_final, 1, kMT, 0, s)(p2, ctas, stats, out);
 }
 
 }  // namespace muster

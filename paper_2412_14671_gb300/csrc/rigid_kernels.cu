@@ -61,6 +61,7 @@ __device__ void table_row(const float* rho, int i, const RigidArgs& a, float* ro
 }
 
 __global__ void k_rigid_table(const float* __restrict__ rho, float* __restrict__ tab, RigidArgs a) {
+  grid_begin();
   const int i = threadIdx.x;
   if (i < a.N) table_row(rho, i, a, tab + 12 * i);
 }
@@ -73,6 +74,7 @@ constexpr int kRigidLanes = 32;
 __global__ void __launch_bounds__(12 * kRigidLanes) k_rigid_grad(const float* __restrict__ rpart,
                                                                  const float* __restrict__ rho, float* __restrict__ grad,
                                                                  RigidArgs a) {
+  grid_begin();
   __shared__ double sh[kRigidLanes][12];
   __shared__ double S[12];
   const int i = blockIdx.x + 1, e = threadIdx.x % 12, l = threadIdx.x / 12;
@@ -106,6 +108,7 @@ __global__ void __launch_bounds__(12 * kRigidLanes) k_rigid_grad(const float* __
 __global__ void k_rigid_step(float* __restrict__ rho, float* __restrict__ m, float* __restrict__ v,
                              const float* __restrict__ grad, const float* __restrict__ sched,
                              const int* __restrict__ step, float* __restrict__ tab, RigidArgs a) {
+  grid_begin();
   const int e = threadIdx.x, n = 6 * (a.N - 1);
   if (e < n) {
     const int s = *step;
@@ -128,6 +131,7 @@ __global__ void k_rigid_step(float* __restrict__ rho, float* __restrict__ m, flo
 
 // u (planar (3, D, H, W), image voxels) += A_i p + b_i of table row `row`
 __global__ void k_add_rigid(float* __restrict__ u, Dims n, const float* __restrict__ row) {
+  grid_begin();
   const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y, z = blockIdx.z;
   if (x >= n.n2) return;
   const size_t V = vox(n), o = ((size_t)z * n.n1 + y) * n.n2 + x;
@@ -137,17 +141,17 @@ __global__ void k_add_rigid(float* __restrict__ u, Dims n, const float* __restri
 }  // namespace
 
 void launch_rigid_table(const float* rho, float* tab, const RigidArgs& a, cudaStream_t s) {
-  k_rigid_table<<<1, 32, 0, s>>>(rho, tab, a);
+  launch(k_rigid_table, 1, 32, 0, s)(rho, tab, a);
 }
 void launch_rigid_grad(const float* rpart, const float* rho, float* grad, const RigidArgs& a, cudaStream_t s) {
-  k_rigid_grad<<<a.N - 1, 12 * kRigidLanes, 0, s>>>(rpart, rho, grad, a);
+  launch(k_rigid_grad, a.N - 1, 12 * kRigidLanes, 0, s)(rpart, rho, grad, a);
 }
 void launch_rigid_step(float* rho, float* m, float* v, const float* grad, const float* sched, const int* step,
                        float* tab, const RigidArgs& a, cudaStream_t s) {
-  k_rigid_step<<<1, 192, 0, s>>>(rho, m, v, grad, sched, step, tab, a);
+  launch(k_rigid_step, 1, 192, 0, s)(rho, m, v, grad, sched, step, tab, a);
 }
 void launch_add_rigid(float* u, Dims n, const float* row, cudaStream_t s) {
-  k_add_rigid<<<dim3((n.n2 + 127) / 128, n.n1, n.n0), 128, 0, s>>>(u, n, row);
+  launch(k_add_rigid, dim3((n.n2 + 127) / 128, n.n1, n.n0), 128, 0, s)(u, n, row);
 }
 
 }  // namespace muster

@@ -71,6 +71,7 @@ constexpr int kThreads = 256, TX = 32;  // k_fixed_stats
 template <int R, int KIND>
 __global__ void __launch_bounds__(kThreads) k_fixed_stats(const float* __restrict__ imgs, float* __restrict__ stats,
                                                           Dims n, int tz, int nzc, float eps) {
+  grid_begin();
   constexpr int WW = 2 * R + 1, TY = 8, RX = TX + 2 * R, RY = TY + 2 * R;
   constexpr int NE = RY * RX, NSLOT = (NE + kThreads - 1) / kThreads;
   __shared__ float sF[NE];
@@ -507,6 +508,7 @@ __global__ void __launch_bounds__(Box<R>::NT, kMinCtas)
     k_sim_fwd(const __grid_constant__ SimMaps maps, const PairDesc* __restrict__ pd, const float* __restrict__ Wb,
               size_t Wstride, float* __restrict__ coef, size_t cstride, double* __restrict__ part, Dims n, Tiles g,
               float eps, int* __restrict__ err) {
+  grid_begin();
   using B = Box<R>;
   constexpr int NM = KIND == 0 ? 2 : 3, NC = KIND == 0 ? 2 : 3;
   extern __shared__ __align__(128) float smem[];
@@ -675,6 +677,7 @@ __global__ void __launch_bounds__(Box<R>::NT, kMinCtas)
     k_sim_bwd(const __grid_constant__ SimMaps maps, const PairDesc* __restrict__ pd, const float* __restrict__ Wb,
               size_t Wstride, const float* __restrict__ coef, size_t cstride, float* __restrict__ dLdW, Dims n, Tiles g,
               float scale, int* __restrict__ err) {
+  grid_begin();
   using B = Box<R>;
   constexpr int NC = KIND == 0 ? 2 : 3, XOFF = TMA ? bwd_xoff<R>() : 0;
   static_assert(!TMA || (2 * R + XOFF) % 4 == 0, "the staged adjoint box must start at a multiple of 4 floats");
@@ -924,11 +927,11 @@ template <int KIND>
 void fixed_stats(dim3 g, const float* imgs, Dims ni, int window, float eps, float* stats, int tz, int nzc,
                  cudaStream_t s) {
   switch (window / 2) {
-    case 1: k_fixed_stats<1, KIND><<<g, kThreads, 0, s>>>(imgs, stats, ni, tz, nzc, eps); break;
-    case 2: k_fixed_stats<2, KIND><<<g, kThreads, 0, s>>>(imgs, stats, ni, tz, nzc, eps); break;
-    case 3: k_fixed_stats<3, KIND><<<g, kThreads, 0, s>>>(imgs, stats, ni, tz, nzc, eps); break;
-    case 4: k_fixed_stats<4, KIND><<<g, kThreads, 0, s>>>(imgs, stats, ni, tz, nzc, eps); break;
-    case 5: k_fixed_stats<5, KIND><<<g, kThreads, 0, s>>>(imgs, stats, ni, tz, nzc, eps); break;
+    case 1: launch(k_fixed_stats<1, KIND>, g, kThreads, 0, s)(imgs, stats, ni, tz, nzc, eps); break;
+    case 2: launch(k_fixed_stats<2, KIND>, g, kThreads, 0, s)(imgs, stats, ni, tz, nzc, eps); break;
+    case 3: launch(k_fixed_stats<3, KIND>, g, kThreads, 0, s)(imgs, stats, ni, tz, nzc, eps); break;
+    case 4: launch(k_fixed_stats<4, KIND>, g, kThreads, 0, s)(imgs, stats, ni, tz, nzc, eps); break;
+    case 5: launch(k_fixed_stats<5, KIND>, g, kThreads, 0, s)(imgs, stats, ni, tz, nzc, eps); break;
     default: break;
   }
 }
@@ -978,7 +981,7 @@ void launch_sim_fwd(const PairDesc* pd, int n_pairs, int batch, int group, const
                     int* err, cudaStream_t s) {
   const Tiles g = sim_tiles(ni, window, kind, n_pairs, batch, group);
   dispatch(window / 2, kind, maps && maps->fwd_ok, [&](auto r, auto k, auto t) {
-    k_sim_fwd<r(), k(), t()><<<ctas(g), Box<r()>::NT, Box<r()>::bytes(2, k() == 0 ? 2 : 3), s>>>(
+    launch(k_sim_fwd<r(), k(), t()>, ctas(g), Box<r()>::NT, Box<r()>::bytes(2, k() == 0 ? 2 : 3), s)(
         maps ? *maps : SimMaps{}, pd, W, Wstride, coef, cs, partials, ni, g, eps, err);
   });
 }
@@ -988,7 +991,7 @@ void launch_sim_bwd(const PairDesc* pd, int n_pairs, int batch, int group, const
   const Tiles g = sim_tiles(ni, window, kind, n_pairs, batch, group);
   dispatch(window / 2, kind, maps && maps->bwd_ok, [&](auto r, auto k, auto t) {
     constexpr int nc = k() == 0 ? 2 : 3;
-    k_sim_bwd<r(), k(), t()><<<ctas(g), Box<r()>::NT, Box<r()>::bytes(nc, nc), s>>>(
+    launch(k_sim_bwd<r(), k(), t()>, ctas(g), Box<r()>::NT, Box<r()>::bytes(nc, nc), s)(
         maps ? *maps : SimMaps{}, pd, W, Wstride, coef, cs, dLdW, ni, g, scale, err);
   });
 }

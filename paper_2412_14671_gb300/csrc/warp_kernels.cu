@@ -32,7 +32,6 @@ constexpr int OX = RX - 2, OY = RY - 2;    // adjoint: flow nodes written per CT
 // (a tensor copy must start on a 16-byte boundary) only while OX is even
 static_assert(OX % 2 == 0, "the staged warp-adjoint box must start at a multiple of 4 floats");
 
-__device__ __forceinline__ float3 f3(float4 a) { return make_float3(a.x, a.y, a.z); }
 
 // The stencil's passes with weights 0.25 / 0.75, scaled by 4 (a power of two commutes with every
 // rounding): a + 3 b with the product rounded first, and 3 b + c in one rounding, as the unscaled
@@ -92,6 +91,7 @@ __device__ __forceinline__ float cell_sample(const Cells& I, float qz, float qy,
 
 // the cells of image volumes (grid y over images)
 __global__ void k_image_cells(const float* __restrict__ in, Dims n, float2* __restrict__ out) {
+  grid_begin();
   const Dims m{n.n0 + 2, n.n1 + 2, n.n2 + 1};
   const unsigned v = blockIdx.x * blockDim.x + threadIdx.x;
   const size_t Vm = vox(m);
@@ -119,6 +119,7 @@ template <bool GRAD, bool RIGID>
 __global__ void __launch_bounds__(BX* BY, kWarpCtas) k_warp(const PairDesc* __restrict__ pd, int n_pairs, Dims ni, Dims nf, int nz,
                                                  float* __restrict__ W, float* __restrict__ gI, size_t stride,
                                                  const float* __restrict__ rig) {
+  grid_begin();
   // the pairs of the launch run beside each other on a tile, so that a moving image's region is read
   // from L2 by all pairs but the first
   unsigned id = blockIdx.x;
@@ -234,6 +235,7 @@ __global__ void __launch_bounds__(RX* RY) k_warp_bwd2(const PairDesc* __restrict
                                                       const float* __restrict__ gIb, size_t stride, Dims ni, Dims nf,
                                                       int fz, int nzc, float* __restrict__ rpart,
                                                       unsigned* __restrict__ gmax) {
+  grid_begin();
   __shared__ float sh[RY][RX][12];
   float gm = 0.f;  // largest |component| of the nodes this thread writes
   // with rpart: sums of dL/dq and dL/dq p^T over the image voxels of the nodes this CTA
@@ -401,6 +403,7 @@ __global__ void __launch_bounds__(RX* RY) k_warp_bwd3t(const __grid_constant__ W
                                                        const PairDesc* __restrict__ pd, Dims ni, Dims nf, int fz,
                                                        int nzc, float* __restrict__ rpart, int* __restrict__ err,
                                                        unsigned* __restrict__ gmax) {
+  grid_begin();
   float gm = 0.f;  // largest |component| of the nodes this thread writes
   __shared__ __align__(8) uint64_t bar[2];
   extern __shared__ __align__(128) float smem_raw[];
@@ -588,20 +591,20 @@ void launch_warp(const PairDesc* pd, int n_pairs, Dims ni, Dims nf, float* W, fl
   const dim3 b(BX, BY);
   if (gI) {
     if (rigid)
-      k_warp<true, true><<<grid, b, 0, s>>>(pd, n_pairs, ni, nf, nz, W, gI, Wstride, rigid);
+      launch(k_warp<true, true>, grid, b, 0, s)(pd, n_pairs, ni, nf, nz, W, gI, Wstride, rigid);
     else
-      k_warp<true, false><<<grid, b, 0, s>>>(pd, n_pairs, ni, nf, nz, W, gI, Wstride, nullptr);
+      launch(k_warp<true, false>, grid, b, 0, s)(pd, n_pairs, ni, nf, nz, W, gI, Wstride, nullptr);
   } else {
     if (rigid)
-      k_warp<false, true><<<grid, b, 0, s>>>(pd, n_pairs, ni, nf, nz, W, nullptr, Wstride, rigid);
+      launch(k_warp<false, true>, grid, b, 0, s)(pd, n_pairs, ni, nf, nz, W, nullptr, Wstride, rigid);
     else
-      k_warp<false, false><<<grid, b, 0, s>>>(pd, n_pairs, ni, nf, nz, W, nullptr, Wstride, nullptr);
+      launch(k_warp<false, false>, grid, b, 0, s)(pd, n_pairs, ni, nf, nz, W, nullptr, Wstride, nullptr);
   }
 }
 
 size_t image_cells(Dims n) { return vox(Dims{n.n0 + 2, n.n1 + 2, n.n2 + 1}); }
 void launch_image_cells(const float* in, int n_images, Dims n, float2* out, cudaStream_t s) {
-  k_image_cells<<<dim3((unsigned)((image_cells(n) + 255) / 256), n_images), 256, 0, s>>>(in, n, out);
+  launch(k_image_cells, dim3((unsigned)((image_cells(n) + 255) / 256), n_images), 256, 0, s)(in, n, out);
 }
 
 int warp_bwd_ctas_per_pair(Dims nf, int batch) {
@@ -642,15 +645,15 @@ void launch_warp_bwd(const PairDesc* pd, int n_pairs, int batch, const float* dL
   const dim3 g(gx, gy, nzc * n_pairs), b(RX, RY);
   if (maps && maps->ok && stride == vox(ni)) {
     if (rigid_part)
-      k_warp_bwd3t<true><<<g, b, kWarpBwd3tBytes, s>>>(*maps, pd, ni, nf, fz, nzc, rigid_part, err, gmax);
+      launch(k_warp_bwd3t<true>, g, b, kWarpBwd3tBytes, s)(*maps, pd, ni, nf, fz, nzc, rigid_part, err, gmax);
     else
-      k_warp_bwd3t<false><<<g, b, kWarpBwd3tBytes, s>>>(*maps, pd, ni, nf, fz, nzc, nullptr, err, gmax);
+      launch(k_warp_bwd3t<false>, g, b, kWarpBwd3tBytes, s)(*maps, pd, ni, nf, fz, nzc, nullptr, err, gmax);
     return;
   }
   if (rigid_part)
-    k_warp_bwd2<true><<<g, b, 0, s>>>(pd, dLdW, gI, stride, ni, nf, fz, nzc, rigid_part, gmax);
+    launch(k_warp_bwd2<true>, g, b, 0, s)(pd, dLdW, gI, stride, ni, nf, fz, nzc, rigid_part, gmax);
   else
-    k_warp_bwd2<false><<<g, b, 0, s>>>(pd, dLdW, gI, stride, ni, nf, fz, nzc, nullptr, gmax);
+    launch(k_warp_bwd2<false>, g, b, 0, s)(pd, dLdW, gI, stride, ni, nf, fz, nzc, nullptr, gmax);
 }
 
 }  // namespace muster
