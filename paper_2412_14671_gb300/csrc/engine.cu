@@ -974,8 +974,10 @@ int create_impl(const int64_t shape[3], int n_sessions, const double spacing[3],
   ctx->fstats.resize(L);
   ctx->cells.resize(L);
   for (int l = 0; l < L; ++l) {
-    ctx->cells[l] = (float2*)A(sizeof(float2) * ctx->N * image_cells(ctx->ni[l]));
-    ctx->imgs[l] = (float*)A(sizeof(float) * ctx->N * nvox(ctx->ni[l]));
+    // images and their cells share an allocation
+    const size_t img_bytes = (sizeof(float) * ctx->N * nvox(ctx->ni[l]) + 255) / 256 * 256;
+    ctx->imgs[l] = (float*)A(img_bytes + sizeof(float2) * ctx->N * image_cells(ctx->ni[l]));
+    if (ctx->imgs[l]) ctx->cells[l] = (float2*)((char*)ctx->imgs[l] + img_bytes);
     ctx->fstats[l] = (float*)A(sizeof(float) * 2 * ctx->N * nvox(ctx->ni[l]));
   }
   ctx->theta = (float4*)A(sizeof(float4) * F * Vf);
