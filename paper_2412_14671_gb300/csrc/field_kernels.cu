@@ -482,8 +482,8 @@ __global__ void k_smooth_axis(const float4* __restrict__ in, float4* __restrict_
 }
 // along axis 2: a CTA per kSR rows
 constexpr int kSR = 32, kSmoothRow = 256;  // rows per CTA, longest staged row (132 KB)
-__global__ void __launch_bounds__(kSR * kSmoothRow / kSO) k_smooth_rows(const float4* __restrict__ in, float4* __restrict__ out, Dims n,
-                              const float* __restrict__ taps, int lo, int hi, int pitch) {
+__global__ void __launch_bounds__(kSR* kSmoothRow / kSO)
+    k_smooth_rows(const float4* __restrict__ in, float4* __restrict__ out, Dims n, const float* __restrict__ taps, int lo, int hi, int pitch) {
   grid_begin();
   extern __shared__ float4 row[];  // [kSR][pitch], then the taps
   const int m = n.n2, rows = n.n0 * n.n1, r0 = blockIdx.x * kSR, nr = min(kSR, rows - r0);
@@ -540,20 +540,22 @@ __device__ __forceinline__ void block_sum3(FF a, FF b, FF c, double* out) {
 // With fx.ain (deterministic mode) G0 is completed with its fixed-point sums, which are cleared.
 // CLEAR: G0 read through G0clr (the same buffer) and cleared after the read (see
 // k_squaring_bwd's Gclr).
-// A CTA takes kRegRuns runs of 256 voxels: its three sums (float-float shuffle trees, then double) cost
+// A CTA takes `runs` runs of 256 voxels: its three sums (float-float shuffle trees, then double) cost
 // about as much as a voxel's whole gradient, so several voxels per thread share them. 9 fields of
-// 80 x 96 x 80: 104 us; one voxel per thread and one thread for the double sums took 157 us.
+// 80 x 96 x 80: 104 us; one voxel per thread and one thread for the double sums took 157 us. On grids
+// of less than kRegRuns runs per SM latency counts instead, and a thread takes fewer (2 fields of 24^3:
+// 5.0 us with one, 7.0 with four).
 constexpr int kRegRuns = 4;
 template <bool CLEAR>
 __global__ void k_reg_grad(const float4* __restrict__ th, const float4* __restrict__ G0,
                            float4* __restrict__ grad, double* __restrict__ part, Dims n, RegArgs a, FxArgs fx,
-                           float4* G0clr) {
+                           float4* G0clr, int runs) {
   grid_begin();
   const int V = (int)vox(n);
   const int f = blockIdx.y, F = a.n_fields;
   FF sss{0.f, 0.f}, sl2{0.f, 0.f}, sts{0.f, 0.f};
-  for (int run = 0; run < kRegRuns; ++run) {
-    const int v = (blockIdx.x * kRegRuns + run) * blockDim.x + threadIdx.x;
+  for (int run = 0; run < runs; ++run) {
+    const int v = (blockIdx.x * runs + run) * blockDim.x + threadIdx.x;
     if (v >= V) break;
     float lss = 0.f, ll2 = 0.f, lts = 0.f;
     const float4* T = th + (size_t)f * V;
@@ -782,15 +784,17 @@ void launch_add(const AddDesc* d, int n, Dims dims, cudaStream_t s) {
     launch(k_add, dim3(blocks_for(vox(dims)), cnt), kThreads, 0, s)(t, (int)vox(dims));
   }
 }
-int reg_blocks(Dims n) { return (int)((vox(n) + kRegRuns * kThreads - 1) / (kRegRuns * kThreads)); }
+int reg_runs(Dims n) { return std::max(1, std::min(kRegRuns, (int)(blocks_for(vox(n)) / device_sm_count()))); }
+int reg_blocks(Dims n) { return (int)((blocks_for(vox(n)) + reg_runs(n) - 1) / reg_runs(n)); }
 void launch_reg_grad(const float4* theta, const float4* G0, float4* grad, double* partials, Dims n,
                      const RegArgs& a, const FxArgs* fx, cudaStream_t s, bool clear_g0) {
   const dim3 g(reg_blocks(n), a.n_fields);
   if (clear_g0 && G0)
     launch(k_reg_grad<true>, g, kThreads, 0, s)(theta, G0, grad, partials, n, a, fx ? *fx : FxArgs{},
-                                             const_cast<float4*>(G0));
+                                                const_cast<float4*>(G0), reg_runs(n));
   else
-    launch(k_reg_grad<false>, g, kThreads, 0, s)(theta, G0, grad, partials, n, a, fx ? *fx : FxArgs{}, nullptr);
+    launch(k_reg_grad<false>, g, kThreads, 0, s)(theta, G0, grad, partials, n, a, fx ? *fx : FxArgs{}, nullptr,
+                                                 reg_runs(n));
 }
 cudaError_t prepare_field_kernels() {
   static std::mutex mu;

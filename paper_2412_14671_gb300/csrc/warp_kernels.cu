@@ -567,20 +567,23 @@ constexpr size_t kWarpBwd3tBytes = 128 + sizeof(float) * 2 * 4 * SARR;
 
 // flow planes per D chunk of the adjoint: every chunk streams two planes more than it
 // writes, so chunks are split only until a launch of `batch` pairs has about four waves of
-// four CTAs on each of 152 SMs (2432 CTAs), and halved only while above 4 planes
+// four CTAs on each of 152 SMs (2432 CTAs), and halved only while above 2 planes
+// (6 pairs of 48^3: 7.5 us at 2 planes, 8.5 at 3)
 int chunk_nodes(int ntiles, int depth, int batch) {
   int fz = depth;
-  while (fz > 4 && (long)batch * ntiles * ((depth + fz - 1) / fz) < 2432) fz = (fz + 1) / 2;
+  while (fz > 2 && (long)batch * ntiles * ((depth + fz - 1) / fz) < 2432) fz = (fz + 1) / 2;
   return fz < 1 ? 1 : fz;
 }
 }  // namespace
 
 // node planes a thread of the forward walks: every walk loads two planes more than it emits, so it
 // is as long as leaves the launch about four waves of four CTAs on every SM, 32 planes at most
-// (90 pairs of 160 x 192 x 160: 2286 us at 8 planes, 2211 at 16, 2170 at 32)
+// (90 pairs of 160 x 192 x 160: 2286 us at 8 planes, 2211 at 16, 2170 at 32). Walks of one plane only
+// where they fit one wave (6 pairs of 48^3, 1.4 waves of them: 7.2 us at 1, 6.2 at 2 and 3, 7.2 at 4)
 static int warp_planes(long tiles, int depth) {
+  const int least = tiles * depth <= (long)kWarpCtas * device_sm_count() ? 1 : 2;
   int nz = 32;
-  while (nz > 1 && tiles * ((depth + nz - 1) / nz) < 16L * device_sm_count()) nz /= 2;
+  while (nz > least && tiles * ((depth + nz - 1) / nz) < 16L * device_sm_count()) nz /= 2;
   return nz;
 }
 void launch_warp(const PairDesc* pd, int n_pairs, Dims ni, Dims nf, float* W, float* gI, size_t Wstride,
