@@ -63,86 +63,112 @@
 namespace muster {
 
 namespace {
-constexpr int kThreads = 256, TX = 32;  // k_fixed_stats
+constexpr int kStatThreads = 128, TX = 32;  // k_fixed_stats
 
 // Statistics of the fixed image of every window, once per session and level:
 // out[0][c] = mu_F and out[1][c] = S_FF (centred sum of squares) at corner c, or for SiLNCC
 // (KIND 0, which needs S_FF only in beta = S_FW / (S_FF + eps)) out[1][c] = 1 / (S_FF + eps).
+// A CTA walks the planes of a 32 x 8 tile: a W task forms 4 neighbouring sums from one read of their
+// inputs, a thread of the H and D sums has 2 rows of a column, and a plane's loads are under way while
+// the plane before is summed. Shared memory bounds it. One 160 x 192 x 160 image, w = 7: 36 us; one sum
+// per thread and pass (twice the shared-memory traffic) and loads between two barriers took 44 us.
+// Every sum adds its terms one after the other.
 template <int R, int KIND>
-__global__ void __launch_bounds__(kThreads) k_fixed_stats(const float* __restrict__ imgs, float* __restrict__ stats,
-                                                          Dims n, int tz, int nzc, float eps) {
+__global__ void __launch_bounds__(kStatThreads) k_fixed_stats(const float* __restrict__ imgs, float* __restrict__ stats,
+                                                              Dims n, int tz, int nzc, float eps) {
   grid_begin();
-  constexpr int WW = 2 * R + 1, TY = 8, RX = TX + 2 * R, RY = TY + 2 * R;
-  constexpr int NE = RY * RX, NSLOT = (NE + kThreads - 1) / kThreads;
-  __shared__ float sF[NE];
-  __shared__ float sx[2][RY][TX];
+  constexpr int WW = 2 * R + 1, TY = 8, RX = TX + 2 * R, RY = TY + 2 * R, PF = (RX + 3) / 4 * 4;
+  constexpr int NE = RY * RX, NSLOT = (NE + kStatThreads - 1) / kStatThreads;
+  constexpr int NO = 4, NI = NO + 2 * R, NV = (NI + 3) / 4, NR = TY * TX / kStatThreads;
+  __shared__ float4 sF[RY][PF / 4];
+  __shared__ float4 sx[2][RY][TX / 4];
   const int img = blockIdx.z / nzc, zc = blockIdx.z - img * nzc;
   const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, z0 = zc * tz;
-  const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
+  const int tid = threadIdx.x, tx = tid & 31, row = tid / 32 * NR;
   const int plane = n.n1 * n.n2;
   const size_t V = (size_t)plane * n.n0;
   const float* __restrict__ F = imgs + (size_t)img * V;
   float* __restrict__ out = stats + (size_t)img * 2 * V;
-  int soff[NSLOT];
-  bool sok[NSLOT];
+  int goff[NSLOT], soff[NSLOT];  // global (-1: outside) and shared position of a thread's inputs
 #pragma unroll
   for (int k = 0; k < NSLOT; ++k) {
-    const int e = tid + kThreads * k;
+    const int e = tid + kStatThreads * k;
     const int ry = e / RX, rx = e - ry * RX;
     const int gy = y0 + ry, gx = x0 + rx;
-    sok[k] = e < NE && gy < n.n1 && gx < n.n2;
-    soff[k] = gy * n.n2 + gx;
+    goff[k] = e < NE && gy < n.n1 && gx < n.n2 ? gy * n.n2 + gx : -1;
+    soff[k] = e < NE ? ry * PF + rx : -1;
   }
   const float shF = F[min(z0 + R, n.n0 - 1) * plane + min(y0 + R, n.n1 - 1) * n.n2 + min(x0 + R, n.n2 - 1)];
   const float inv_nw = 1.f / (float)(WW * WW * WW);
-  float ring[2][WW] = {}, S[2] = {0.f, 0.f};
+  float ring[NR][2][WW] = {}, S[NR][2] = {};
   const int zend = min(z0 + tz, n.n0);
   const int niter = (zend - z0) + 2 * R;
+  float next[NSLOT];
+  auto load = [&](int z) {
+#pragma unroll
+    for (int k = 0; k < NSLOT; ++k) next[k] = z < n.n0 && goff[k] >= 0 ? F[z * plane + goff[k]] - shF : 0.f;
+  };
+  load(z0);
   for (int base = 0; base < niter; base += WW) {
 #pragma unroll
     for (int j = 0; j < WW; ++j) {
       const int it = base + j;
       if (it >= niter) break;
-      const int zin = z0 + it;
 #pragma unroll
-      for (int k = 0; k < NSLOT; ++k) {
-        const int e = tid + kThreads * k;
-        if (e < NE) sF[e] = (zin < n.n0 && sok[k]) ? F[zin * plane + soff[k]] - shF : 0.f;
-      }
+      for (int k = 0; k < NSLOT; ++k)
+        if (soff[k] >= 0) reinterpret_cast<float*>(sF)[soff[k]] = next[k];
       __syncthreads();
-      for (int ry = ty; ry < RY; ry += kThreads / 32) {
-        float a0 = 0.f, a1 = 0.f;
-        const float* pf = sF + ry * RX + tx;
+      load(z0 + it + 1);
+      for (int t = tid; t < RY * (TX / NO); t += kStatThreads) {
+        const int ry = t / (TX / NO), run = t % (TX / NO);
+        float v[4 * NV], a0[NO] = {}, a1[NO] = {};
 #pragma unroll
-        for (int k = 0; k < WW; ++k) {
-          a0 += pf[k];
-          a1 = fmaf(pf[k], pf[k], a1);
+        for (int q = 0; q < NV; ++q) {
+          const float4 f = sF[ry][run + q];
+          v[4 * q] = f.x, v[4 * q + 1] = f.y, v[4 * q + 2] = f.z, v[4 * q + 3] = f.w;
         }
-        sx[0][ry][tx] = a0;
-        sx[1][ry][tx] = a1;
+#pragma unroll
+        for (int o = 0; o < NO; ++o)
+#pragma unroll
+          for (int k = 0; k < WW; ++k) {
+            a0[o] += v[o + k];
+            a1[o] = fmaf(v[o + k], v[o + k], a1[o]);
+          }
+        sx[0][ry][run] = make_float4(a0[0], a0[1], a0[2], a0[3]);
+        sx[1][ry][run] = make_float4(a1[0], a1[1], a1[2], a1[3]);
       }
       __syncthreads();
 #pragma unroll
       for (int m = 0; m < 2; ++m) {
-        float v = 0.f;
+        float h[NR + 2 * R];
 #pragma unroll
-        for (int k = 0; k < WW; ++k) v += sx[m][ty + k][tx];
-        S[m] += v - ring[m][j];
-        ring[m][j] = v;
-        if (j == WW - 1) {
-          float t = 0.f;
+        for (int k = 0; k < NR + 2 * R; ++k) h[k] = reinterpret_cast<const float*>(sx[m][row + k])[tx];
 #pragma unroll
-          for (int k = 0; k < WW; ++k) t += ring[m][k];
-          S[m] = t;
+        for (int i = 0; i < NR; ++i) {
+          float v = 0.f;
+#pragma unroll
+          for (int k = 0; k < WW; ++k) v += h[i + k];
+          S[i][m] += v - ring[i][m][j];
+          ring[i][m][j] = v;
+          if (j == WW - 1) {
+            float t = 0.f;
+#pragma unroll
+            for (int k = 0; k < WW; ++k) t += ring[i][m][k];
+            S[i][m] = t;
+          }
         }
       }
       if (it >= 2 * R) {
-        const int cz = zin - 2 * R, cy = y0 + ty, cx = x0 + tx;
-        if (cx < n.n2 && cy < n.n1) {
-          const int o = cz * plane + cy * n.n2 + cx;
-          out[o] = S[0] * inv_nw + shF;
-          const float sff = fmaxf(S[1] - S[0] * S[0] * inv_nw, 0.f);
-          out[V + o] = KIND == 0 ? 1.f / (sff + eps) : sff;
+        const int cz = z0 + it - 2 * R, cx = x0 + tx;
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+          const int cy = y0 + row + i;
+          if (cx < n.n2 && cy < n.n1) {
+            const int o = cz * plane + cy * n.n2 + cx;
+            out[o] = S[i][0] * inv_nw + shF;
+            const float sff = fmaxf(S[i][1] - S[i][0] * S[i][0] * inv_nw, 0.f);
+            out[V + o] = KIND == 0 ? 1.f / (sff + eps) : sff;
+          }
         }
       }
     }
@@ -927,11 +953,11 @@ template <int KIND>
 void fixed_stats(dim3 g, const float* imgs, Dims ni, int window, float eps, float* stats, int tz, int nzc,
                  cudaStream_t s) {
   switch (window / 2) {
-    case 1: launch(k_fixed_stats<1, KIND>, g, kThreads, 0, s)(imgs, stats, ni, tz, nzc, eps); break;
-    case 2: launch(k_fixed_stats<2, KIND>, g, kThreads, 0, s)(imgs, stats, ni, tz, nzc, eps); break;
-    case 3: launch(k_fixed_stats<3, KIND>, g, kThreads, 0, s)(imgs, stats, ni, tz, nzc, eps); break;
-    case 4: launch(k_fixed_stats<4, KIND>, g, kThreads, 0, s)(imgs, stats, ni, tz, nzc, eps); break;
-    case 5: launch(k_fixed_stats<5, KIND>, g, kThreads, 0, s)(imgs, stats, ni, tz, nzc, eps); break;
+    case 1: launch(k_fixed_stats<1, KIND>, g, kStatThreads, 0, s)(imgs, stats, ni, tz, nzc, eps); break;
+    case 2: launch(k_fixed_stats<2, KIND>, g, kStatThreads, 0, s)(imgs, stats, ni, tz, nzc, eps); break;
+    case 3: launch(k_fixed_stats<3, KIND>, g, kStatThreads, 0, s)(imgs, stats, ni, tz, nzc, eps); break;
+    case 4: launch(k_fixed_stats<4, KIND>, g, kStatThreads, 0, s)(imgs, stats, ni, tz, nzc, eps); break;
+    case 5: launch(k_fixed_stats<5, KIND>, g, kStatThreads, 0, s)(imgs, stats, ni, tz, nzc, eps); break;
     default: break;
   }
 }
