@@ -28,13 +28,16 @@ namespace muster {
 // ramp between two of them. No kernel touches memory before the wait; results of earlier kernels
 // are there too, since the predecessor waited for them in turn. One exponential of 80 x 96 x 80
 // (8 kernels): 76 -> 53 us per call. In a graph such edges cost more than they hide (20 captured steps of
-// 3 sessions of 48^3: 2890 us with them, 2180 without), so a launch under capture is a plain one.
+// 3 sessions of 48^3: 2890 us with them, 2180 without), so a launch under capture is a plain one. So is
+// one with overlap = false: an SM divides its L1 and shared memory anew only when it is idle, so a kernel that
+// lives on L1 must not start beside one that fills shared memory (the forward warp after the warp adjoint, 34
+// pairs of 256^3: 3.2 ms alone, 5.4 ms with the L1 that the adjoint leaves).
 __device__ __forceinline__ void grid_begin() {
   asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
 }
 // launch(kernel, grid, block, dynamic shared memory, stream)(arguments)
 template <class... P>
-auto launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t shared, cudaStream_t s) {
+auto launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t shared, cudaStream_t s, bool overlap = true) {
   return [=](P... args) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     const bool known = cudaStreamIsCapturing(s, &cap) == cudaSuccess;
@@ -44,7 +47,7 @@ auto launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t shared, cudaStre
     at.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid, cfg.blockDim = block, cfg.dynamicSmemBytes = shared, cfg.stream = s;
-    cfg.attrs = &at, cfg.numAttrs = known && cap == cudaStreamCaptureStatusNone ? 1 : 0;
+    cfg.attrs = &at, cfg.numAttrs = overlap && known && cap == cudaStreamCaptureStatusNone ? 1 : 0;
     void* p[] = {(void*)&args...};
     cudaLaunchKernelExC(&cfg, (const void*)kernel, p);
   };

@@ -594,14 +594,14 @@ void launch_warp(const PairDesc* pd, int n_pairs, Dims ni, Dims nf, float* W, fl
   const dim3 b(BX, BY);
   if (gI) {
     if (rigid)
-      launch(k_warp<true, true>, grid, b, 0, s)(pd, n_pairs, ni, nf, nz, W, gI, Wstride, rigid);
+      launch(k_warp<true, true>, grid, b, 0, s, false)(pd, n_pairs, ni, nf, nz, W, gI, Wstride, rigid);
     else
-      launch(k_warp<true, false>, grid, b, 0, s)(pd, n_pairs, ni, nf, nz, W, gI, Wstride, nullptr);
+      launch(k_warp<true, false>, grid, b, 0, s, false)(pd, n_pairs, ni, nf, nz, W, gI, Wstride, nullptr);
   } else {
     if (rigid)
-      launch(k_warp<false, true>, grid, b, 0, s)(pd, n_pairs, ni, nf, nz, W, nullptr, Wstride, rigid);
+      launch(k_warp<false, true>, grid, b, 0, s, false)(pd, n_pairs, ni, nf, nz, W, nullptr, Wstride, rigid);
     else
-      launch(k_warp<false, false>, grid, b, 0, s)(pd, n_pairs, ni, nf, nz, W, nullptr, Wstride, nullptr);
+      launch(k_warp<false, false>, grid, b, 0, s, false)(pd, n_pairs, ni, nf, nz, W, nullptr, Wstride, nullptr);
   }
 }
 
