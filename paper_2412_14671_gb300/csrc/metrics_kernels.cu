@@ -34,14 +34,15 @@ __device__ __forceinline__ float dstep(float lo, float mid, float hi, int p, int
   return 0.5f * (hi - lo);
 }
 
-// A thread owns NX neighbouring voxels of a row (4 with 16-byte loads when the width is a multiple
-// of 4 and the fields are 16-byte aligned, else 1) and walks a chunk of D with the planes z-1, z, z+1 of
-// the three components in registers. The rows y-1 and y+1 of plane z are loads that hit the L1 or
-// L2 lines of the neighbouring threads' own rows; x-1 and x+NX come from the neighbouring lanes, or
-// from memory at a row's or warp's end. DRAM is the floor (16 bytes per voxel, 12 us at 160 x 192 x 160);
-// the latency of a plane's nine loads per thread bounds it, so 3 CTAs of 80 registers share an SM and
-// the walk is short. 160 x 192 x 160: 28 us; with 2 CTAs per SM 36 us, with runs of 2 voxels 29 us, of 1 47 us;
-// staging every plane of a 32 x 8 tile in shared memory behind two barriers took 39 us.
+// A thread owns NX neighbouring voxels of each of NY rows and walks a chunk of D with the planes z-1, z,
+// z+1 of the three components in registers: 4 or 2 of one row with 16- or 8-byte loads where the width is
+// a multiple and the fields are aligned, else one of two rows, which read the row between them once. The
+// rows beside the run are loads that hit the L1 or L2 lines of the neighbouring threads' own rows; x-1 and
+// x+NX come from the neighbouring lanes, or from memory at a row's or warp's end. DRAM is the floor (16 bytes
+// per voxel, 12 us at 160 x 192 x 160); the latency of a plane's loads bounds it, so 3 or 4 CTAs share an SM and
+// the walk is short. 160 x 192 x 160: 28 us with runs of 4 (36 us with 2 CTAs per SM, 29 us with runs of 2), 160 x
+// 192 x 161 41 us (46 us with one voxel of one or four rows); staging every plane of a 32 x 8 tile in shared
+// memory behind two barriers took 41 and 47 us.
 template <int NX>
 struct Run {
   float v[NX];
@@ -52,72 +53,91 @@ __device__ __forceinline__ Run<NX> load_run(const float* __restrict__ p) {
   if constexpr (NX == 4) {
     const float4 t = __ldg(reinterpret_cast<const float4*>(p));
     r.v[0] = t.x, r.v[1] = t.y, r.v[2] = t.z, r.v[3] = t.w;
+  } else if constexpr (NX == 2) {
+    const float2 t = __ldg(reinterpret_cast<const float2*>(p));
+    r.v[0] = t.x, r.v[1] = t.y;
   } else {
     r.v[0] = __ldg(p);
   }
   return r;
 }
-template <int NX>
-__global__ void __launch_bounds__(kJT, 3) k_jacobian_det(const float* __restrict__ u, Dims n,
-                                                         float* __restrict__ J, int zchunk) {
+template <int NX, int NY>
+__global__ void __launch_bounds__(kJT, NX == 4 ? 3 : 4) k_jacobian_det(const float* __restrict__ u, Dims n,
+                                                                       float* __restrict__ J, int zchunk) {
   grid_begin();
   const int runs = n.n2 / NX, i = blockIdx.x * kJT + threadIdx.x, lane = threadIdx.x & 31;
-  const bool in = i < runs * n.n1;
-  const int y = in ? i / runs : 0, x = in ? (i - y * runs) * NX : 0;
+  const bool in = i < runs * ((n.n1 + NY - 1) / NY);
+  const int y = in ? i / runs * NY : 0, x = in ? i % runs * NX : 0;
   const int z0 = blockIdx.y * zchunk, z1 = min(z0 + zchunk, n.n0);
   const size_t V = vox(n);
   const ptrdiff_t plane = (ptrdiff_t)n.n1 * n.n2;
-  const int below = y > 0 ? -n.n2 : 0, above = y < n.n1 - 1 ? n.n2 : 0;
+  int row[NY];  // rows of the run from its first one, the volume's last row repeated
+#pragma unroll
+  for (int r = 0; r < NY; ++r) row[r] = min(r, n.n1 - 1 - y) * n.n2;
+  const int below = y > 0 ? -n.n2 : 0, above = min(NY, n.n1 - 1 - y) * n.n2;
   const bool left = x > 0, right = x + NX < n.n2;  // x-1 and x+NX exist
   const float* f = u + (size_t)y * n.n2 + x + z0 * plane;
-  Run<NX> prv[3], cur[3], nxt[3];
+  Run<NX> prv[3][NY], cur[3][NY], nxt[3][NY];
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    cur[c] = load_run<NX>(f + c * V);
-    prv[c] = z0 > 0 ? load_run<NX>(f + c * V - plane) : cur[c];
-  }
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int r = 0; r < NY; ++r) {
+      cur[c][r] = load_run<NX>(f + c * V + row[r]);
+      prv[c][r] = z0 > 0 ? load_run<NX>(f + c * V + row[r] - plane) : cur[c][r];
+    }
   for (int z = z0; z < z1; ++z, f += plane) {
     Run<NX> lo[3], hi[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      nxt[c] = z + 1 < n.n0 ? load_run<NX>(f + c * V + plane) : cur[c];
+#pragma unroll
+      for (int r = 0; r < NY; ++r) nxt[c][r] = z + 1 < n.n0 ? load_run<NX>(f + c * V + row[r] + plane) : cur[c][r];
       lo[c] = load_run<NX>(f + c * V + below);
       hi[c] = load_run<NX>(f + c * V + above);
     }
-    float M[NX][3][3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      // the voxels beside the run: a run of the same row in the next lane, else memory
-      float l = __shfl_up_sync(0xffffffffu, cur[c].v[NX - 1], 1), r = __shfl_down_sync(0xffffffffu, cur[c].v[0], 1);
-      if (lane == 0 && left) l = __ldg(f + c * V - 1);
-      if (lane == 31 && right) r = __ldg(f + c * V + NX);
+    for (int r = 0; r < NY; ++r) {
+      float M[NX][3][3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const Run<NX>& me = cur[c][r];
+        // the voxels beside the run: a run of the same row in the next lane, else memory
+        float l = __shfl_up_sync(0xffffffffu, me.v[NX - 1], 1), g = __shfl_down_sync(0xffffffffu, me.v[0], 1);
+        if (lane == 0 && left) l = __ldg(f + c * V + row[r] - 1);
+        if (lane == 31 && right) g = __ldg(f + c * V + row[r] + NX);
+#pragma unroll
+        for (int k = 0; k < NX; ++k) {
+          const float mid = me.v[k];
+          M[k][c][0] = (c == 0 ? 1.f : 0.f) + dstep(prv[c][r].v[k], mid, nxt[c][r].v[k], z, n.n0);
+          M[k][c][1] = (c == 1 ? 1.f : 0.f) + dstep(r > 0 ? cur[c][r > 0 ? r - 1 : 0].v[k] : lo[c].v[k], mid,
+                                                    r < NY - 1 ? cur[c][r < NY - 1 ? r + 1 : r].v[k] : hi[c].v[k], y + r, n.n1);
+          M[k][c][2] = (c == 2 ? 1.f : 0.f) + dstep(k > 0 ? me.v[k > 0 ? k - 1 : 0] : l, mid,
+                                                    k < NX - 1 ? me.v[k < NX - 1 ? k + 1 : k] : g, x + k, n.n2);
+        }
+      }
+      float det[NX];
 #pragma unroll
       for (int k = 0; k < NX; ++k) {
-        const float mid = cur[c].v[k];
-        M[k][c][0] = (c == 0 ? 1.f : 0.f) + dstep(prv[c].v[k], mid, nxt[c].v[k], z, n.n0);
-        M[k][c][1] = (c == 1 ? 1.f : 0.f) + dstep(lo[c].v[k], mid, hi[c].v[k], y, n.n1);
-        M[k][c][2] = (c == 2 ? 1.f : 0.f) + dstep(k > 0 ? cur[c].v[k - 1] : l, mid, k < NX - 1 ? cur[c].v[k + 1] : r, x + k, n.n2);
+        const float(*A)[3] = M[k];
+        det[k] = A[0][0] * (A[1][1] * A[2][2] - A[1][2] * A[2][1]) - A[0][1] * (A[1][0] * A[2][2] - A[1][2] * A[2][0]) +
+                 A[0][2] * (A[1][0] * A[2][1] - A[1][1] * A[2][0]);
+      }
+      if (in && y + r < n.n1) {
+        float* o = J + (size_t)z * plane + (size_t)y * n.n2 + row[r] + x;
+        if constexpr (NX == 4)
+          *reinterpret_cast<float4*>(o) = make_float4(det[0], det[1], det[2], det[3]);
+        else if constexpr (NX == 2)
+          *reinterpret_cast<float2*>(o) = make_float2(det[0], det[1]);
+        else
+          o[0] = det[0];
       }
     }
-    float det[NX];
 #pragma unroll
-    for (int k = 0; k < NX; ++k) {
-      const float(*A)[3] = M[k];
-      det[k] = A[0][0] * (A[1][1] * A[2][2] - A[1][2] * A[2][1]) - A[0][1] * (A[1][0] * A[2][2] - A[1][2] * A[2][0]) +
-               A[0][2] * (A[1][0] * A[2][1] - A[1][1] * A[2][0]);
-    }
-    if (in) {
-      float* o = J + (size_t)z * plane + (size_t)y * n.n2 + x;
-      if constexpr (NX == 4)
-        *reinterpret_cast<float4*>(o) = make_float4(det[0], det[1], det[2], det[3]);
-      else
-        o[0] = det[0];
-    }
+    for (int c = 0; c < 3; ++c)
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      prv[c] = cur[c];
-      cur[c] = nxt[c];
-    }
+      for (int r = 0; r < NY; ++r) {
+        prv[c][r] = cur[c][r];
+        cur[c][r] = nxt[c][r];
+      }
   }
 }
 
@@ -334,18 +354,21 @@ __global__ void __launch_bounds__(kMT) k_metrics_final(const double* __restrict_
 }  // namespace
 
 void launch_jacobian_det(const float* u, Dims n, float* J, cudaStream_t s) {
-  const bool four = n.n2 % 4 == 0 && (reinterpret_cast<uintptr_t>(u) & 15) == 0 && (reinterpret_cast<uintptr_t>(J) & 15) == 0;
+  const uintptr_t at = reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(J);
+  const int nx = n.n2 % 4 == 0 && at % 16 == 0 ? 4 : n.n2 % 2 == 0 && at % 8 == 0 ? 2 : 1;
   // D chunks so that the grid has at least 8 CTAs per SM of the device (5: 30 us, 8 to 30: 28 us)
-  const size_t runs = (size_t)n.n1 * (four ? n.n2 / 4 : n.n2);
+  const size_t runs = (size_t)(nx > 1 ? n.n1 : (n.n1 + 1) / 2) * (n.n2 / nx);
   const unsigned gx = (unsigned)((runs + kJT - 1) / kJT);
   const long want = 8L * device_sm_count();
   int zc = n.n0;
   while (zc > 4 && (long)gx * ((n.n0 + zc - 1) / zc) < want) zc = (zc + 1) / 2;
   const dim3 g(gx, (n.n0 + zc - 1) / zc);
-  if (four)
-    launch(k_jacobian_det<4>, g, kJT, 0, s)(u, n, J, zc);
+  if (nx == 4)
+    launch(k_jacobian_det<4, 1>, g, kJT, 0, s)(u, n, J, zc);
+  else if (nx == 2)
+    launch(k_jacobian_det<2, 1>, g, kJT, 0, s)(u, n, J, zc);
   else
-    launch(k_jacobian_det<1>, g, kJT, 0, s)(u, n, J, zc);
+    launch(k_jacobian_det<1, 2>, g, kJT, 0, s)(u, n, J, zc);
 }
 
 size_t metrics_scratch_doubles() { return (size_t)kMCtas * (kP1 + kP2) + kP1; }

@@ -27,11 +27,12 @@ def test_smoothing_runs(shape, omega):
     assert np.abs(v - vo).max() <= (sum(nf) + 3) * 2.0**-24 * np.abs(theta).max()
 
 
-# Rows of 1, 2 and 33 runs of 4 voxels (lanes at both ends of a warp), and fields that start 4 bytes
-# off a 16-byte boundary; tolerance of the determinant's 12 products of values up to about 3.
-@pytest.mark.parametrize("shape", [(3, 2, 4), (1, 1, 8), (5, 3, 132), (70, 9, 12)])
-@pytest.mark.parametrize("shift", [0, 1])
-def test_jacobian_runs_of_four(shape, shift):
+# Rows of 1, 2 and 33 runs of 4 voxels, of runs of 2 and single voxels of two rows (an odd number of rows, one
+# row), lanes at both ends of a warp, and fields that start 4 or 8 bytes off a 16-byte boundary;
+# tolerance of the determinant's 12 products of values up to about 3.
+@pytest.mark.parametrize("shape", [(3, 2, 4), (1, 1, 8), (5, 3, 132), (70, 9, 12), (3, 5, 2), (6, 7, 66), (4, 1, 35), (9, 5, 97)])
+@pytest.mark.parametrize("shift", [0, 1, 2])
+def test_jacobian_runs(shape, shift):
     n = 3 * int(np.prod(shape))
     flat = torch.zeros(n + 4, device="cuda")
     u = flat[shift:shift + n].view((3,) + shape)
