@@ -696,10 +696,12 @@ void launch_squaring_first(const float4* theta, float4* u0, float4* u1, int n_fi
                            cudaStream_t s, int nf, unsigned* zero) {
   const dim3 g(blocks_for(vox(n)), groups(2 * n_fields, nf));
   if (nf == 1)
-    launch(k_squaring_first<1>, g, kThreads, 0, s)(theta, u0, u1, n, 2 * n_fields, n_fields, scale, zero);
+    launch(k_squaring_first<1>, g, kThreads, 0, s, false)(theta, u0, u1, n, 2 * n_fields, n_fields, scale, zero);
   else
-    launch(k_squaring_first<2>, g, kThreads, 0, s)(theta, u0, u1, n, 2 * n_fields, n_fields, scale, zero);
+    launch(k_squaring_first<2>, g, kThreads, 0, s, false)(theta, u0, u1, n, 2 * n_fields, n_fields, scale, zero);
 }
+// Plain launches (see launch): the kernels that can follow one that fills shared memory (the first squaring
+// after smoothing; the composition adjoints, or the first squaring adjoint, after the warp adjoint).
 // grid of the 2-D layout: W tiles, H tiles, D planes x groups of fields
 dim3 grid2(Dims n, int count, int nf) {
   return dim3((n.n2 + kT2 - 1) / kT2, (n.n1 + kT2 - 1) / kT2, (unsigned)n.n0 * groups(count, nf));
@@ -708,13 +710,13 @@ template <int NF>
 void squaring_bwd_nf(const float4* u, const float4* Gin, float4* Gout, int n_fields2, Dims n, const FxArgs* fx,
                      const PairGradTab& pg, float4* Gclr, cudaStream_t s) {
   if (fx)
-    launch(k_squaring_bwd<true, NF>, grid2(n, n_fields2, NF), kThreads, 0, s)(u, Gin, Gout, n, n_fields2, *fx, pg,
+    launch(k_squaring_bwd<true, NF>, grid2(n, n_fields2, NF), kThreads, 0, s, !pg.G)(u, Gin, Gout, n, n_fields2, *fx, pg,
                                                                           nullptr);
   else if (Gclr)
-    launch(k_squaring_bwd<false, NF, true>, dim3(blocks_for(vox(n)), groups(n_fields2, NF)), kThreads, 0, s)(
+    launch(k_squaring_bwd<false, NF, true>, dim3(blocks_for(vox(n)), groups(n_fields2, NF)), kThreads, 0, s, !pg.G)(
         u, Gin, Gout, n, n_fields2, FxArgs{}, pg, Gclr);
   else
-    launch(k_squaring_bwd<false, NF>, dim3(blocks_for(vox(n)), groups(n_fields2, NF)), kThreads, 0, s)(
+    launch(k_squaring_bwd<false, NF>, dim3(blocks_for(vox(n)), groups(n_fields2, NF)), kThreads, 0, s, !pg.G)(
         u, Gin, Gout, n, n_fields2, FxArgs{}, pg, nullptr);
 }
 // the 2-D layout puts planes x field groups on grid z (at most 65535): one field per thread
@@ -733,7 +735,7 @@ void launch_squaring_bwd(const float4* u, const float4* Gin, float4* Gout, int n
   PairGradTab t{};
   if (pg && n_fields2 <= kMaxDescPerLaunch) t = *pg;
   if (fx && dz_fits(n, n_fields2)) {
-    launch(k_squaring_bwd_dz, grid_dz(n, n_fields2), kThreads, 0, s)(u, Gin, n, *fx, t);
+    launch(k_squaring_bwd_dz, grid_dz(n, n_fields2), kThreads, 0, s, !t.G)(u, Gin, n, *fx, t);
     return;
   }
   nf = fx_nf(fx, n, n_fields2, nf);
@@ -758,9 +760,9 @@ void launch_compose(const ComposeDesc* d, int n_chains, Dims n, cudaStream_t s, 
 template <int NF>
 void compose_bwd_nf(const ComposeBwdTab& t, int n_chains, Dims n, const FxArgs* fx, cudaStream_t s) {
   if (fx)
-    launch(k_compose_bwd<true, NF>, grid2(n, n_chains, NF), kThreads, 0, s)(t, n, n_chains, *fx);
+    launch(k_compose_bwd<true, NF>, grid2(n, n_chains, NF), kThreads, 0, s, false)(t, n, n_chains, *fx);
   else
-    launch(k_compose_bwd<false, NF>, dim3(blocks_for(vox(n)), groups(n_chains, NF)), kThreads, 0, s)(t, n, n_chains,
+    launch(k_compose_bwd<false, NF>, dim3(blocks_for(vox(n)), groups(n_chains, NF)), kThreads, 0, s, false)(t, n, n_chains,
                                                                                                FxArgs{});
 }
 void launch_compose_bwd(const ComposeBwdDesc* d, int n_chains, Dims n, const FxArgs* fx, cudaStream_t s, int nf) {
@@ -769,7 +771,7 @@ void launch_compose_bwd(const ComposeBwdDesc* d, int n_chains, Dims n, const FxA
     ComposeBwdTab t;
     for (int c = 0; c < cnt; ++c) t.d[c] = d[c0 + c];
     if (fx && dz_fits(n, cnt))
-      launch(k_compose_bwd_dz, grid_dz(n, cnt), kThreads, 0, s)(t, n, *fx);
+      launch(k_compose_bwd_dz, grid_dz(n, cnt), kThreads, 0, s, false)(t, n, *fx);
     else if (fx_nf(fx, n, cnt, nf) == 1)
       compose_bwd_nf<1>(t, cnt, n, fx, s);
     else
@@ -781,7 +783,7 @@ void launch_add(const AddDesc* d, int n, Dims dims, cudaStream_t s) {
     const int cnt = std::min(kMaxDescPerLaunch, n - c0);
     AddTab t;
     for (int c = 0; c < cnt; ++c) t.d[c] = d[c0 + c];
-    launch(k_add, dim3(blocks_for(vox(dims)), cnt), kThreads, 0, s)(t, (int)vox(dims));
+    launch(k_add, dim3(blocks_for(vox(dims)), cnt), kThreads, 0, s, false)(t, (int)vox(dims));
   }
 }
 int reg_runs(Dims n) { return std::max(1, std::min(kRegRuns, (int)(blocks_for(vox(n)) / device_sm_count()))); }
