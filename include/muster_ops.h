@@ -14,6 +14,10 @@
  * the order of `stream`. The pool keeps up to 256 MiB of unused scratch between calls (so that
  * a call does not map memory anew) and gives it back when a device allocation of the
  * library fails; while `stream` is being captured, the graph owns the scratch instead.
+ *
+ * Calls that return nothing to the host (the similarity calls with loss NULL, muster_op_exp,
+ * muster_op_downsample, muster_op_jacobian_det) can be captured into a CUDA graph and replayed. A
+ * call that returns a host value waits for `stream`, which a capture does not allow.
  */
 #ifndef MUSTER_OPS_H
 #define MUSTER_OPS_H

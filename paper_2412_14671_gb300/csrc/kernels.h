@@ -219,6 +219,15 @@ void launch_jacobian_det(const float* u, Dims n, float* J, cudaStream_t s);
 size_t metrics_scratch_doubles();
 void launch_deformation_metrics(const float* ut, const float* ue, const unsigned char* roi, Dims n, double* scratch,
                                 double* out, cudaStream_t s);
+// Head of the scratch of a stateless similarity call: out and the step, flag and wait-failure words, all
+// zero at first, and the pair's descriptor. Written by a kernel that takes the descriptor by value: a copy
+// from the caller's stack would leave a captured graph with the address of a dead frame.
+struct OpHead {
+  double out[6];
+  int ints[4];
+  PairDesc pd;
+};
+void launch_op_head(OpHead* head, const PairDesc& pd, cudaStream_t s);
 // ops.cu: gives the unused scratch that the stateless calls keep back to the device
 void trim_op_pools();
 // single-CTA deterministic loss reduction; writes out[0..4], hist[*step], flag, ++*step

@@ -153,31 +153,25 @@ int muster_op_similarity(const float* F, const float* W, int64_t D, int64_t H, i
   }
   const int NC = sim_ncoef(kind);
   const SimGeom g = sim_geom(n, window, 0, kind);
-  // scratch: [head: out 6 doubles, step, flag and wait-failure ints, descriptor | partials | coefficients |
-  // F statistics]; the head starts as zeros and the descriptor, in one copy
-  struct Head {
-    double out[6];
-    int ints[4];
-    PairDesc pd;
-  };
-  const size_t off_part = (sizeof(Head) + 255) / 256 * 256;
+  // scratch: [head | partials | coefficients | F statistics]
+  const size_t off_part = (sizeof(OpHead) + 255) / 256 * 256;
   const size_t off_coef = (off_part + sizeof(double) * (size_t)g.ctas + 255) / 256 * 256;
   const size_t off_stat = off_coef + sizeof(float) * NC * V;
   const size_t bytes = off_stat + sizeof(float) * 2 * V;
   char* buf = nullptr;
   OK_(op_alloc((void**)&buf, bytes, s));
-  Head* d = (Head*)buf;
+  OpHead* d = (OpHead*)buf;
   double* part = (double*)(buf + off_part);
   float* coef = (float*)(buf + off_coef);
   float* stat = (float*)(buf + off_stat);
-  Head h{};
+  OpHead h{};
   h.pd.Ii = F;
   h.pd.Fs = stat;
-  cudaError_t e = cudaMemcpyAsync(d, &h, sizeof(h), cudaMemcpyHostToDevice, s);
   SimMaps maps;
   make_sim_maps(&maps, W, 1, F, 1, coef, n, window, kind);
-  if (e == cudaSuccess) e = prepare_kernels();
+  cudaError_t e = prepare_kernels();
   if (e == cudaSuccess) {
+    launch_op_head(d, h.pd, s);
     launch_fixed_stats(F, 1, 0, n, window, kind, eps, stat, s);
     launch_sim_fwd(&d->pd, 1, 0, 1, W, V, coef, V, part, n, window, kind, eps, &maps, d->ints + 2, s);
     if (dLdW) {
@@ -189,7 +183,7 @@ int muster_op_similarity(const float* F, const float* W, int64_t D, int64_t H, i
                        d->ints + 1, 0, s);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess && loss) e = cudaMemcpyAsync(&h, d, offsetof(Head, pd), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess && loss) e = cudaMemcpyAsync(&h, d, offsetof(OpHead, pd), cudaMemcpyDeviceToHost, s);
   cudaFreeAsync(buf, s);
   if (e != cudaSuccess) return op_cuda(e, "similarity launches");
   if (loss) {

@@ -21,10 +21,10 @@ void set_ops_error(const std::string& m);  // ops.cu
 
 namespace {
 
-// layout of the scratch: [8 doubles of results | ints | CTA partial sums | descriptor | coefficients |
-// window statistics of F]
-constexpr size_t kMaxCtas = (size_t)1 << 17;                           // partial sums of the forward kernel
-constexpr size_t kHead = (64 + 8 * kMaxCtas + 64 + 255) / 256 * 256;  // results, counters, partials, descriptor
+// layout of the scratch: [head | CTA partial sums | coefficients | window statistics of F]
+constexpr size_t kMaxCtas = (size_t)1 << 17;  // partial sums of the forward kernel
+constexpr size_t kOpHead = (sizeof(OpHead) + 255) / 256 * 256;
+constexpr size_t kHead = kOpHead + 8 * kMaxCtas;
 constexpr size_t kCoefBytes = (size_t)3 * 4 * MUSTER_NOALLOC_MAX_VOXELS;  // up to 3 coefficient volumes
 constexpr size_t kStatBytes = (size_t)2 * 4 * MUSTER_NOALLOC_MAX_VOXELS;  // mu_F and S_FF volumes
 constexpr size_t kScratchBytes = kHead + kCoefBytes + kStatBytes;
@@ -91,44 +91,39 @@ int muster_op_similarity_noalloc(const float* F, const float* W, int64_t D, int6
     return MUSTER_OK;
   }
   const SimGeom g = sim_geom(n, window, 0, kind);
-  const size_t off_part = 64, off_desc = off_part + sizeof(double) * (size_t)g.ctas;
-  if ((size_t)g.ctas > kMaxCtas || off_desc + sizeof(PairDesc) > kHead)
+  if ((size_t)g.ctas > kMaxCtas)
     return na_fail(MUSTER_EINVAL, "volume shape needs more partial sums than the fixed scratch holds");
   void* base = nullptr;
   int rc = scratch_address(&base);
   if (rc) return rc;
   char* buf = (char*)base;
-  double* out = (double*)buf;
-  int* ints = (int*)(buf + 48);
-  double* part = (double*)(buf + off_part);
-  PairDesc* pd = (PairDesc*)(buf + off_desc);
+  OpHead* d = (OpHead*)buf;
+  double* part = (double*)(buf + kOpHead);
   float* coef = (float*)(buf + kHead);
   float* stat = (float*)(buf + kHead + kCoefBytes);
-  PairDesc h{};
-  h.Ii = F;
-  h.Fs = stat;
-  // results and counters must start at zero: the array keeps the previous call's contents
-  e = cudaMemsetAsync(buf, 0, 64, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(pd, &h, sizeof(h), cudaMemcpyHostToDevice, s);
-  if (e != cudaSuccess) return na_fail(MUSTER_ECUDA, cudaGetErrorString(e));
+  PairDesc pd{};
+  pd.Ii = F;
+  pd.Fs = stat;
   SimMaps maps;
   make_sim_maps(&maps, W, 1, F, 1, coef, n, window, kind);
   if ((e = prepare_kernels()) != cudaSuccess) return na_fail(MUSTER_ECUDA, cudaGetErrorString(e));
+  // the head anew: the array keeps the previous call's contents
+  launch_op_head(d, pd, s);
   launch_fixed_stats(F, 1, 0, n, window, kind, eps, stat, s);
-  launch_sim_fwd(pd, 1, 0, 1, W, V, coef, V, part, n, window, kind, eps, &maps, ints + 2, s);
-  launch_loss_reduce(part, g.ctas, nullptr, 0, 1.0 / (double)NR, 0.0, 0.0, 0.f, 0.f, 0.f, out, nullptr, ints,
-                     ints + 1, 0, s);
+  launch_sim_fwd(&d->pd, 1, 0, 1, W, V, coef, V, part, n, window, kind, eps, &maps, d->ints + 2, s);
+  launch_loss_reduce(part, g.ctas, nullptr, 0, 1.0 / (double)NR, 0.0, 0.0, 0.f, 0.f, 0.f, d->out, nullptr, d->ints,
+                     d->ints + 1, 0, s);
   if (dLdW) {
     const int nw = window * window * window;
     const float scale = kind == MUSTER_SILNCC ? (float)(2.0 / ((double)nw * (double)NR)) : (float)(1.0 / (double)NR);
-    launch_sim_bwd(pd, 1, 0, 1, W, V, coef, V, dLdW, n, window, kind, scale, &maps, ints + 2, s);
+    launch_sim_bwd(&d->pd, 1, 0, 1, W, V, coef, V, dLdW, n, window, kind, scale, &maps, d->ints + 2, s);
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return na_fail(MUSTER_ECUDA, cudaGetErrorString(e));
   if (loss) {
     double host_out[2] = {0.0, 0.0};
     int host_err = 0;
-    if ((e = cudaMemcpyAsync(host_out, out, sizeof(double) * 2, cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(&host_err, ints + 2, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+    if ((e = cudaMemcpyAsync(host_out, d->out, sizeof(double) * 2, cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+        (e = cudaMemcpyAsync(&host_err, d->ints + 2, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
         (e = cudaStreamSynchronize(s)) != cudaSuccess)
       return na_fail(MUSTER_ECUDA, cudaGetErrorString(e));
     if (host_err) return na_fail(MUSTER_ETIMEOUT, "a bounded wait for an input copy ran out");
