@@ -125,7 +125,8 @@ typedef struct {
                              Chunks change where the window sums restart and the order of the
                              loss partial sums, so results differ in the last bits between values
                              (each value is reproducible) */
-  /* optional device allocator (e.g. a framework's caching allocator); both or neither */
+  /* optional device allocator (e.g. a framework's caching allocator); both or neither. A block
+     that alloc refuses (NULL) is asked for once more before the call gives up */
   void* (*alloc)(size_t bytes, void* user);
   void (*free)(void* ptr, void* user);
   void* alloc_user;

@@ -12,8 +12,10 @@
  *
  * Scratch comes from a memory pool of the library on the current device and is released in
  * the order of `stream`. The pool keeps up to 256 MiB of unused scratch between calls (so that
- * a call does not map memory anew) and gives it back when a device allocation of the
- * library fails; while `stream` is being captured, the graph owns the scratch instead.
+ * a call does not map memory anew). When a device allocation of the library fails, by
+ * cudaMalloc or by a context's alloc callback, the scratch that the device has released
+ * by then goes back and the allocation is tried once more. While `stream` is being captured,
+ * the graph owns the scratch instead.
  *
  * Calls that return nothing to the host (the similarity calls with loss NULL, muster_op_exp,
  * muster_op_downsample, muster_op_jacobian_det) can be captured into a CUDA graph and replayed. A

@@ -220,16 +220,17 @@ int check_launch(muster_ctx* ctx, const char* where) {
 
 void* dalloc(muster_ctx* ctx, size_t bytes) {
   if (bytes == 0) bytes = 16;
-  void* ptr = nullptr;
-  if (ctx->p.alloc) {
-    ptr = ctx->p.alloc(bytes, ctx->p.alloc_user);
-  } else if (cudaMalloc(&ptr, bytes) != cudaSuccess) {
+  auto get = [&]() -> void* {
+    if (ctx->p.alloc) return ctx->p.alloc(bytes, ctx->p.alloc_user);
+    void* p = nullptr;
+    if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
     cudaGetLastError();
+    return nullptr;
+  };
+  void* ptr = get();
+  if (!ptr) {  // the stateless calls' unused scratch may make room, whoever allocates
     trim_op_pools();
-    if (cudaMalloc(&ptr, bytes) != cudaSuccess) {
-      cudaGetLastError();
-      ptr = nullptr;
-    }
+    ptr = get();
   }
   if (ptr) ctx->allocs.push_back(ptr);
   return ptr;

@@ -37,8 +37,9 @@ bool dims_ok(int64_t D, int64_t H, int64_t W) {
 // ---- scratch of the stateless calls: a memory pool of the library per device. The default pool gives
 // everything back at each synchronisation, so a call that returns a number to the host paid for
 // mapping its scratch again every time (about 200 us of the 290 us of a 48^3 similarity). This one
-// keeps at most kPoolKeep bytes of unused scratch; a failed allocation, of a call here or of a
-// context, gives all of it back first. Allocation and release are ordered by the caller's stream.
+// keeps at most kPoolKeep bytes of unused scratch; after a failed allocation, of a call here or of a
+// context (by cudaMalloc or its own callback), what the device has released goes back and the
+// allocation is tried once more. Allocation and release are ordered by the caller's stream.
 namespace {
 constexpr uint64_t kPoolKeep = (uint64_t)256 << 20;
 std::mutex g_pool_mu;
