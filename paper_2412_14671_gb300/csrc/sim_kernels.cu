@@ -194,16 +194,31 @@ struct Box {
   static constexpr int WT = (NTASK + 31) / 32 * 32;         // W threads
   static constexpr int NT = kHD + WT;
   static constexpr int PX = R <= 2 ? 36 : 44;               // row pitch of a staged plane
-  static constexpr int PS = 36;                             // row pitch of the W sums
   static constexpr int TS = (RY * PX + 31) & ~31;           // floats of one staged plane (128-byte multiple)
-  static_assert(PX >= kTX - kXO + 4 * NV && PX % 8 == 4 && PS % 8 == 4, "pitches");
-  __host__ __device__ static constexpr int sx_floats(int nm) { return nm * RY * PS; }
+  static_assert(PX >= kTX - kXO + 4 * NV && PX % 8 == 4, "pitch");
+  __host__ __device__ static constexpr int sx_floats(int nm) { return nm * RY * kTX; }
   __host__ __device__ static constexpr int ring_floats(int nm) { return WW * nm * kTX * kTY; }
-  // dynamic shared memory: [2 stages][nin][TS], [2 planes][nm] W sums, D ring
+  // dynamic shared memory: [2 stages][nin][TS] without the last one's padding, [2 planes][nm] W sums, D
+  // ring, two mbarriers
+  __host__ __device__ static constexpr int sx_at(int nin) { return (2 * nin - 1) * TS + RY * PX; }
+  __host__ __device__ static constexpr int bar_at(int nin, int nm) {
+    return sx_at(nin) + 2 * sx_floats(nm) + ring_floats(nm);
+  }
+  static_assert(RY * PX % 4 == 0, "the W sums and the ring are moved by 16 bytes");
   __host__ __device__ static constexpr size_t bytes(int nin, int nm) {
-    return sizeof(float) * (size_t)(2 * nin * TS + 2 * sx_floats(nm) + ring_floats(nm));
+    return sizeof(float) * (size_t)bar_at(nin, nm) + 2 * sizeof(uint64_t);
+  }
+  // CTAs that an SM's 228 KB hold (1 KB of each CTA's share is the system's, shares are multiples of
+  // 128 bytes), 4 at most: the register budget is cut for these. Cut for 3, the SiLNCC forward of w = 7 takes 12 %
+  // longer; cut for 4 where only 2 fit, the kernels of w = 11 spilled 76 to 92 bytes.
+  static constexpr int min_ctas(int nin, int nm) {
+    const size_t fit = (228 << 10) / ((bytes(nin, nm) + 1024 + 127) / 128 * 128);
+    return fit > 4 ? 4 : (int)fit;
   }
 };
+// position of W sum x of row r, without its row's base: odd rows swap neighbouring runs of 4, so that the two rows
+// that 8 lanes of a W warp write with 16-byte stores take all banks once
+__device__ __forceinline__ int sx_col(int x, int r) { return x ^ (4 * (r & 1)); }
 
 // x offset of the adjoint's staged box: its first column x0 - 2R is rounded down to a
 // multiple of 4 (16-byte aligned tile coordinate), so the box starts XOFF columns early
@@ -432,24 +447,23 @@ struct Stages {
   }
 };
 
-// the 8 sums of one moment of a W task, of values or of products, into the W sums
-__device__ __forceinline__ void store8(float* __restrict__ dst, const float (&o)[kXO]) {
-  *reinterpret_cast<float4*>(dst) = make_float4(o[0], o[1], o[2], o[3]);
-  *reinterpret_cast<float4*>(dst + 4) = make_float4(o[4], o[5], o[6], o[7]);
-}
+// the 8 sums of one moment of a W task, of values or of products, into the W sums: the first 4 to
+// d0, the others to d1
 template <int R>
-__device__ __forceinline__ void w_sums(const float* v, float* __restrict__ dst) {
+__device__ __forceinline__ void w_sums(const float* v, float* __restrict__ d0, float* __restrict__ d1) {
   float o[kXO];
   runsum<Box<R>::WW, 4>(v, o);
   runsum<Box<R>::WW, 4>(v + 4, o + 4);
-  store8(dst, o);
+  *reinterpret_cast<float4*>(d0) = make_float4(o[0], o[1], o[2], o[3]);
+  *reinterpret_cast<float4*>(d1) = make_float4(o[4], o[5], o[6], o[7]);
 }
 template <int R>
-__device__ __forceinline__ void w_sums(const float* a, const float* b, float* __restrict__ dst) {
+__device__ __forceinline__ void w_sums(const float* a, const float* b, float* __restrict__ d0, float* __restrict__ d1) {
   float o[kXO];
   runsum4<Box<R>::WW>(a, b, o);
   runsum4<Box<R>::WW>(a + 4, b + 4, o + 4);
-  store8(dst, o);
+  *reinterpret_cast<float4*>(d0) = make_float4(o[0], o[1], o[2], o[3]);
+  *reinterpret_cast<float4*>(d1) = make_float4(o[4], o[5], o[6], o[7]);
 }
 
 // H and D passes of one plane for a thread's column and rows: S += newest - oldest plane sum,
@@ -474,13 +488,15 @@ struct Ring {
   __device__ __forceinline__ void plane(const float* sx2, int h, int niter, int col, int row) {
     using B = Box<R>;
     bar_sync(kBarFull + (h & 1), B::NT);
-    const float* sx = sx2 + (h & 1) * B::sx_floats(NM) + row * B::PS + col;
+    static_assert(kYO % 2 == 0, "a thread's first row is even");
+    const float* sx = sx2 + (h & 1) * B::sx_floats(NM) + row * kTX;
+    const float* sxk[2] = {sx + sx_col(col, 0), sx + sx_col(col, 1)};
     float a[NM][kYO];
 #pragma unroll
     for (int m = 0; m < NM; ++m) {
       float v[kYO + 2 * R];
 #pragma unroll
-      for (int k = 0; k < kYO + 2 * R; ++k) v[k] = sx[(m * B::RY + k) * B::PS];
+      for (int k = 0; k < kYO + 2 * R; ++k) v[k] = sxk[k & 1][(m * B::RY + k) * kTX];
 #pragma unroll
       for (int i = 0; i < kYO; i += 2) runsum<B::WW, 2>(v + i, a[m] + i);
     }
@@ -525,12 +541,9 @@ __device__ __forceinline__ int corners_holding(int k, int last, int reach) {
   return max(0, min(k, last) - max(0, k - reach) + 1);
 }
 
-// CTAs per SM the register budget is cut for (shared memory allows 4 for w <= 7)
-constexpr int kMinCtas = 4;
-
 // Forward of one pair (see the head of the file).
 template <int R, int KIND, bool TMA>
-__global__ void __launch_bounds__(Box<R>::NT, kMinCtas)
+__global__ void __launch_bounds__(Box<R>::NT, Box<R>::min_ctas(2, KIND == 0 ? 2 : 3))
     k_sim_fwd(const __grid_constant__ SimMaps maps, const PairDesc* __restrict__ pd, const float* __restrict__ Wb,
               size_t Wstride, float* __restrict__ coef, size_t cstride, double* __restrict__ part, Dims n, Tiles g,
               float eps, int* __restrict__ err) {
@@ -538,9 +551,8 @@ __global__ void __launch_bounds__(Box<R>::NT, kMinCtas)
   using B = Box<R>;
   constexpr int NM = KIND == 0 ? 2 : 3, NC = KIND == 0 ? 2 : 3;
   extern __shared__ __align__(128) float smem[];
-  float* sx2 = smem + 4 * B::TS;  // stages: [2][F, W][TS]
-  __shared__ __align__(8) uint64_t bar[2];
-  __shared__ float sh[2 * (B::NT / 32)];
+  float* sx2 = smem + B::sx_at(2);  // stages: [2][F, W][TS]
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + B::bar_at(2, NM));
   const Tile t = tile_of(g);
   const int plane = n.n1 * n.n2;
   const PairDesc d = pd[t.pair];
@@ -582,10 +594,12 @@ __global__ void __launch_bounds__(Box<R>::NT, kMinCtas)
           f[4 * q] = a.x - shF, f[4 * q + 1] = a.y - shF, f[4 * q + 2] = a.z - shF, f[4 * q + 3] = a.w - shF;
           w[4 * q] = b.x - shW, w[4 * q + 1] = b.y - shW, w[4 * q + 2] = b.z - shW, w[4 * q + 3] = b.w - shW;
         }
-        float* sx = sx2 + (it & 1) * B::sx_floats(NM) + row * B::PS + xs;
-        w_sums<R>(w, sx);
-        w_sums<R>(f, w, sx + (NM - 1) * B::RY * B::PS);
-        if (KIND == 1) w_sums<R>(w, w, sx + B::RY * B::PS);
+        float* sx = sx2 + (it & 1) * B::sx_floats(NM) + row * kTX;
+        float *d0 = sx + sx_col(xs, row), *d1 = sx + sx_col(xs + 4, row);
+        constexpr int M = B::RY * kTX;
+        w_sums<R>(w, d0, d1);
+        w_sums<R>(f, w, d0 + (NM - 1) * M, d1 + (NM - 1) * M);
+        if (KIND == 1) w_sums<R>(w, w, d0 + M, d1 + M);
       }
       bar_arrive(kBarFull + (it & 1), B::NT);
       if (KIND == 0) {
@@ -694,12 +708,13 @@ __global__ void __launch_bounds__(Box<R>::NT, kMinCtas)
     }
   }
   const float sgn = KIND == 0 && wt < 0 ? -1.f : 1.f;
-  const double sum = block_sum<B::NT>(FF{sgn * acc.hi, sgn * acc.lo}, sh);
+  // the warp sums take the place of the W sums, which no thread reads any more past the barrier
+  const double sum = block_sum<B::NT>(FF{sgn * acc.hi, sgn * acc.lo}, sx2);
   if (threadIdx.x == 0) part[t.part] = KIND == 0 ? sum / (double)(B::WW * B::WW * B::WW) : sum;
 }
 
 template <int R, int KIND, bool TMA>
-__global__ void __launch_bounds__(Box<R>::NT, kMinCtas)
+__global__ void __launch_bounds__(Box<R>::NT, Box<R>::min_ctas(KIND == 0 ? 2 : 3, KIND == 0 ? 2 : 3))
     k_sim_bwd(const __grid_constant__ SimMaps maps, const PairDesc* __restrict__ pd, const float* __restrict__ Wb,
               size_t Wstride, const float* __restrict__ coef, size_t cstride, float* __restrict__ dLdW, Dims n, Tiles g,
               float scale, int* __restrict__ err) {
@@ -708,8 +723,8 @@ __global__ void __launch_bounds__(Box<R>::NT, kMinCtas)
   constexpr int NC = KIND == 0 ? 2 : 3, XOFF = TMA ? bwd_xoff<R>() : 0;
   static_assert(!TMA || (2 * R + XOFF) % 4 == 0, "the staged adjoint box must start at a multiple of 4 floats");
   extern __shared__ __align__(128) float smem[];
-  float* sx2 = smem + 2 * NC * B::TS;  // stages: [2][NC][TS]
-  __shared__ __align__(8) uint64_t bar[2];
+  float* sx2 = smem + B::sx_at(NC);  // stages: [2][NC][TS]
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + B::bar_at(NC, NC));
   const Tile t = tile_of(g);
   const int plane = n.n1 * n.n2;
   const int zend = min(t.z0 + g.tz, n.n0), niter = (zend - t.z0) + 2 * R;
@@ -737,7 +752,8 @@ __global__ void __launch_bounds__(Box<R>::NT, kMinCtas)
       if (it >= 2) bar_sync(kBarEmpty + (it & 1), B::NT);
       st.wait(it);
       if (on) {
-        float* sx = sx2 + (it & 1) * B::sx_floats(NC) + row * B::PS + xs;
+        float* sx = sx2 + (it & 1) * B::sx_floats(NC) + row * kTX;
+        float *d0 = sx + sx_col(xs, row), *d1 = sx + sx_col(xs + 4, row);
 #pragma unroll
         for (int m = 0; m < NC; ++m) {
           float v[4 * B::NV];
@@ -747,7 +763,7 @@ __global__ void __launch_bounds__(Box<R>::NT, kMinCtas)
             const float4 a = src[q];
             v[4 * q] = a.x, v[4 * q + 1] = a.y, v[4 * q + 2] = a.z, v[4 * q + 3] = a.w;
           }
-          w_sums<R>(v + XOFF, sx + m * B::RY * B::PS);
+          w_sums<R>(v + XOFF, d0 + m * B::RY * kTX, d1 + m * B::RY * kTX);
         }
       }
       bar_arrive(kBarFull + (it & 1), B::NT);
