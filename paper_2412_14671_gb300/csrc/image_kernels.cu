@@ -98,13 +98,8 @@ __global__ void __launch_bounds__(4 * kThreads)
   }
 }
 
-__global__ void k_op_head(OpHead* __restrict__ head, PairDesc pd) {
-  grid_begin();
-  *head = OpHead{{}, {}, pd};
-}
 }  // namespace
 
-void launch_op_head(OpHead* head, const PairDesc& pd, cudaStream_t s) { launch(k_op_head, 1, 1, 0, s)(head, pd); }
 void launch_down2(const float* in, Dims n, float* out, Dims m, int n_images, cudaStream_t s) {
   launch(k_down2, dim3(blocks_for(vox(m)), n_images), kThreads, 0, s)(in, n, out, m);
 }

@@ -155,10 +155,19 @@ SimGeom sim_geom(Dims ni, int window, int batch, int kind = 0);  // sim_kernels.
 // kernel attributes (dynamic shared memory limits), set once per device; call with the
 // device current before any launch or capture on it
 cudaError_t prepare_kernels();
+// Head of the scratch of a stateless similarity call: out and the step, flag and wait-failure words, all
+// zero at first, and the pair's descriptor.
+struct OpHead {
+  double out[6];
+  int ints[4];
+  PairDesc pd;
+};
 // mu_F and S_FF of every window corner of each image: stats = n_images x 2 planes; with
-// kind 0 (SiLNCC) the second plane holds 1 / (S_FF + eps) instead of S_FF
+// kind 0 (SiLNCC) the second plane holds 1 / (S_FF + eps) instead of S_FF. head (nullable): written too,
+// from pd by value. A copy from the caller's stack would leave a captured graph with the address of a dead
+// frame, and a kernel of its own would add 3 us to a 48^3 call.
 void launch_fixed_stats(const float* imgs, int n_images, int batch, Dims ni, int window, int kind, float eps,
-                        float* stats, cudaStream_t s);
+                        float* stats, cudaStream_t s, OpHead* head = nullptr, const PairDesc& pd = PairDesc{});
 int sim_ncoef(int kind);
 // maps for W (capacity n_pairs volumes), the n_images fixed images and the coefficient
 // buffer (n_pairs * NC volumes), all with stride nvox(ni) between volumes
@@ -219,15 +228,6 @@ void launch_jacobian_det(const float* u, Dims n, float* J, cudaStream_t s);
 size_t metrics_scratch_doubles();
 void launch_deformation_metrics(const float* ut, const float* ue, const unsigned char* roi, Dims n, double* scratch,
                                 double* out, cudaStream_t s);
-// Head of the scratch of a stateless similarity call: out and the step, flag and wait-failure words, all
-// zero at first, and the pair's descriptor. Written by a kernel that takes the descriptor by value: a copy
-// from the caller's stack would leave a captured graph with the address of a dead frame.
-struct OpHead {
-  double out[6];
-  int ints[4];
-  PairDesc pd;
-};
-void launch_op_head(OpHead* head, const PairDesc& pd, cudaStream_t s);
 // ops.cu: gives the unused scratch that the stateless calls keep back to the device
 void trim_op_pools();
 // single-CTA deterministic loss reduction; writes out[0..4], hist[*step], flag, ++*step

@@ -172,8 +172,7 @@ int muster_op_similarity(const float* F, const float* W, int64_t D, int64_t H, i
   make_sim_maps(&maps, W, 1, F, 1, coef, n, window, kind);
   cudaError_t e = prepare_kernels();
   if (e == cudaSuccess) {
-    launch_op_head(d, h.pd, s);
-    launch_fixed_stats(F, 1, 0, n, window, kind, eps, stat, s);
+    launch_fixed_stats(F, 1, 0, n, window, kind, eps, stat, s, d, h.pd);
     launch_sim_fwd(&d->pd, 1, 0, 1, W, V, coef, V, part, n, window, kind, eps, &maps, d->ints + 2, s);
     if (dLdW) {
       const int nw = window * window * window;

@@ -107,9 +107,8 @@ int muster_op_similarity_noalloc(const float* F, const float* W, int64_t D, int6
   SimMaps maps;
   make_sim_maps(&maps, W, 1, F, 1, coef, n, window, kind);
   if ((e = prepare_kernels()) != cudaSuccess) return na_fail(MUSTER_ECUDA, cudaGetErrorString(e));
-  // the head anew: the array keeps the previous call's contents
-  launch_op_head(d, pd, s);
-  launch_fixed_stats(F, 1, 0, n, window, kind, eps, stat, s);
+  // the head is written anew: the array keeps the previous call's contents
+  launch_fixed_stats(F, 1, 0, n, window, kind, eps, stat, s, d, pd);
   launch_sim_fwd(&d->pd, 1, 0, 1, W, V, coef, V, part, n, window, kind, eps, &maps, d->ints + 2, s);
   launch_loss_reduce(part, g.ctas, nullptr, 0, 1.0 / (double)NR, 0.0, 0.0, 0.f, 0.f, 0.f, d->out, nullptr, d->ints,
                      d->ints + 1, 0, s);

@@ -75,8 +75,10 @@ constexpr int kStatThreads = 128, TX = 32;  // k_fixed_stats
 // Every sum adds its terms one after the other.
 template <int R, int KIND>
 __global__ void __launch_bounds__(kStatThreads) k_fixed_stats(const float* __restrict__ imgs, float* __restrict__ stats,
-                                                              Dims n, int tz, int nzc, float eps) {
+                                                              Dims n, int tz, int nzc, float eps,
+                                                              OpHead* __restrict__ head, PairDesc pd) {
   grid_begin();
+  if (head && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) *head = OpHead{{}, {}, pd};
   constexpr int WW = 2 * R + 1, TY = 8, RX = TX + 2 * R, RY = TY + 2 * R, PF = (RX + 3) / 4 * 4;
   constexpr int NE = RY * RX, NSLOT = (NE + kStatThreads - 1) / kStatThreads;
   constexpr int NO = 4, NI = NO + 2 * R, NV = (NI + 3) / 4, NR = TY * TX / kStatThreads;
@@ -967,27 +969,27 @@ unsigned ctas(const Tiles& g) { return (unsigned)g.gx * g.gy * g.nzc * g.np; }
 
 template <int KIND>
 void fixed_stats(dim3 g, const float* imgs, Dims ni, int window, float eps, float* stats, int tz, int nzc,
-                 cudaStream_t s) {
+                 OpHead* head, const PairDesc& pd, cudaStream_t s) {
   switch (window / 2) {
-    case 1: launch(k_fixed_stats<1, KIND>, g, kStatThreads, 0, s)(imgs, stats, ni, tz, nzc, eps); break;
-    case 2: launch(k_fixed_stats<2, KIND>, g, kStatThreads, 0, s)(imgs, stats, ni, tz, nzc, eps); break;
-    case 3: launch(k_fixed_stats<3, KIND>, g, kStatThreads, 0, s)(imgs, stats, ni, tz, nzc, eps); break;
-    case 4: launch(k_fixed_stats<4, KIND>, g, kStatThreads, 0, s)(imgs, stats, ni, tz, nzc, eps); break;
-    case 5: launch(k_fixed_stats<5, KIND>, g, kStatThreads, 0, s)(imgs, stats, ni, tz, nzc, eps); break;
+    case 1: launch(k_fixed_stats<1, KIND>, g, kStatThreads, 0, s)(imgs, stats, ni, tz, nzc, eps, head, pd); break;
+    case 2: launch(k_fixed_stats<2, KIND>, g, kStatThreads, 0, s)(imgs, stats, ni, tz, nzc, eps, head, pd); break;
+    case 3: launch(k_fixed_stats<3, KIND>, g, kStatThreads, 0, s)(imgs, stats, ni, tz, nzc, eps, head, pd); break;
+    case 4: launch(k_fixed_stats<4, KIND>, g, kStatThreads, 0, s)(imgs, stats, ni, tz, nzc, eps, head, pd); break;
+    case 5: launch(k_fixed_stats<5, KIND>, g, kStatThreads, 0, s)(imgs, stats, ni, tz, nzc, eps, head, pd); break;
     default: break;
   }
 }
 }  // namespace
 
 void launch_fixed_stats(const float* imgs, int n_images, int batch, Dims ni, int window, int kind, float eps,
-                        float* stats, cudaStream_t s) {
+                        float* stats, cudaStream_t s, OpHead* head, const PairDesc& pd) {
   const int gx = (ni.n2 + TX - 1) / TX, gy = (ni.n1 + 7) / 8;
   const int tz = chunk_planes(gx * gy, ni, window, kind, 16, 128, batch), nzc = (ni.n0 + tz - 1) / tz;
   const dim3 g(gx, gy, nzc * n_images);
   if (kind == 0)
-    fixed_stats<0>(g, imgs, ni, window, eps, stats, tz, nzc, s);
+    fixed_stats<0>(g, imgs, ni, window, eps, stats, tz, nzc, head, pd, s);
   else
-    fixed_stats<1>(g, imgs, ni, window, eps, stats, tz, nzc, s);
+    fixed_stats<1>(g, imgs, ni, window, eps, stats, tz, nzc, head, pd, s);
 }
 
 cudaError_t prepare_kernels() {
