@@ -22,7 +22,7 @@
 
 namespace muster {
 
-// Every kernel starts with grid_begin() and is launched with launch(): its CTAs may take their places
+// Every kernel starts with grid_begin() or grid_wait() and is launched with launch(): its CTAs may take their places
 // while the last ones of its predecessor in the stream still run, and wait there until that
 // kernel has finished and its writes are visible, so a chain of small kernels pays no drain, dispatch and
 // ramp between two of them. No kernel touches memory before the wait; results of earlier kernels
@@ -36,6 +36,11 @@ namespace muster {
 __device__ __forceinline__ void grid_begin() {
   asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
 }
+// For kernels whose CTAs run long (the window sums): their dependents start when the CTAs have exited, which still
+// hides the launch. Started with the last CTAs they would crowd onto the SMs that those leave free, several on
+// one, and stay there (similarity and gradient of one pair with grid_begin, then with this: 80^3, w = 7, SiLNCC 85
+// and 75 us; LNCC 128^3, w = 3, 64 CTAs, 262 and 189 us, 160 x 192 x 161, w = 7, 777 and 586 us).
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // launch(kernel, grid, block, dynamic shared memory, stream)(arguments)
 template <class... P>
 auto launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t shared, cudaStream_t s, bool overlap = true) {

@@ -77,7 +77,7 @@ template <int R, int KIND>
 __global__ void __launch_bounds__(kStatThreads) k_fixed_stats(const float* __restrict__ imgs, float* __restrict__ stats,
                                                               Dims n, int tz, int nzc, float eps,
                                                               OpHead* __restrict__ head, PairDesc pd) {
-  grid_begin();
+  grid_wait();
   if (head && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) *head = OpHead{{}, {}, pd};
   constexpr int WW = 2 * R + 1, TY = 8, RX = TX + 2 * R, RY = TY + 2 * R, PF = (RX + 3) / 4 * 4;
   constexpr int NE = RY * RX, NSLOT = (NE + kStatThreads - 1) / kStatThreads;
@@ -549,7 +549,7 @@ __global__ void __launch_bounds__(Box<R>::NT, Box<R>::min_ctas(2, KIND == 0 ? 2 
     k_sim_fwd(const __grid_constant__ SimMaps maps, const PairDesc* __restrict__ pd, const float* __restrict__ Wb,
               size_t Wstride, float* __restrict__ coef, size_t cstride, double* __restrict__ part, Dims n, Tiles g,
               float eps, int* __restrict__ err) {
-  grid_begin();
+  grid_wait();
   using B = Box<R>;
   constexpr int NM = KIND == 0 ? 2 : 3, NC = KIND == 0 ? 2 : 3;
   extern __shared__ __align__(128) float smem[];
@@ -720,7 +720,7 @@ __global__ void __launch_bounds__(Box<R>::NT, Box<R>::min_ctas(KIND == 0 ? 2 : 3
     k_sim_bwd(const __grid_constant__ SimMaps maps, const PairDesc* __restrict__ pd, const float* __restrict__ Wb,
               size_t Wstride, const float* __restrict__ coef, size_t cstride, float* __restrict__ dLdW, Dims n, Tiles g,
               float scale, int* __restrict__ err) {
-  grid_begin();
+  grid_wait();
   using B = Box<R>;
   constexpr int NC = KIND == 0 ? 2 : 3, XOFF = TMA ? bwd_xoff<R>() : 0;
   static_assert(!TMA || (2 * R + XOFF) % 4 == 0, "the staged adjoint box must start at a multiple of 4 floats");
@@ -966,7 +966,6 @@ Tiles sim_tiles(Dims ni, int window, int kind, int n_pairs, int batch, int group
   return g;
 }
 unsigned ctas(const Tiles& g) { return (unsigned)g.gx * g.gy * g.nzc * g.np; }
-
 template <int KIND>
 void fixed_stats(dim3 g, const float* imgs, Dims ni, int window, float eps, float* stats, int tz, int nzc,
                  OpHead* head, const PairDesc& pd, cudaStream_t s) {
