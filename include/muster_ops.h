@@ -95,8 +95,9 @@ int muster_op_jacobian_det(const float* u, int64_t D, int64_t H, int64_t W, floa
    trace(A)/3 of the least-squares fit u_est = A u_true + b; [3..11] A row-major;
    [12..14] b; [15] the number of ROI voxels (all 0 when it is 0). Each voxel's terms and
    each thread's running sums are double-float values (a pair of floats, about 48
-   significant bits); the per-CTA and final sums are FP64 in a fixed order over a grid of
-   three CTAs per SM (at most 768), so a device gives the same result on every run.
+   significant bits, at any number of terms); the per-CTA sums have the precision of FP64
+   and the final sums are FP64, in a fixed order over a grid of three CTAs per SM (at most
+   768), so a device gives the same result on every run.
    Takes about 150 KB of device scratch; synchronises `stream`. */
 int muster_op_deformation_metrics(const float* u_true, const float* u_est, const uint8_t* roi, int64_t D,
                                   int64_t H, int64_t W, double out[16], void* stream);
