@@ -125,6 +125,10 @@ typedef struct {
                              Chunks change where the window sums restart and the order of the
                              loss partial sums, so results differ in the last bits between values
                              (each value is reproducible) */
+  int plain_images;       /* the forward warp samples cells (I(x), I(x + 1) - I(x)) of the images, 8 bytes
+                             per voxel, session and level beside the images' 4 and their statistics' 8
+                             (with a border of one cell). 0: when the device has room for them after
+                             everything else, 1: never. The results do not depend on it */
   /* optional device allocator (e.g. a framework's caching allocator); both or neither. A block
      that alloc refuses (NULL) is asked for once more before the call gives up */
   void* (*alloc)(size_t bytes, void* user);
@@ -141,7 +145,8 @@ void muster_default_params(muster_params* p);
 /* Creates a context for n_sessions (>= 2) images of shape[3] = (D, H, W) voxels
    with spacing[3] mm (recorded and reported; the objective is in voxel units).
    Allocates every device buffer of the whole schedule up front; MUSTER_EOOM if
-   they do not fit. *out is NULL on failure. */
+   they do not fit (without the cells of plain_images, which it can do without).
+   *out is NULL on failure. */
 int muster_create(const int64_t shape[3], int n_sessions, const double spacing[3],
                   const muster_params* params, muster_ctx** out);
 
@@ -185,7 +190,8 @@ int muster_run(muster_ctx* ctx, double* final_loss);
 int muster_advance(muster_ctx* ctx, int max_steps, int* finished);
 
 /* Device bytes that muster_create would allocate for this problem (for admission
-   control of concurrent registrations). No device is needed. */
+   control of concurrent registrations), the cells among them unless plain_images is 1.
+   No device is needed. */
 int muster_footprint(const int64_t shape[3], int n_sessions, const muster_params* params, size_t* bytes);
 
 /* Loss and gradient at `level` for parameters v (device, (N-1,3,d,h,w) of that level's

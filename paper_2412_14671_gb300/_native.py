@@ -51,6 +51,7 @@ class MusterParams(ctypes.Structure):
         ("rigid_lr", ctypes.c_float),
         ("flow_nf", ctypes.c_int),
         ("chunk_pct", ctypes.c_int),
+        ("plain_images", ctypes.c_int),
         ("alloc", ALLOC_FN),
         ("free", FREE_FN),
         ("alloc_user", ctypes.c_void_p),

@@ -104,7 +104,7 @@ struct muster_ctx {
   std::string err;
   std::vector<Dims> ni, nf;
   std::vector<float*> imgs;
-  std::vector<float2*> cells;  // per level: the cells of every image (moving images of the warp)
+  std::vector<float2*> cells;  // per level: the cells of every image (moving images of the warp); empty without cells
   std::vector<float*> fstats;  // per level: window statistics (mu_F, S_FF or 1/(S_FF+eps)) of every session
   std::vector<double> times;
   bool have_images = false;
@@ -411,7 +411,8 @@ int build_all_tables(muster_ctx* ctx) {
       for (int k = 0; k < N; ++k) {
         if (k == i) continue;
         PairDesc d;
-        d.Ic = ctx->cells[l] + (size_t)k * image_cells(ctx->ni[l]);
+        d.Ic = ctx->cells.empty() ? nullptr : ctx->cells[l] + (size_t)k * image_cells(ctx->ni[l]);
+        d.Ik = im + (size_t)k * Vi;
         d.Ii = im + (size_t)i * Vi;
         d.Fs = ctx->fstats[l] + (size_t)i * 2 * Vi;
         d.fi = i;
@@ -586,7 +587,7 @@ int forward_adjoint(muster_ctx* ctx, int l, const float4* th) {
       {
         // I_k once per moving session, U per pair, W and grad I_k per pair-voxel
         Scope s(ctx, KK_WARP, (double)n_moving * Vi * 4.0 + (double)nb * (Vi * 16.0 + Vf * 16.0));
-        launch_warp(pd, nb, ni, nf, ctx->Wbuf, ctx->gI, Vi, ctx->rigid ? ctx->rig_tab : nullptr, ctx->stream);
+        launch_warp(pd, nb, !ctx->cells.empty(), ni, nf, ctx->Wbuf, ctx->gI, Vi, ctx->rigid ? ctx->rig_tab : nullptr, ctx->stream);
       }
       {
         // W and the NC coefficient volumes per pair; F, mu_F and S_FF once per fixed session
@@ -756,6 +757,7 @@ int validate_params(const muster_params* p, std::string& why) {
   if (p->rigid && !(p->lr > 0.f)) return why = "rigid registration needs lr > 0", 1;
   if (p->flow_nf < 0 || p->flow_nf > 2) return why = "flow_nf must be 0, 1 or 2", 1;
   if (p->chunk_pct < 0 || p->chunk_pct > 800) return why = "chunk_pct must be 0..800", 1;
+  if (p->plain_images != 0 && p->plain_images != 1) return why = "plain_images must be 0 or 1", 1;
   return 0;
 }
 
@@ -973,13 +975,11 @@ int create_impl(const int64_t shape[3], int n_sessions, const double spacing[3],
   const int L = ctx->L;
   ctx->imgs.resize(L);
   ctx->fstats.resize(L);
-  ctx->cells.resize(L);
   for (int l = 0; l < L; ++l) {
-    // images and their cells share an allocation
+    // images and their statistics share an allocation
     const size_t img_bytes = (sizeof(float) * ctx->N * nvox(ctx->ni[l]) + 255) / 256 * 256;
-    ctx->imgs[l] = (float*)A(img_bytes + sizeof(float2) * ctx->N * image_cells(ctx->ni[l]));
-    if (ctx->imgs[l]) ctx->cells[l] = (float2*)((char*)ctx->imgs[l] + img_bytes);
-    ctx->fstats[l] = (float*)A(sizeof(float) * 2 * ctx->N * nvox(ctx->ni[l]));
+    ctx->imgs[l] = (float*)A(img_bytes + sizeof(float) * 2 * ctx->N * nvox(ctx->ni[l]));
+    if (ctx->imgs[l]) ctx->fstats[l] = (float*)((char*)ctx->imgs[l] + img_bytes);
   }
   ctx->theta = (float4*)A(sizeof(float4) * F * Vf);
   ctx->theta_tmp = (float4*)A(sizeof(float4) * F * Vf);
@@ -1028,6 +1028,18 @@ int create_impl(const int64_t shape[3], int n_sessions, const double spacing[3],
     ctx->gmax_dev = (unsigned*)A(sizeof(unsigned) * 4);
   }
   ctx->d_pairs_all = (PairDesc*)A(sizeof(PairDesc) * P * L);
+  // the cells of every level come last, in one block: a device that has no room for them still runs the
+  // series, on the images themselves
+  if (!params->plain_images && ok) {
+    std::vector<size_t> at(L);
+    size_t bytes = 0;
+    for (int l = 0; l < L; ++l) at[l] = bytes, bytes += (sizeof(float2) * ctx->N * image_cells(ctx->ni[l]) + 255) / 256 * 256;
+    planned += bytes;
+    if (char* c = dry_bytes ? nullptr : (char*)dalloc(ctx, bytes)) {
+      ctx->cells.resize(L);
+      for (int l = 0; l < L; ++l) ctx->cells[l] = (float2*)(c + at[l]);
+    }
+  }
   if (dry_bytes) {
     *dry_bytes = planned;
     delete ctx;
@@ -1157,7 +1169,7 @@ int muster_set_images(muster_ctx* ctx, const float* imgs, int on_device, const d
     Scope s(ctx, KK_DOWN2, (double)N * (nvox(ctx->ni[l + 1]) + nvox(ctx->ni[l])) * 4.0);
     launch_down2(ctx->imgs[l + 1], ctx->ni[l + 1], ctx->imgs[l], ctx->ni[l], N, ctx->stream);
   }
-  for (int l = 0; l < L; ++l) launch_image_cells(ctx->imgs[l], N, ctx->ni[l], ctx->cells[l], ctx->stream);
+  for (int l = 0; l < (int)ctx->cells.size(); ++l) launch_image_cells(ctx->imgs[l], N, ctx->ni[l], ctx->cells[l], ctx->stream);
   // window statistics of every session as a fixed image, per level (images do not change)
   for (int l = 0; l < L; ++l) launch_fixed_stats(ctx->imgs[l], N, 1, ctx->ni[l], ctx->p.window, ctx->p.similarity, ctx->p.sim_eps,
                                             ctx->fstats[l], ctx->stream);
@@ -1500,7 +1512,7 @@ int muster_get_fields(muster_ctx* ctx, int kind, int i, int j, float* out, int o
         if (ctx->rigid) launch_add_rigid(dst, ni, ctx->rig_tab + 12 * i, ctx->stream);  // total deformation
         n = 3 * Vi;
       } else {
-        launch_warp(ctx->d_pairs + pidx(ctx, j, i), 1, ni, nf, dst, nullptr, Vi, ctx->rigid ? ctx->rig_tab : nullptr,
+        launch_warp(ctx->d_pairs + pidx(ctx, j, i), 1, !ctx->cells.empty(), ni, nf, dst, nullptr, Vi, ctx->rigid ? ctx->rig_tab : nullptr,
                     ctx->stream);
         n = Vi;
       }

@@ -46,7 +46,8 @@ struct PairGradTab {
   int slot_pair[kMaxDescPerLaunch];
 };
 struct PairDesc {   // ordered pair (k -> i): pulls image k onto grid i
-  const float2* Ic; // cells of the moving image (launch_image_cells)
+  const float2* Ic; // cells of the moving image (launch_image_cells), null in a context without cells
+  const float* Ik;  // moving image
   const float* Ii;  // fixed image
   const float* Fs;  // window statistics of the fixed image: mu_F then S_FF planes
   const float4* U;  // pair displacement on the flow grid
@@ -136,8 +137,9 @@ void launch_down2(const float* in, Dims n, float* out, Dims m, int n_images, cud
 size_t image_cells(Dims n);
 void launch_image_cells(const float* in, int n_images, Dims n, float2* out, cudaStream_t s);
 // warp_kernels.cu; both require nf = ceil(ni / 2) per axis
-// W: n_pairs volumes at stride Wstride; gI (nullable): grad I_k at the sample points, 3 planes per pair
-void launch_warp(const PairDesc* pd, int n_pairs, Dims ni, Dims nf, float* W, float* gI, size_t Wstride,
+// W: n_pairs volumes at stride Wstride; gI (nullable): grad I_k at the sample points, 3 planes per pair.
+// cells: sample the pairs' cells, else the images themselves (the same values bit for bit)
+void launch_warp(const PairDesc* pd, int n_pairs, bool cells, Dims ni, Dims nf, float* W, float* gI, size_t Wstride,
                  const float* rigid, cudaStream_t s);
 void launch_upsample_disp(const float4* U, Dims nf, Dims ni, float* out_planar, cudaStream_t s);
 // *count += number of NaN/Inf values in x[0, n)

@@ -61,6 +61,36 @@ struct Cells {
     p00 = p, p01 = p + n2, p10 = p + (size_t)n1 * n2, p11 = p10 + n2;
     hz = n.n0 - 0.5f, hy = n.n1 - 0.5f, hx = n.n2 - 0.5f;
   }
+  // the cells of rows (y, y + 1) of planes (z, z + 1) at the positions b of cell_axis
+  __device__ __forceinline__ void load(unsigned bz, unsigned by, unsigned bx, float2 (&v)[2][2]) const {
+    const unsigned o = (bz * n1 + by) * n2 + bx - k;
+    v[0][0] = __ldg(p00 + o), v[0][1] = __ldg(p01 + o), v[1][0] = __ldg(p10 + o), v[1][1] = __ldg(p11 + o);
+  }
+};
+// The same cells made on the way from the image itself, for a context whose device has no room for them
+// (8 bytes per voxel): two loads and a subtraction per cell (an evaluation of 8 x 160^3 takes 6039 us, with
+// cells 5936).
+struct Voxels {
+  const float* p;
+  int n1, n2, mz, my, mx;  // rows per plane, row pitch, last index per axis
+  float hz, hy, hx;
+  __device__ __forceinline__ Voxels(const float* image, Dims n) {
+    p = image, n1 = n.n1, n2 = n.n2, mz = n.n0 - 1, my = n.n1 - 1, mx = n.n2 - 1;
+    hz = n.n0 - 0.5f, hy = n.n1 - 0.5f, hx = n.n2 - 0.5f;
+  }
+  __device__ __forceinline__ void load(unsigned bz, unsigned by, unsigned bx, float2 (&v)[2][2]) const {
+    const int z = (int)(bz - 0x4B000001u), y = (int)(by - 0x4B000001u), x = (int)(bx - 0x4B000001u);  // -1 .. n - 1
+    const int zs[2] = {max(z, 0), min(z + 1, mz)}, ys[2] = {max(y, 0), min(y + 1, my)};
+    const int x0 = max(x, 0), x1 = min(x + 1, mx);
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        const float* row = p + (zs[a] * n1 + ys[b]) * n2;
+        const float l = __ldg(row + x0), r = __ldg(row + x1);
+        v[a][b] = make_float2(l, __fsub_rn(r, l));
+      }
+  }
 };
 // one axis: c = q clamped (a NaN to -1/2), bits of floor(c) + 1 + 2^23 (adding 2^23 + 1 rounded
 // down leaves floor(c) + 1 in the last bits: full-rate adds instead of FRND and F2I), t = c - floor(c)
@@ -70,13 +100,14 @@ __device__ __forceinline__ unsigned cell_axis(float q, float hi, float& t) {
   t = c - (r - 8388609.f);
   return __float_as_uint(r);
 }
-// S[I](q), with GRAD its derivative in g
-template <bool GRAD>
-__device__ __forceinline__ float cell_sample(const Cells& I, float qz, float qy, float qx, float3& g) {
+// S[I](q), with GRAD its derivative in g; I: Cells or Voxels
+template <bool GRAD, class Source>
+__device__ __forceinline__ float cell_sample(const Source& I, float qz, float qy, float qx, float3& g) {
   float tz, ty, tx;
   const unsigned bz = cell_axis(qz, I.hz, tz), by = cell_axis(qy, I.hy, ty), bx = cell_axis(qx, I.hx, tx);
-  const unsigned o = (bz * I.n1 + by) * I.n2 + bx - I.k;
-  const float2 v00 = __ldg(I.p00 + o), v01 = __ldg(I.p01 + o), v10 = __ldg(I.p10 + o), v11 = __ldg(I.p11 + o);
+  float2 v[2][2];
+  I.load(bz, by, bx, v);
+  const float2 v00 = v[0][0], v01 = v[0][1], v10 = v[1][0], v11 = v[1][1];
   const float c00 = fmaf(tx, v00.y, v00.x), c01 = fmaf(tx, v01.y, v01.x);
   const float c10 = fmaf(tx, v10.y, v10.x), c11 = fmaf(tx, v11.y, v11.x);
   const float y0 = c01 - c00, y1 = c11 - c10;
@@ -115,7 +146,7 @@ __global__ void k_image_cells(const float* __restrict__ in, Dims n, float2* __re
 // 331 us; a 2 x 2 x 2 block per thread with eight 4-byte gathers per voxel took 2714 us / 141 us /
 // 24.1 ms / 366 us. Streaming stores keep the images in L2 (5 % of the first two). Staging U in
 // shared memory, 48 registers for 5 CTAs and 8 warps' rows per CTA instead of 4 or 16 were within 3 %.
-template <bool GRAD, bool RIGID>
+template <bool GRAD, bool RIGID, bool CELLS>
 __global__ void __launch_bounds__(BX* BY, kWarpCtas) k_warp(const PairDesc* __restrict__ pd, int n_pairs, Dims ni, Dims nf, int nz,
                                                  float* __restrict__ W, float* __restrict__ gI, size_t stride,
                                                  const float* __restrict__ rig) {
@@ -131,7 +162,12 @@ __global__ void __launch_bounds__(BX* BY, kWarpCtas) k_warp(const PairDesc* __re
   const int my = (int)(id % gy) * BY + threadIdx.y, m0 = (int)(id / gy) * nz;
   if (x >= ni.n2 || my >= nf.n1) return;
   const PairDesc d = pd[pair];
-  const Cells I(d.Ic, ni);
+  const auto I = [&] {
+    if constexpr (CELLS)
+      return Cells(d.Ic, ni);
+    else
+      return Voxels(d.Ik, ni);
+  }();
   const int fp = nf.n1 * nf.n2, plane = ni.n1 * ni.n2;
   // along W voxel x takes 3 parts of node x / 2 and one of the node on its side; the product is
   // rounded before the sum for even voxels (lower) and in it for odd ones (upper): fma(ca, cb P, Q)
@@ -586,22 +622,24 @@ static int warp_planes(long tiles, int depth) {
   while (nz > least && tiles * ((depth + nz - 1) / nz) < 16L * device_sm_count()) nz /= 2;
   return nz;
 }
-void launch_warp(const PairDesc* pd, int n_pairs, Dims ni, Dims nf, float* W, float* gI, size_t Wstride,
+void launch_warp(const PairDesc* pd, int n_pairs, bool cells, Dims ni, Dims nf, float* W, float* gI, size_t Wstride,
                  const float* rigid, cudaStream_t s) {
   const int gx = (ni.n2 + BX - 1) / BX, gy = (nf.n1 + BY - 1) / BY;
   const int nz = warp_planes((long)gx * gy * n_pairs, nf.n0);
   const unsigned grid = (unsigned)gx * gy * ((nf.n0 + nz - 1) / nz) * n_pairs;
-  const dim3 b(BX, BY);
-  if (gI) {
-    if (rigid)
-      launch(k_warp<true, true>, grid, b, 0, s, false)(pd, n_pairs, ni, nf, nz, W, gI, Wstride, rigid);
+  auto go = [&](auto kernel) {
+    launch(kernel, grid, dim3(BX, BY), 0, s, false)(pd, n_pairs, ni, nf, nz, W, gI, Wstride, rigid);
+  };
+  if (cells) {
+    if (gI)
+      rigid ? go(k_warp<true, true, true>) : go(k_warp<true, false, true>);
     else
-      launch(k_warp<true, false>, grid, b, 0, s, false)(pd, n_pairs, ni, nf, nz, W, gI, Wstride, nullptr);
+      rigid ? go(k_warp<false, true, true>) : go(k_warp<false, false, true>);
   } else {
-    if (rigid)
-      launch(k_warp<false, true>, grid, b, 0, s, false)(pd, n_pairs, ni, nf, nz, W, nullptr, Wstride, rigid);
+    if (gI)
+      rigid ? go(k_warp<true, true, false>) : go(k_warp<true, false, false>);
     else
-      launch(k_warp<false, false>, grid, b, 0, s, false)(pd, n_pairs, ni, nf, nz, W, nullptr, Wstride, nullptr);
+      rigid ? go(k_warp<false, true, false>) : go(k_warp<false, false, false>);
   }
 }
 

@@ -92,6 +92,10 @@ class EngineBackend:
 
         return footprint(job.images.shape[1:], job.images.shape[0], **self._params(job))
 
+    def lean(self, job: Job) -> Job:
+        """The job in less device memory: its warps sample the images themselves, with the same results."""
+        return dataclasses.replace(job, params=dict(job.params, plain_images=1))
+
     def create(self, job: Job):
         from .api import Muster
 
@@ -225,6 +229,9 @@ class MusterServer:
 
     def submit(self, job: Job) -> None:
         need = int(self.backend.footprint(job))
+        if need > self.budget and hasattr(self.backend, "lean"):
+            job = self.backend.lean(job)
+            need = int(self.backend.footprint(job))
         if need > self.budget:
             raise ValueError("job %d needs %d bytes, more than the whole budget" % (job.id, need))
         self.queue.append((job, need))

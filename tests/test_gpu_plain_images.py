@@ -1,0 +1,68 @@
+"""Contexts without the cells of their images (plain_images, or a device that refuses the cells' block): the forward
+warp samples the images themselves, with the same results bit for bit, and everything that needs the warp runs."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2412_14671_gb300 as m
+from paper_2412_14671_gb300 import _native, phantom
+
+pytestmark = pytest.mark.gpu
+
+
+def _results(shape, N, allocator=None, **kw):
+    """gradient and loss of an evaluation with displacements that leave the volume, a registration's
+    velocities and a warped image"""
+    imgs = torch.from_numpy(phantom.blob_series(shape, N, seed=17)["images"]).cuda()
+    nf = [(a + 1) // 2 for a in shape]
+    v = 2.0 * torch.randn([N - 1, 3] + nf, generator=torch.Generator(device="cuda").manual_seed(3), device="cuda")
+    with m.Muster(shape, N, allocator=allocator, n_levels=1, steps_per_level=[4], n_squarings=4, window=3, deterministic=1,
+                  **kw) as reg:
+        reg.set_images(imgs)
+        g = torch.zeros_like(v)
+        loss = reg.eval(v, 0, g)
+        reg.run()
+        return [torch.tensor(loss), g, reg.velocities(0), reg.get_field(m.WARPED, 0, N - 1, level=0)]
+
+
+@pytest.mark.parametrize("rigid", [0, 1])
+@pytest.mark.parametrize("shape,N", [((16, 20, 24), 3), ((13, 9, 35), 4), ((1, 12, 33), 3), ((5, 1, 64), 2)])
+def test_same_bits_without_cells(shape, N, rigid):
+    for a, b in zip(_results(shape, N, rigid=rigid), _results(shape, N, rigid=rigid, plain_images=1)):
+        assert torch.equal(a, b)
+
+
+def test_a_refused_block_of_cells_leaves_a_working_context():
+    shape, N = (13, 9, 35), 4
+    cells = 8 * N * (shape[0] + 2) * (shape[1] + 2) * (shape[2] + 1)
+    stream, live, refused = torch.cuda.default_stream(), set(), []
+
+    def alloc(nbytes, user):
+        if abs(int(nbytes) - cells) < 256:
+            refused.append(int(nbytes))
+            return None
+        p = torch.cuda.caching_allocator_alloc(int(nbytes), torch.cuda.current_device(), stream)
+        live.add(p)
+        return p
+
+    def release(ptr, user):
+        live.discard(ptr)
+        torch.cuda.caching_allocator_delete(ptr)
+
+    fns = (_native.ALLOC_FN(alloc), _native.FREE_FN(release))
+    for a, b in zip(_results(shape, N), _results(shape, N, allocator=fns)):
+        assert torch.equal(a, b)
+    assert len(refused) == 2 and not live  # refused, and refused again after the pool was given back
+
+
+def test_memory_without_cells():
+    shape, N = (96, 112, 96), 6
+    kw = dict(n_levels=1, steps_per_level=[1], window=7)
+    cells = 8 * N * (shape[0] + 2) * (shape[1] + 2) * (shape[2] + 1)
+    assert 0 <= m.footprint(shape, N, **kw) - m.footprint(shape, N, plain_images=1, **kw) - cells < 256
+    need = m.footprint(shape, N, plain_images=1, **kw)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    with m.Muster(shape, N, plain_images=1, **kw):
+        took = free - torch.cuda.mem_get_info()[0]
+    assert need <= took <= need * 1.02 + 64 * 2**20, (need, took)
