@@ -1158,7 +1158,10 @@ int muster_set_images(muster_ctx* ctx, const float* imgs, int on_device, const d
   CK(cudaMemcpyAsync(top, imgs, sizeof(float) * N * Vi, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
                      ctx->stream));
   CK(cudaMemsetAsync(ctx->count_dev, 0, sizeof(int), ctx->stream));
-  launch_count_nonfinite(top, (size_t)N * Vi, ctx->count_dev, ctx->stream);
+  if (ctx->cells.empty())
+    launch_count_nonfinite(top, (size_t)N * Vi, ctx->count_dev, ctx->stream);
+  else  // the cells of the finest level look at every voxel on their way
+    launch_image_cells(top, N, ctx->ni[L - 1], ctx->cells[L - 1], ctx->count_dev, ctx->stream);
   CK(cudaMemcpyAsync(&ctx->hbox->bad, ctx->count_dev, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   ctx->have_images = false;
   ctx->level = -1;
@@ -1169,7 +1172,8 @@ int muster_set_images(muster_ctx* ctx, const float* imgs, int on_device, const d
     Scope s(ctx, KK_DOWN2, (double)N * (nvox(ctx->ni[l + 1]) + nvox(ctx->ni[l])) * 4.0);
     launch_down2(ctx->imgs[l + 1], ctx->ni[l + 1], ctx->imgs[l], ctx->ni[l], N, ctx->stream);
   }
-  for (int l = 0; l < (int)ctx->cells.size(); ++l) launch_image_cells(ctx->imgs[l], N, ctx->ni[l], ctx->cells[l], ctx->stream);
+  for (int l = 0; l + 1 < (int)ctx->cells.size(); ++l)
+    launch_image_cells(ctx->imgs[l], N, ctx->ni[l], ctx->cells[l], nullptr, ctx->stream);
   // window statistics of every session as a fixed image, per level (images do not change)
   for (int l = 0; l < L; ++l) launch_fixed_stats(ctx->imgs[l], N, 1, ctx->ni[l], ctx->p.window, ctx->p.similarity, ctx->p.sim_eps,
                                             ctx->fstats[l], ctx->stream);

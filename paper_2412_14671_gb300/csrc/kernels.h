@@ -135,7 +135,8 @@ void launch_planar_to_f4(const float* in, float4* out, int n_fields, size_t V, c
 void launch_down2(const float* in, Dims n, float* out, Dims m, int n_images, cudaStream_t s);
 // images as cells along W with a replicated border, as the forward warp samples them (warp_kernels.cu)
 size_t image_cells(Dims n);
-void launch_image_cells(const float* in, int n_images, Dims n, float2* out, cudaStream_t s);
+// bad (nullable): set to non-zero if a voxel is not finite
+void launch_image_cells(const float* in, int n_images, Dims n, float2* out, int* bad, cudaStream_t s);
 // warp_kernels.cu; both require nf = ceil(ni / 2) per axis
 // W: n_pairs volumes at stride Wstride; gI (nullable): grad I_k at the sample points, 3 planes per pair.
 // cells: sample the pairs' cells, else the images themselves (the same values bit for bit)

@@ -63,25 +63,35 @@
 namespace muster {
 
 namespace {
-constexpr int kStatThreads = 128, TX = 32;  // k_fixed_stats
+constexpr int TX = 32;  // k_fixed_stats
 
 // Statistics of the fixed image of every window, once per session and level:
 // out[0][c] = mu_F and out[1][c] = S_FF (centred sum of squares) at corner c, or for SiLNCC
 // (KIND 0, which needs S_FF only in beta = S_FW / (S_FF + eps)) out[1][c] = 1 / (S_FF + eps).
 // A CTA walks the planes of a 32 x 8 tile: a W task forms 4 neighbouring sums from one read of their
-// inputs, a thread of the H and D sums has 2 rows of a column, and a plane's loads are under way while
-// the plane before is summed. Shared memory bounds it. One 160 x 192 x 160 image, w = 7: 36 us; one sum
-// per thread and pass (twice the shared-memory traffic) and loads between two barriers took 44 us.
-// Every sum adds its terms one after the other.
+// inputs, a thread of the H and D sums has 1 or 2 rows of a column, and a plane's loads are under way while
+// the plane before is summed. Every sum adds its terms one after the other, whatever the threads.
+// Shared memory and, in small launches, latency bound it; which number of threads and register budget serves
+// both best was measured for each instantiation, over 1 to 10 images of 48^3 to 256^3 (StatCut). w = 7, us, on
+// 10, 4 and 2 images of 160 x 192 x 160 and one in the chunks of a stateless call: SiLNCC 275, 131, 69, 32 (128
+// threads uncapped 352, 171, 87, 35), LNCC 322, 152, 77, 59 (564, 280, 148, 115); one sum per thread and pass with
+// its loads between two barriers took 401, 194, 95, 84 and 378, 181, 88, 78.
 template <int R, int KIND>
-__global__ void __launch_bounds__(kStatThreads) k_fixed_stats(const float* __restrict__ imgs, float* __restrict__ stats,
-                                                              Dims n, int tz, int nzc, float eps,
-                                                              OpHead* __restrict__ head, PairDesc pd) {
+struct StatCut {
+  static constexpr int kCut[2][5][2] = {{{128, 8}, {128, 8}, {256, 4}, {128, 0}, {256, 4}},
+                                        {{256, 0}, {256, 6}, {256, 0}, {256, 4}, {256, 4}}};
+  static constexpr int threads = kCut[KIND][R - 1][0], ctas = kCut[KIND][R - 1][1];  // CTAs per SM at least (0: no cap)
+};
+template <int R, int KIND>
+__global__ void __launch_bounds__(StatCut<R, KIND>::threads, StatCut<R, KIND>::ctas)
+    k_fixed_stats(const float* __restrict__ imgs, float* __restrict__ stats, Dims n, int tz, int nzc, float eps,
+                  OpHead* __restrict__ head, PairDesc pd) {
   grid_wait();
+  constexpr int NT = StatCut<R, KIND>::threads;
   if (head && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) *head = OpHead{{}, {}, pd};
   constexpr int WW = 2 * R + 1, TY = 8, RX = TX + 2 * R, RY = TY + 2 * R, PF = (RX + 3) / 4 * 4;
-  constexpr int NE = RY * RX, NSLOT = (NE + kStatThreads - 1) / kStatThreads;
-  constexpr int NO = 4, NI = NO + 2 * R, NV = (NI + 3) / 4, NR = TY * TX / kStatThreads;
+  constexpr int NE = RY * RX, NSLOT = (NE + NT - 1) / NT;
+  constexpr int NO = 4, NI = NO + 2 * R, NV = (NI + 3) / 4, NR = TY * TX / NT;
   __shared__ float4 sF[RY][PF / 4];
   __shared__ float4 sx[2][RY][TX / 4];
   const int img = blockIdx.z / nzc, zc = blockIdx.z - img * nzc;
@@ -94,7 +104,7 @@ __global__ void __launch_bounds__(kStatThreads) k_fixed_stats(const float* __res
   int goff[NSLOT], soff[NSLOT];  // global (-1: outside) and shared position of a thread's inputs
 #pragma unroll
   for (int k = 0; k < NSLOT; ++k) {
-    const int e = tid + kStatThreads * k;
+    const int e = tid + NT * k;
     const int ry = e / RX, rx = e - ry * RX;
     const int gy = y0 + ry, gx = x0 + rx;
     goff[k] = e < NE && gy < n.n1 && gx < n.n2 ? gy * n.n2 + gx : -1;
@@ -121,7 +131,7 @@ __global__ void __launch_bounds__(kStatThreads) k_fixed_stats(const float* __res
         if (soff[k] >= 0) reinterpret_cast<float*>(sF)[soff[k]] = next[k];
       __syncthreads();
       load(z0 + it + 1);
-      for (int t = tid; t < RY * (TX / NO); t += kStatThreads) {
+      for (int t = tid; t < RY * (TX / NO); t += NT) {
         const int ry = t / (TX / NO), run = t % (TX / NO);
         float v[4 * NV], a0[NO] = {}, a1[NO] = {};
 #pragma unroll
@@ -966,17 +976,10 @@ Tiles sim_tiles(Dims ni, int window, int kind, int n_pairs, int batch, int group
   return g;
 }
 unsigned ctas(const Tiles& g) { return (unsigned)g.gx * g.gy * g.nzc * g.np; }
-template <int KIND>
-void fixed_stats(dim3 g, const float* imgs, Dims ni, int window, float eps, float* stats, int tz, int nzc,
-                 OpHead* head, const PairDesc& pd, cudaStream_t s) {
-  switch (window / 2) {
-    case 1: launch(k_fixed_stats<1, KIND>, g, kStatThreads, 0, s)(imgs, stats, ni, tz, nzc, eps, head, pd); break;
-    case 2: launch(k_fixed_stats<2, KIND>, g, kStatThreads, 0, s)(imgs, stats, ni, tz, nzc, eps, head, pd); break;
-    case 3: launch(k_fixed_stats<3, KIND>, g, kStatThreads, 0, s)(imgs, stats, ni, tz, nzc, eps, head, pd); break;
-    case 4: launch(k_fixed_stats<4, KIND>, g, kStatThreads, 0, s)(imgs, stats, ni, tz, nzc, eps, head, pd); break;
-    case 5: launch(k_fixed_stats<5, KIND>, g, kStatThreads, 0, s)(imgs, stats, ni, tz, nzc, eps, head, pd); break;
-    default: break;
-  }
+template <int R, int KIND>
+void fixed_stats(dim3 g, const float* imgs, Dims ni, float eps, float* stats, int tz, int nzc, OpHead* head,
+                 const PairDesc& pd, cudaStream_t s) {
+  launch(k_fixed_stats<R, KIND>, g, StatCut<R, KIND>::threads, 0, s)(imgs, stats, ni, tz, nzc, eps, head, pd);
 }
 }  // namespace
 
@@ -985,10 +988,9 @@ void launch_fixed_stats(const float* imgs, int n_images, int batch, Dims ni, int
   const int gx = (ni.n2 + TX - 1) / TX, gy = (ni.n1 + 7) / 8;
   const int tz = chunk_planes(gx * gy, ni, window, kind, 16, 128, batch), nzc = (ni.n0 + tz - 1) / tz;
   const dim3 g(gx, gy, nzc * n_images);
-  if (kind == 0)
-    fixed_stats<0>(g, imgs, ni, window, eps, stats, tz, nzc, head, pd, s);
-  else
-    fixed_stats<1>(g, imgs, ni, window, eps, stats, tz, nzc, head, pd, s);
+  dispatch(window / 2, kind, false, [&](auto r, auto k, auto) {
+    fixed_stats<r(), k()>(g, imgs, ni, eps, stats, tz, nzc, head, pd, s);
+  });
 }
 
 cudaError_t prepare_kernels() {

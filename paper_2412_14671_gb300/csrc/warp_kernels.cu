@@ -120,18 +120,35 @@ __device__ __forceinline__ float cell_sample(const Source& I, float qz, float qy
   return fmaf(tz, z0, c0);
 }
 
-// the cells of image volumes (grid y over images)
-__global__ void k_image_cells(const float* __restrict__ in, Dims n, float2* __restrict__ out) {
+// The cells of image volumes (grid y over images), a warp per row, 4 cells under way per thread; bad (nullable) is
+// set if a voxel is not finite. DRAM bounds it (12 bytes per voxel). 10 x 160 x 192 x 160 in four levels: 130 us
+// with the check; a thread per cell that found its place by three integer divisions took 269 us, and
+// the check as a pass of its own 84 us more.
+constexpr int kCellRows = 8, kCellRun = 4;
+__global__ void __launch_bounds__(32 * kCellRows) k_image_cells(const float* __restrict__ in, Dims n, float2* __restrict__ out,
+                                                                int* __restrict__ bad) {
   grid_begin();
-  const Dims m{n.n0 + 2, n.n1 + 2, n.n2 + 1};
-  const unsigned v = blockIdx.x * blockDim.x + threadIdx.x;
-  const size_t Vm = vox(m);
-  if (v >= Vm) return;
-  const int x = (int)(v % (unsigned)m.n2) - 1, r = (int)(v / (unsigned)m.n2), y = r % m.n1, z = r / m.n1;
+  const int rows = (n.n0 + 2) * (n.n1 + 2), r = blockIdx.x * kCellRows + threadIdx.y;
+  if (r >= rows) return;
+  const int z = r / (n.n1 + 2), y = r - z * (n.n1 + 2);
   const int yi = min(max(y - 1, 0), n.n1 - 1), zi = min(max(z - 1, 0), n.n0 - 1);
   const float* row = in + blockIdx.y * vox(n) + ((size_t)zi * n.n1 + yi) * n.n2;
-  const float a = row[max(x, 0)], b = row[min(x + 1, n.n2 - 1)];
-  out[blockIdx.y * Vm + v] = make_float2(a, b - a);
+  float2* o = out + ((size_t)blockIdx.y * rows + r) * (n.n2 + 1);
+  bool fine = true;
+  for (int x0 = (int)threadIdx.x; x0 <= n.n2; x0 += 32 * kCellRun) {  // cell x0 is that of voxel x0 - 1
+    float a[kCellRun], b[kCellRun];
+#pragma unroll
+    for (int k = 0; k < kCellRun; ++k) {
+      const int x = min(x0 + 32 * k, n.n2) - 1;
+      a[k] = __ldg(row + max(x, 0)), b[k] = __ldg(row + min(x + 1, n.n2 - 1));
+    }
+#pragma unroll
+    for (int k = 0; k < kCellRun; ++k) {
+      fine = fine && isfinite(a[k]);
+      if (x0 + 32 * k <= n.n2) o[x0 + 32 * k] = make_float2(a[k], __fsub_rn(b[k], a[k]));
+    }
+  }
+  if (bad && !fine) atomicOr(bad, 1);
 }
 
 // ---- W(p) = S[I_k](p + U~(p)) for every image voxel of the pair batch; with GRAD the
@@ -644,8 +661,9 @@ void launch_warp(const PairDesc* pd, int n_pairs, bool cells, Dims ni, Dims nf, 
 }
 
 size_t image_cells(Dims n) { return vox(Dims{n.n0 + 2, n.n1 + 2, n.n2 + 1}); }
-void launch_image_cells(const float* in, int n_images, Dims n, float2* out, cudaStream_t s) {
-  launch(k_image_cells, dim3((unsigned)((image_cells(n) + 255) / 256), n_images), 256, 0, s)(in, n, out);
+void launch_image_cells(const float* in, int n_images, Dims n, float2* out, int* bad, cudaStream_t s) {
+  const unsigned rows = (unsigned)(n.n0 + 2) * (n.n1 + 2);
+  launch(k_image_cells, dim3((rows + kCellRows - 1) / kCellRows, n_images), dim3(32, kCellRows), 0, s)(in, n, out, bad);
 }
 
 int warp_bwd_ctas_per_pair(Dims nf, int batch) {

@@ -66,3 +66,22 @@ def test_memory_without_cells():
     with m.Muster(shape, N, plain_images=1, **kw):
         took = free - torch.cuda.mem_get_info()[0]
     assert need <= took <= need * 1.02 + 64 * 2**20, (need, took)
+
+
+@pytest.mark.parametrize("plain", [0, 1])
+@pytest.mark.parametrize("at", [(0, 0, 0, 0), (2, 12, 8, 34), (1, 0, 8, 33), (0, 12, 0, 1), (2, 6, 4, 17)])
+@pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
+def test_non_finite_images_are_refused(plain, at, value):
+    """the first and last voxel of the series, edges and the middle; the context takes good images afterwards"""
+    shape, N = (13, 9, 35), 3
+    imgs = phantom.blob_series(shape, N, seed=18)["images"]
+    bad = imgs.copy()
+    bad[at] = value
+    with m.Muster(shape, N, n_levels=2, steps_per_level=[1, 1], window=3, plain_images=plain) as reg:
+        with pytest.raises(m.MusterError) as e:
+            reg.set_images(torch.from_numpy(bad).cuda())
+        assert e.value.code == _native.EINVAL
+        with pytest.raises(m.MusterError):
+            reg.run()
+        reg.set_images(torch.from_numpy(imgs).cuda())
+        assert np.isfinite(reg.run())
