@@ -16,11 +16,13 @@
 // What bounds them: the shared-memory pipe (bytes moved through L1 per output), then instruction
 // issue. The layout is chosen for both: 8 sums per W task read 14 inputs (w = 7) instead of 10 for
 // every 4, four rows per H/D thread read 10 W sums instead of 16, the ring moves 16 bytes per
-// access, and the row pitches (4 modulo 8 floats) keep the W task's accesses free of bank conflicts.
+// access, and the pitch of the staged rows (4 modulo 8 floats) and the order of the W sums in theirs (sx_col) keep
+// the W task's accesses free of bank conflicts.
 // Measured on 90 pairs of 160 x 192 x 160, w = 7, SiLNCC: forward 1729 us, adjoint 1451 us (L1 data
 // pipe 76 and 81 % busy, DRAM 39 and 57 %); one role per thread with a barrier per plane, W sums in
-// runs of 4 and two rows per thread took 2605 and 1802 us. 4 CTAs of 7 warps run on an SM; cut for
-// 3, the forward takes 12 % longer.
+// runs of 4 and two rows per thread took 2605 and 1802 us. 4 CTAs of 7 warps run on an SM; larger windows and
+// LNCC's third moment leave room for 3 or 2 (Box::min_ctas). 56 pairs of 160^3, forward / adjoint: SiLNCC w = 7 965 /
+// 775 us, w = 11 1202 / 1007 us; LNCC w = 7 1492 / 1283 us, w = 11 1981 / 1378 us.
 //
 // The order of the additions is part of the results, and the layout keeps it: along W runs of 4
 // sums (a pairwise tree, then a running sum), along H runs of 2, along D the ring. An optimiser
@@ -943,7 +945,8 @@ int chunk_for(int ntiles, int depth, int min_chunk, int threads, int batch) {
 // more chunks fill more SMs. The cost of a chunking is its planes per CTA times the time of a plane at
 // its CTAs per SM: c <= 4 resident CTAs take about 0.55 + 0.21 c us per plane (one 160 x 192 x 160
 // pair, w = 7, forward: 0.97 us at 2, 1.39 us at 4), and more than 4 follow one another. That pair runs
-// in 10 chunks (forward and adjoint 57 us), where the rule above takes 2 (148 us).
+// in 10 chunks (forward and adjoint 57 us), where the rule above takes 2 (148 us). The figures of w = 7
+// serve every window and the statistics too: chunks are part of the results.
 int filling_chunks(long tiles, int depth, int reach) {
   const long sms = device_sm_count();
   auto wave = [](long c) { return c ? 26 + 10 * c : 0; };
