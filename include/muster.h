@@ -128,7 +128,7 @@ typedef struct {
   int plain_images;       /* the forward warp samples cells (I(x), I(x + 1) - I(x)) of the images, 8 bytes
                              per voxel, session and level beside the images' 4 and their statistics' 8
                              (with a border of one cell). 0: when the device has room for them after
-                             everything else, 1: never. The results do not depend on it */
+                             everything else (and 512 MiB beside large ones), 1: never. The results do not depend on it */
   /* optional device allocator (e.g. a framework's caching allocator); both or neither. A block
      that alloc refuses (NULL) is asked for once more before the call gives up */
   void* (*alloc)(size_t bytes, void* user);

@@ -1035,7 +1035,12 @@ int create_impl(const int64_t shape[3], int n_sessions, const double spacing[3],
     size_t bytes = 0;
     for (int l = 0; l < L; ++l) at[l] = bytes, bytes += (sizeof(float2) * ctx->N * image_cells(ctx->ni[l]) + 255) / 256 * 256;
     planned += bytes;
-    if (char* c = dry_bytes ? nullptr : (char*)dalloc(ctx, bytes)) {
+    // large cells leave what graphs, kernels and the caller take later; what a callback's allocator holds in
+    // reserve is not seen here
+    size_t left = 0, total = 0;
+    const bool room = params->alloc || bytes < ((size_t)64 << 20) || cudaMemGetInfo(&left, &total) != cudaSuccess ||
+                      left >= bytes + ((size_t)512 << 20);
+    if (char* c = dry_bytes || !room ? nullptr : (char*)dalloc(ctx, bytes)) {
       ctx->cells.resize(L);
       for (int l = 0; l < L; ++l) ctx->cells[l] = (float2*)(c + at[l]);
     }

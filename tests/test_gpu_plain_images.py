@@ -85,3 +85,29 @@ def test_non_finite_images_are_refused(plain, at, value):
             reg.run()
         reg.set_images(torch.from_numpy(imgs).cuda())
         assert np.isfinite(reg.run())
+
+
+def test_large_cells_leave_room_on_a_nearly_full_device():
+    """with room for the cells but little more, a context leaves them out, with the same results"""
+    shape, N = (128, 128, 128), 6
+    kw = dict(n_levels=1, steps_per_level=[1], n_squarings=4, window=3, deterministic=1, pair_batch=4)
+    lean, full = m.footprint(shape, N, plain_images=1, **kw), m.footprint(shape, N, **kw)
+    assert full - lean > 64 * 2**20
+    imgs = torch.rand((N,) + shape, generator=torch.Generator(device="cuda").manual_seed(4), device="cuda")
+    v = torch.randn([N - 1, 3, 64, 64, 64], generator=torch.Generator(device="cuda").manual_seed(5), device="cuda")
+    grads = []
+    for fill in (False, True):
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        free = torch.cuda.mem_get_info()[0]
+        filler = torch.empty(free - full - (384 << 20), dtype=torch.uint8, device="cuda") if fill else None  # never touched
+        free = torch.cuda.mem_get_info()[0]
+        with m.Muster(shape, N, **kw) as reg:
+            took = free - torch.cuda.mem_get_info()[0]
+            assert (took < lean + (full - lean) // 2) == fill, (took, lean, full)
+            reg.set_images(imgs)
+            grads.append(torch.zeros_like(v))
+            reg.eval(v, 0, grads[-1])
+        del filler
+        torch.cuda.empty_cache()
+    assert torch.equal(*grads)
